@@ -152,9 +152,13 @@ int cos_copy_times(cos_graph_t g, double* dst, void* stream);
 
 /*
  * Evaluate the path sum of every attached sample (Fig. 1; Sec. II.C): one
- * persistent kernel computes, tile of samples by tile, the propagator table,
- * walks the levels in order, writes the sink value per sample, and finally
- * reduces the samples -- either level-synchronous (cooperative launch, a
+ * persistent kernel forms the propagators, walks the levels in order, writes the
+ * sink value per sample, and finally reduces the samples.  Graphs whose widest
+ * level and propagator slots fit shared memory run on chip where that is expected
+ * to be faster and the tuning names no launch shape (see cos_tuning): a thread
+ * block carries a chunk of samples through every level, waits for no other block
+ * and allocates nothing.  Otherwise tile of samples by tile in the workspace --
+ * either level-synchronous (cooperative launch, a
  * grid-wide barrier between levels) or from a work queue (see cos_tuning.schedule).
  * The level-synchronous schedule allocates nothing when per_sample_out is given
  * (without it, the first evaluation of a larger sample set allocates an internal
@@ -175,6 +179,8 @@ int cos_copy_times(cos_graph_t g, double* dst, void* stream);
  * Errors: COS_ERR_STATE (no samples attached), COS_ERR_INVALID (mode),
  *         COS_ERR_CUDA, COS_ERR_TIMEOUT, COS_ERR_OVERFLOW (count mode, exact
  *         count > 2^63-1; the wrapped results are still written).
+ * Results do not depend on which of these kernels runs (bitwise; times far outside
+ * [-beta, beta] aside, whose propagators may differ by 1e-10 in FP32 mixed mode).
  */
 int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean_out, void* stream);
 
@@ -245,15 +251,20 @@ int cos_mc_values(cos_mc_t m, double* per_walker_out, void* stream);
 int cos_mc_destroy(cos_mc_t m);
 
 /*
- * Graph facts, written to info[0..n) in this order (n <= 10):
+ * Graph facts, written to info[0..n) in this order (n <= 11):
  *   0 L, 1 N, 2 E, 3 number of propagator slots P, 4 widest level W_max,
  *   5 path count mod 2^64 (from ingest), 6 path-count overflow flag,
- *   7 K, 8 D, 9 device ordinal
+ *   7 K, 8 D, 9 device ordinal, 10 modes that run on chip with the current tuning
+ *   and sample count: bits 0..2 the modes, bit 4 FP32 mixed with COS_EVAL_ABS
  */
 int cos_graph_info(cos_graph_t g, int64_t* info, int32_t n);
 
 /*
- * Launch shape used by cos_evaluate.  Fields <= 0 mean "automatic".
+ * Launch shape used by cos_evaluate.  Fields <= 0 mean "automatic".  The fields
+ * describe the kernels that work in the workspace; when all but tile_samples and
+ * timeout_ms are automatic, an evaluation may run on chip instead (cos_evaluate), and
+ * cos_get_tuning reports the shape it would have otherwise.  A phase trace
+ * (cos_set_trace) also keeps an evaluation off the chip.
  *   samples_per_lane  1, 2 or 4 consecutive samples per thread (vector width)
  *   tile_samples      samples per tile (rounded up to 32 * samples_per_lane)
  *   rows_per_warp     consecutive destination rows one warp takes per work item (<= 31);
@@ -321,7 +332,8 @@ int cos_get_tuning(cos_graph_t g, int32_t mode, cos_tuning* tuning);
  * Time launch shapes for `mode` on g's attached samples (both schedules, 8/16/31
  * rows per warp, two vector widths; fields already set > 0 stay fixed), keep the
  * fastest as g's tuning and, if best is non-NULL, store its resolved form there.
- * Runs 36 evaluations at most on `stream` (writing per_sample_out, which may be
+ * An evaluation that the automatic shape runs on chip is timed too, and the shape stays
+ * automatic when that is the fastest.  Runs 39 evaluations at most on `stream` (writing per_sample_out, which may be
  * NULL) and synchronizes; results are bitwise the same for every candidate.
  * The paper has no counterpart; cos_batch_autotune does the same for batches.
  */
@@ -336,7 +348,9 @@ int cos_autotune(cos_graph_t g, int32_t mode, void* per_sample_out, void* stream
  * samples, each level per tile, the sample reduction); the per-graph phase chains
  * are interleaved into one task list that a persistent grid drains through a
  * ticket counter, each item waiting only for the previous phase of its own graph
- * (of its own window of sample chunks when window_chunks > 0).
+ * (of its own window of sample chunks when window_chunks > 0).  Members that run on
+ * chip (cos_evaluate) follow in launches of their own, chunk by chunk from a ticket
+ * counter, when neither the batch nor the member names a launch shape.
  * The launch (counter reset + kernel) is captured into a CUDA graph on first use
  * and replayed by every later cos_batch_launch.
  *
@@ -356,8 +370,8 @@ int cos_autotune(cos_graph_t g, int32_t mode, void* per_sample_out, void* stream
  *                     tile_samples, blocks_per_sm, timeout_ms, window_chunks,
  *                     prefetch; other fields come from each graph.
  *   cos_batch_autotune  times every (samples_per_lane, rows_per_warp, layout)
- *                     candidate on the batch itself, keeps the fastest and returns
- *                     it in *best.
+ *                     candidate on the batch itself (and the automatic shape, where it
+ *                     runs members on chip), keeps the fastest and returns it in *best.
  *   cos_batch_launch  enqueue one evaluation of all graphs on `stream`.  The first
  *                     launch of a plan uploads it (stream-ordered) and runs the
  *                     kernel directly; the second captures counter reset + kernel

@@ -26,16 +26,21 @@
 #include <cstring>
 #include <vector>
 
+#include "cos_chip.cuh"
 #include "cos_items.cuh"
 #include "cos_tasks.cuh"
 
 namespace cosgpu {
 namespace {
 
+constexpr int kChipLaunches = 9;   // on-chip launches of a batch: 3 lane widths x 3 CTA sizes
+
 struct BatchCtrl {
     unsigned long long ticket;
     int err;
     int err_task;
+    unsigned chip_ticket[kChipLaunches];
+    unsigned chip_exits[kChipLaunches];
 };
 
 struct BatchArgs {
@@ -212,15 +217,25 @@ struct cos_batch {
     std::vector<int> counts_overflow;
     std::vector<int32_t> joins;
     std::vector<uint64_t> member_gen;   // each member's generation when the plan was made
+    // members evaluated on chip, grouped by launch (lane width, CTA size)
+    struct ChipLaunch {
+        int lane_bytes, threads, smem, first, n, chunks;
+    };
+    std::vector<ChipParams> chip;
+    std::vector<ChipLaunch> chip_launches;
+    int sms = 0;
+    bool general_only = false;          // one graph under the windowed schedule: never on chip
     Task* h_tasks = nullptr;
     int32_t* h_joins = nullptr;
     WalkParams* h_params = nullptr;
+    ChipParams* h_chip = nullptr;
     double* h_means = nullptr;
     BatchCtrl* h_ctrl = nullptr;
     // device buffers (grow only)
     Task* d_tasks = nullptr;
     int32_t* d_joins = nullptr;
     WalkParams* d_params = nullptr;
+    ChipParams* d_chip = nullptr;
     unsigned* d_done = nullptr;
     double* d_means = nullptr;
     BatchCtrl* d_ctrl = nullptr;
@@ -237,7 +252,7 @@ struct cos_batch {
     // identical plan (the usual repeated evaluation) is not copied again.
     cudaEvent_t staged = nullptr;
     bool staged_valid = false;
-    size_t staged_tasks = 0, staged_joins = 0, staged_params = 0;
+    size_t staged_tasks = 0, staged_joins = 0, staged_params = 0, staged_chip = 0;
     int launches_since_plan = 0;
     // captured launch (counter reset + kernel), built on the second launch of a plan
     cudaGraph_t cgraph = nullptr;
@@ -270,23 +285,27 @@ void free_buffers(cos_batch* b) {
     cudaFree(b->d_tasks);
     cudaFree(b->d_joins);
     cudaFree(b->d_params);
+    cudaFree(b->d_chip);
     cudaFree(b->d_done);
     cudaFree(b->d_means);
     cudaFree(b->d_ctrl);
     cudaFreeHost(b->h_joins);
     cudaFreeHost(b->h_tasks);
     cudaFreeHost(b->h_params);
+    cudaFreeHost(b->h_chip);
     cudaFreeHost(b->h_means);
     cudaFreeHost(b->h_ctrl);
     b->d_tasks = nullptr;
     b->d_joins = nullptr;
     b->d_params = nullptr;
+    b->d_chip = nullptr;
     b->d_done = nullptr;
     b->d_means = nullptr;
     b->d_ctrl = nullptr;
     b->h_tasks = nullptr;
     b->h_joins = nullptr;
     b->h_params = nullptr;
+    b->h_chip = nullptr;
     b->h_means = nullptr;
     b->h_ctrl = nullptr;
     b->cap_tasks = b->cap_graphs = b->cap_joins = 0;
@@ -331,9 +350,13 @@ int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins) 
     }
     if (ngraphs > b->cap_graphs) {
         cudaFree(b->d_params);
+        cudaFree(b->d_chip);
         cudaFree(b->d_means);
         cudaFreeHost(b->h_params);
+        cudaFreeHost(b->h_chip);
         cudaFreeHost(b->h_means);
+        b->d_chip = nullptr;
+        b->h_chip = nullptr;
         b->d_params = nullptr;
         b->d_means = nullptr;
         b->h_params = nullptr;
@@ -342,6 +365,8 @@ int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins) 
         if ((e = cudaMalloc(&b->d_params, sizeof(WalkParams) * cap)) != cudaSuccess ||
             (e = cudaMalloc(&b->d_means, 2 * sizeof(double) * cap)) != cudaSuccess ||
             (e = cudaMallocHost(&b->h_params, sizeof(WalkParams) * cap)) != cudaSuccess ||
+            (e = cudaMalloc(&b->d_chip, sizeof(ChipParams) * cap)) != cudaSuccess ||
+            (e = cudaMallocHost(&b->h_chip, sizeof(ChipParams) * cap)) != cudaSuccess ||
             (e = cudaMallocHost(&b->h_means, 2 * sizeof(double) * cap)) != cudaSuccess)
             return set_error(COS_ERR_OOM, "batch parameters: %s", cudaGetErrorString(e));
         b->cap_graphs = cap;
@@ -364,6 +389,16 @@ int plan(cos_batch* b) {
     // per graph: its tasks in issue order; dep and joins as indices into the same list
     std::vector<std::vector<Task>> lists((size_t)b->n);
     std::vector<std::vector<std::vector<int32_t>>> local_joins((size_t)b->n);
+    // members that fit on chip, unless the batch or the member names a launch shape
+    struct OnChip {
+        int32_t g;
+        ChipParams p;
+        ChipPlan plan;
+    };
+    std::vector<OnChip> on_chip;
+    const cos_tuning& bt = b->tuning;
+    const bool chip_ok = !b->general_only && bt.samples_per_lane <= 0 && bt.rows_per_warp <= 0 && bt.blocks_per_sm <= 0 &&
+                         bt.layout <= 0 && bt.schedule <= 0 && bt.window_chunks <= 0 && bt.prefetch <= 0;
     for (int32_t g = 0; g < b->n; ++g) {
         cos_tuning tn;
         int rc = prepare_walk(b->graphs[(size_t)g], mode, &force, b->outs[(size_t)g], &b->params[(size_t)g], &tn);
@@ -373,6 +408,17 @@ int plan(cos_batch* b) {
         graph_view(b->graphs[(size_t)g], &gv);
         b->counts_overflow[(size_t)g] = gv.count_overflow;
         b->member_gen[(size_t)g] = gv.generation;
+        if (chip_ok) {
+            OnChip oc;
+            int yes = 0;
+            rc = prepare_chip(b->graphs[(size_t)g], mode, b->outs[(size_t)g], &oc.p, &oc.plan, &b->sms, &yes);
+            if (rc != COS_OK) return rc;
+            if (yes) {
+                oc.g = g;
+                on_chip.push_back(oc);
+                continue;   // no tasks
+            }
+        }
         graph_task_chain(b->params[(size_t)g], gv.widths_host, base_mode(mode), chv, force.window_chunks, g, false,
                          g == 0 && getenv("COS_TEST_STALL_TASK") != nullptr, lists[(size_t)g],
                          local_joins[(size_t)g]);
@@ -428,6 +474,26 @@ int plan(cos_batch* b) {
                              std::max<size_t>(b->joins.size(), 1));
     if (rc != COS_OK) return rc;
     for (int32_t g = 0; g < b->n; ++g) b->params[(size_t)g].mean_out = b->d_means + 2 * g;   // (mean R, mean A)
+    // one launch per (lane width, CTA size), its longest evaluations first
+    std::stable_sort(on_chip.begin(), on_chip.end(), [](const OnChip& x, const OnChip& y) {
+        if (x.plan.lane_bytes != y.plan.lane_bytes) return x.plan.lane_bytes > y.plan.lane_bytes;
+        if (x.plan.threads != y.plan.threads) return x.plan.threads > y.plan.threads;
+        return x.plan.cost > y.plan.cost;
+    });
+    b->chip.clear();
+    b->chip_launches.clear();
+    for (OnChip& oc : on_chip) {
+        if (b->chip_launches.empty() || b->chip_launches.back().lane_bytes != oc.plan.lane_bytes ||
+            b->chip_launches.back().threads != oc.plan.threads)
+            b->chip_launches.push_back({oc.plan.lane_bytes, oc.plan.threads, 0, (int)b->chip.size(), 0, 0});
+        cos_batch::ChipLaunch& cl = b->chip_launches.back();
+        oc.p.mean_out = b->d_means + 2 * oc.g;
+        oc.p.first_chunk = cl.chunks;
+        cl.chunks += oc.p.nchunks;
+        cl.n++;
+        cl.smem = std::max(cl.smem, oc.plan.smem);
+        b->chip.push_back(oc.p);
+    }
     drop_capture(b);
     b->planned = true;
     b->uploaded = false;
@@ -438,7 +504,8 @@ int plan(cos_batch* b) {
 // Counter reset + kernel: the part of a launch that is captured and replayed.
 int enqueue_run(cos_batch* b, cudaStream_t st) {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(b->d_done, 0, sizeof(unsigned) * std::max<int32_t>(b->ntasks, 1), st)) != cudaSuccess ||
+    if ((b->ntasks > 0 &&
+         (e = cudaMemsetAsync(b->d_done, 0, sizeof(unsigned) * b->ntasks, st)) != cudaSuccess) ||
         (e = cudaMemsetAsync(b->d_ctrl, 0, sizeof(BatchCtrl), st)) != cudaSuccess)
         return set_error(COS_ERR_CUDA, "reset batch counters: %s", cudaGetErrorString(e));
     BatchArgs a;
@@ -456,14 +523,21 @@ int enqueue_run(cos_batch* b, cudaStream_t st) {
     const size_t smem = (size_t)b->smem;
     if (b->total > 0 && (e = cudaLaunchKernel(k, dim3(b->grid), dim3(kThreads), args, smem, st)) != cudaSuccess)
         return set_error(COS_ERR_CUDA, "batch launch: %s", cudaGetErrorString(e));
+    for (size_t q = 0; q < b->chip_launches.size(); ++q) {
+        const cos_batch::ChipLaunch& cl = b->chip_launches[q];
+        const int rc = launch_chip_list(b->mode, cl.lane_bytes, cl.threads, cl.smem, b->d_chip + cl.first, cl.n, cl.chunks,
+                                        &b->d_ctrl->chip_ticket[q], &b->d_ctrl->chip_exits[q], b->sms, st);
+        if (rc != COS_OK) return rc;
+    }
     return COS_OK;
 }
 
 // Stream-ordered upload of the plan from pinned staging buffers.
 int upload(cos_batch* b, cudaStream_t st) {
-    const size_t nt = b->tasks.size(), nj = b->joins.size(), np = (size_t)b->n;
+    const size_t nt = b->tasks.size(), nj = b->joins.size(), np = (size_t)b->n, nc = b->chip.size();
     // The device already holds this exact plan (the kernel only reads it).
     if (b->staged_valid && b->staged_tasks == nt && b->staged_joins == nj && b->staged_params == np &&
+        b->staged_chip == nc && (nc == 0 || memcmp(b->h_chip, b->chip.data(), sizeof(ChipParams) * nc) == 0) &&
         (nt == 0 || memcmp(b->h_tasks, b->tasks.data(), sizeof(Task) * nt) == 0) &&
         (nj == 0 || memcmp(b->h_joins, b->joins.data(), sizeof(int32_t) * nj) == 0) &&
         (np == 0 || memcmp(b->h_params, b->params.data(), sizeof(WalkParams) * np) == 0)) {
@@ -487,12 +561,17 @@ int upload(cos_batch* b, cudaStream_t st) {
         memcpy(b->h_params, b->params.data(), sizeof(WalkParams) * b->n);
         e = cudaMemcpyAsync(b->d_params, b->h_params, sizeof(WalkParams) * b->n, cudaMemcpyHostToDevice, st);
     }
+    if (e == cudaSuccess && nc) {
+        memcpy(b->h_chip, b->chip.data(), sizeof(ChipParams) * nc);
+        e = cudaMemcpyAsync(b->d_chip, b->h_chip, sizeof(ChipParams) * nc, cudaMemcpyHostToDevice, st);
+    }
     if (e == cudaSuccess) e = cudaEventRecord(b->staged, st);
     if (e != cudaSuccess) return set_error(COS_ERR_CUDA, "upload plan: %s", cudaGetErrorString(e));
     b->staged_valid = true;
     b->staged_tasks = nt;
     b->staged_joins = nj;
     b->staged_params = np;
+    b->staged_chip = nc;
     b->uploaded = true;
     return COS_OK;
 }
@@ -516,6 +595,7 @@ int cosgpu::launch_windowed(cos_graph_t g, cos_batch_t* cache, int mode, void* p
     if (!b) {
         b = new (std::nothrow) cos_batch();
         if (!b) return set_error(COS_ERR_OOM, "host allocation failed");
+        b->general_only = true;
         *cache = b;
     }
     b->mode = mode;
@@ -679,19 +759,26 @@ int cos_batch_autotune(cos_batch_t b, void* stream, cos_tuning* best_out) {
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     int rc = COS_OK;
-    const int layouts[] = {1, 2, 3, 4};
+    // the first candidate is the tuning as it is, where it lets members run on chip
+    const int layouts[] = {0, 1, 2, 3, 4};
     for (int lay : layouts)
     for (int v : vecs) {
-        if (mode_has_abs(b->mode) && lay != 1) continue;    // sums of |path|: wide layout only
+        if (lay == 0 && v != vecs[0]) continue;
+        if (mode_has_abs(b->mode) && lay > 1) continue;     // sums of |path|: wide layout only
         if (base_mode(b->mode) == COS_MODE_FP64 && v == 4) continue;   // register-heavy; never faster in FP64
         if (lay == 2 && v == 1) continue;                   // identical to the wide layout
         for (int r : rpws) {
             cos_tuning t = base;
-            t.samples_per_lane = v;
-            t.rows_per_warp = r;
-            t.layout = lay;
+            if (lay == 0) {
+                if (r != rpws[0]) continue;
+            } else {
+                t.samples_per_lane = v;
+                t.rows_per_warp = r;
+                t.layout = lay;
+            }
             b->tuning = t;
             rc = plan(b);
+            if (lay == 0 && rc == COS_OK && b->chip.empty()) continue;
             if (rc == COS_OK) rc = upload(b, st);
             if (rc != COS_OK) break;
             float ms_best = 1e30f;

@@ -1,0 +1,1199 @@
+// On-chip walk: a CTA carries a chunk of samples through the whole evaluation --
+// exponentials, propagators, every level, sink -- in shared memory.
+//
+// The general kernels keep node values and propagators in global memory: every edge and
+// sample moves a parent value and a propagator (8 bytes in FP32) from L2 to an SM, and
+// the node values of the samples in flight, which exceed L2, move to HBM and back at
+// every level.  Here a chunk has only as many samples as the widest level and the
+// propagator slots of the graph allow in 227 KB of shared memory (8 float or 4 double
+// samples on the medium graph), so neither leaves the SM; global memory serves the
+// times, the edge words (4 bytes per edge and chunk, from L2) and one result per sample.
+//   level buffer  [row][RB bytes]: node values of the current level, RB bytes per row; the
+//                 next level goes to its free end, or, when both do not fit, to
+//   TMEM          until every row has read its parents: a second level buffer would halve
+//                 RB.  A thread stores and later loads only its own values (tcgen05.st /
+//                 ld, its warp's lanes), 256 KB per SM.
+//   propagators   [slot][RB bytes] of the chunk
+// A lane owns one 16-byte piece (8 or 4 when rows are that narrow) of two destination rows
+// and sums their in-edges in CSR order with the arithmetic of the general kernels, so the
+// results are bitwise theirs.
+//
+// What bounds it (ncu, medium graph, FP32, 16,384 samples): the shared-memory pipe, two
+// 16-byte reads per edge and lane, 68 % of all cycles busy, a third of that bank conflicts
+// that the row order of cos_chip.h leaves; issue slots 38 %, DRAM 0.  A chunk of 8 samples
+// takes 66,000 cycles, 43,000 of them in its four levels of 4,096 rows, 10,000 in the
+// propagators; a small level costs some 900 cycles whatever it holds.  Medium graph, 65,536
+// samples, before (general kernels) and after: FP32 2.35 -> 1.66 ms, with A 3.00 -> 2.24,
+// count 3.2 -> 1.91.  The FP64 walk is bound by the FP64 pipe on both paths (6.3 / 6.9 ms).
+//
+// CTAs never wait for one another: a CTA that has no chunk left sums its share of the
+// blocks of kReduceBlock samples that are complete, the last CTA the others, and it forms
+// the mean, in the fixed order of the general kernels (summing a block as soon as it is
+// complete put every sum, 8 us of dependent FP64 additions, on the one CTA that was
+// already last: 130 us per 16 blocks).
+#include <algorithm>
+#include <cstdio>
+#include <type_traits>
+
+#include "cos_chip.cuh"
+#include "cos_chip.h"
+#include "cos_items.cuh"
+
+namespace cosgpu {
+namespace {
+
+// ---------------------------------------------------------------- tensor memory
+
+__device__ __forceinline__ void tmem_alloc(unsigned* smem_dst, unsigned cols) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)), "r"(cols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc(unsigned addr, unsigned cols) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(cols) : "memory");
+}
+
+// A lane's pieces of its two rows as 32-bit registers.
+template <int LB>
+struct alignas(16) Pair {
+    unsigned w[LB / 2];
+};
+
+template <int LB>
+__device__ __forceinline__ void tmem_put(unsigned addr, const Pair<LB>& x) {
+    if constexpr (LB == 16)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr), "r"(x.w[0]),
+                     "r"(x.w[1]), "r"(x.w[2]), "r"(x.w[3]), "r"(x.w[4]), "r"(x.w[5]), "r"(x.w[6]), "r"(x.w[7])
+                     : "memory");
+    else if constexpr (LB == 8)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(x.w[0]), "r"(x.w[1]),
+                     "r"(x.w[2]), "r"(x.w[3])
+                     : "memory");
+    else
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(x.w[0]), "r"(x.w[1])
+                     : "memory");
+}
+// (the values may be used after tmem_wait_ld)
+template <int LB>
+__device__ __forceinline__ void tmem_get(unsigned addr, Pair<LB>& x) {
+    if constexpr (LB == 16)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(x.w[0]), "=r"(x.w[1]), "=r"(x.w[2]), "=r"(x.w[3]), "=r"(x.w[4]), "=r"(x.w[5]), "=r"(x.w[6]),
+                       "=r"(x.w[7])
+                     : "r"(addr)
+                     : "memory");
+    else if constexpr (LB == 8)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(x.w[0]), "=r"(x.w[1]), "=r"(x.w[2]), "=r"(x.w[3])
+                     : "r"(addr)
+                     : "memory");
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(x.w[0]), "=r"(x.w[1]) : "r"(addr) : "memory");
+}
+// Ties the loaded registers to the wait, so that no use of them moves ahead of it.
+template <int LB>
+__device__ __forceinline__ void tmem_wait_ld(Pair<LB>& x) {
+    if constexpr (LB == 16)
+        asm volatile("tcgen05.wait::ld.sync.aligned;"
+                     : "+r"(x.w[0]), "+r"(x.w[1]), "+r"(x.w[2]), "+r"(x.w[3]), "+r"(x.w[4]), "+r"(x.w[5]), "+r"(x.w[6]),
+                       "+r"(x.w[7])::"memory");
+    else if constexpr (LB == 8)
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(x.w[0]), "+r"(x.w[1]), "+r"(x.w[2]), "+r"(x.w[3])::"memory");
+    else
+        asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(x.w[0]), "+r"(x.w[1])::"memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// ---------------------------------------------------------------- shared-memory layout
+
+// Scratch of the propagator phase, in the level buffer behind the zero row and the root's
+// (256 bytes): one word per pair (i, j) whose bit b says t_i >= t_j for sample b, then
+// three arrays [kinds][D][pitch] of 8 bytes.
+constexpr int kScratchAt = 256;
+__host__ __device__ constexpr int chip_pair_bytes(int D) { return (4 * D * D + 15) / 16 * 16; }
+// Values between the rows (kind, time) of a scratch array: two more than the samples, so
+// that the rows of neighbouring slots start in different banks (and stay 16-byte aligned).
+__host__ __device__ constexpr int chip_pitch(int s) { return s > 1 ? s + 2 : 1; }
+
+// A level before the sink of at most this many rows has a place of its own, so that the
+// sink is summed while the next chunk's exponentials are formed in the level buffer.
+constexpr int kTailRows = 64;
+
+// Constants of the graph: the mode's 2^{j/64} table (128 values of 8 bytes), then per
+// kind coef+ and coef- as doubles, the same as float-float pairs, eps, and one word per
+// kind (1: float-float arithmetic applies).
+__host__ __device__ constexpr int chip_coef_bytes(int K) { return 1024 + 44 * K; }
+struct Consts {
+    const double* tab;
+    const double* cf;
+    const float2* cff;
+    const double* eps;
+    const int* ff;
+    __device__ __forceinline__ Consts(const unsigned char* sm, int off, int K)
+        : tab(reinterpret_cast<const double*>(sm + off)), cf(tab + 128), cff(reinterpret_cast<const float2*>(cf + 2 * K)),
+          eps(reinterpret_cast<const double*>(cff + 2 * K)), ff(reinterpret_cast<const int*>(eps + K)) {}
+};
+
+__host__ __device__ constexpr int round128(int64_t x) { return (int)((x + 127) / 128 * 128); }
+
+struct ChipArgs {
+    ChipParams one;
+    const ChipParams* list;   // nullptr: `one`, chunks dealt out by CTA number
+    unsigned* ticket;
+    unsigned* exits;          // CTAs that have left (zero between launches)
+    int n, total;
+    int tmem_cols;
+    int few;                  // so few blocks of samples that the last CTA sums them all
+};
+
+// ---------------------------------------------------------------- propagators of a chunk
+
+// Once per graph and CTA: constants of every kind, level and group tables, the zero
+// propagator row.
+template <int MODE>
+__device__ __forceinline__ void chip_setup(const ChipParams& p, unsigned char* sm) {
+    int4* tab = reinterpret_cast<int4*>(sm + p.tab_off);
+    for (int x = threadIdx.x; x < p.g.tables; x += blockDim.x)
+        if (x >= p.L) tab[x] = __ldg(p.g.lev + x);
+    if (threadIdx.x == 0) {
+        // where each level goes: a free part of the level buffer, or through TMEM (sign bit)
+        // to its start once every parent is read; the level before the sink to its own place
+        const int rb = 1 << p.rb_log2;
+        int cur = p.L == 2 ? p.tail_off : 0, before = round128(2 * rb);
+        for (int l = 0; l + 1 < p.L; ++l) {
+            int4 lv = l ? __ldg(p.g.lev + l) : make_int4(1, 1, 0, 0);
+            if (l > 0) {
+                const int need = round128((int64_t)(lv.x + 1) * rb);
+                const bool tail = l + 2 == p.L && p.tail_off >= 0;
+                const bool staged = !tail && before + need > p.lev_bytes;
+                cur = tail ? p.tail_off : staged || cur != 0 ? 0 : p.lev_bytes - need;
+                before = need;
+                lv.w = cur | (staged ? (int)0x80000000 : 0);
+            } else {
+                lv.w = cur;
+            }
+            tab[l] = lv;
+        }
+    }
+    if constexpr (!Traits<MODE>::kCount) {
+        const int gb = (1 << p.rb_log2) >> (Traits<MODE>::kAbs ? 1 : 0);
+        if ((int)threadIdx.x * 4 < gb) reinterpret_cast<unsigned*>(sm + p.g_off + (size_t)p.P * gb)[threadIdx.x] = 0u;
+        const Consts c(sm, p.coef_off, p.K);
+        const double* tab64 = p.exp_tab + (Traits<MODE>::kBase == COS_MODE_FP32_MIXED ? 128 : 0);
+        for (int x = threadIdx.x; x < 128; x += blockDim.x) const_cast<double*>(c.tab)[x] = __ldg(tab64 + x);
+        // kinds from the last thread downwards, a thread per prefactor
+        for (int x = blockDim.x - 1 - threadIdx.x; x < 2 * p.K; x += blockDim.x) {
+            const int k = x < p.K ? x : x - p.K;
+            const double e = __ldg(p.eps + k), be = p.beta * e;
+            // -1/(1+e^{-beta eps}) (tau >= 0), 1/(1+e^{beta eps}) (tau < 0)
+            const double v = (x < p.K ? -1.0 : 1.0) / (1.0 + exp(x < p.K ? -be : be));
+            const_cast<double*>(c.cf)[x] = v;
+            const_cast<float2*>(c.cff)[x] = split_ff(v);
+            if (x >= p.K) continue;
+            const_cast<double*>(c.eps)[k] = e;
+            const_cast<int*>(c.ff)[k] = fabs(e) * p.beta <= 30.0 ? 1 : 0;
+        }
+    }
+}
+
+// Start the copy of a chunk's times into the times buffer [D][s].
+template <int MODE>
+__device__ __forceinline__ void chip_times(const ChipParams& p, unsigned char* sm, int chunk) {
+    if constexpr (!Traits<MODE>::kCount) {
+        double* st = reinterpret_cast<double*>(sm + p.times_off);
+        const int sl = p.s_log2, n = p.D << sl;
+        const double* t = p.t + ((int64_t)chunk << sl);
+        for (int x = threadIdx.x; x < n; x += blockDim.x)
+            cp_async_lane<8>(st + x, t + (int64_t)(x >> sl) * p.t_ld + (x & ((1 << sl) - 1)));
+        cp_async_commit();
+    }
+}
+
+// |x| <= 30 by 32-bit integer comparison (false for NaN).
+__device__ __forceinline__ bool within_30(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    return hi < 0x403e0000u || (hi == 0x403e0000u && __double2loint(x) == 0);
+}
+
+// Exponentials of the kinds [k0, k0 + kn), times and samples of the chunk, with the
+// arithmetic of item_props of the general kernels.  Returns whether a time lies so far
+// outside [-beta, beta] that float-float arithmetic does not apply (then the caller
+// repeats the pass in double).
+template <int MODE>
+__device__ __forceinline__ bool chip_exps(const ChipParams& p, unsigned char* sm, int k0, int kn, bool in_double) {
+    using Tr = Traits<MODE>;
+    const int sl = p.s_log2, s = 1 << sl, D = p.D, DS = D << sl, n = kn * DS, pitch = chip_pitch(s), np = kn * D * pitch;
+    const double* st = reinterpret_cast<const double*>(sm + p.times_off);
+    const Consts c(sm, p.coef_off, p.K);
+    double* fa = reinterpret_cast<double*>(sm + kScratchAt + chip_pair_bytes(D));   // [kn][D][pitch]: coef+ e^{-eps t}
+    double* fb = fa + np;                                                           // coef- e^{-eps t}
+    double* fc = fb + np;                                                           // e^{+eps t}
+    const int T = blockDim.x;
+    bool far = false;
+    if (Tr::kBase == COS_MODE_FP32_MIXED && !in_double) {
+        // two independent chains per thread; warp 0, which has a sink to sum, comes last
+        const int half = (n + 1) / 2;
+        for (int x0 = T - 1 - (int)threadIdx.x; x0 < half; x0 += T) {
+            float2 em[2], ep[2];
+            int k[2], at[2];
+            bool ok[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int x = x0 + u * half < n ? x0 + u * half : x0;
+                const unsigned r = (unsigned)x >> sl;
+                at[u] = (int)r * pitch + (x & (s - 1));
+                const int kk = D == 1 ? (int)r : (int)__umulhi(r, p.d_magic);
+                k[u] = k0 + kk;
+                const double arg = c.eps[k[u]] * st[x - kk * DS];
+                ok[u] = within_30(arg);
+                exp_pair_ff(ok[u] ? arg : 0.0, reinterpret_cast<const float2*>(c.tab), em[u], ep[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (!c.ff[k[u]]) continue;   // (formed in double below)
+                if (!ok[u]) far = true;
+                reinterpret_cast<float2*>(fa)[at[u]] = mul_ff2(c.cff[k[u]], em[u]);
+                reinterpret_cast<float2*>(fb)[at[u]] = mul_ff2(c.cff[p.K + k[u]], em[u]);
+                reinterpret_cast<float2*>(fc)[at[u]] = ep[u];
+            }
+        }
+    }
+    for (int x = T - 1 - (int)threadIdx.x; x < n; x += T) {
+        const unsigned r = (unsigned)x >> sl;
+        const int kk = D == 1 ? (int)r : (int)__umulhi(r, p.d_magic), k = k0 + kk;
+        if (Tr::kBase == COS_MODE_FP32_MIXED && !in_double && c.ff[k]) continue;
+        const double arg = c.eps[k] * st[x - kk * DS];
+        double em, ep;
+        if constexpr (Tr::kBase == COS_MODE_FP32_MIXED) exp_pair(arg, p.exp_tab, em, ep);   // (rare: the table at hand is the other)
+        else exp_pair_at(arg, c.tab, em, ep);
+        const int at = (int)r * pitch + (x & (s - 1));
+        fa[at] = c.cf[k] * em;
+        fb[at] = c.cf[p.K + k] * em;
+        fc[at] = ep;
+    }
+    return far;
+}
+
+// Bit b of pair (i, j): t_i >= t_j of the chunk's sample b.
+__device__ __forceinline__ void chip_pairs(const ChipParams& p, unsigned char* sm) {
+    const int sl = p.s_log2, s = 1 << sl, D = p.D, n = (D * D) << sl, lane = threadIdx.x & 31;
+    const double* st = reinterpret_cast<const double*>(sm + p.times_off);
+    unsigned* pair = reinterpret_cast<unsigned*>(sm + kScratchAt);
+    for (int x0 = ((int)threadIdx.x & ~31); x0 < n; x0 += blockDim.x) {
+        const int x = min(x0 + lane, n - 1), q = x >> sl, b = x & (s - 1);
+        const int i = D == 1 ? q : (int)__umulhi((unsigned)q, p.d_magic), j = q - i * D;
+        const bool ge = key_ge(time_order_key(st[(i << sl) + b]), time_order_key(st[(j << sl) + b]));
+        const unsigned bits = __ballot_sync(0xffffffffu, ge);
+        if (x0 + lane < n && b == 0) pair[q] = s == 32 ? bits : (bits >> lane) & ((1u << s) - 1u);
+    }
+}
+
+// This thread's slots of the kinds [k0, k0 + kn): pieces x, x + T, ... below `end`, the
+// first kAhead descriptors loaded (ahead of the exponentials).
+constexpr int kAhead = 4;
+struct SlotRange {
+    int x, end;
+    uint2 sd[kAhead];
+    __device__ __forceinline__ void load(const ChipParams& p, int pl) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+            if (x + u * (int)blockDim.x < end) sd[u] = __ldg(p.g.slots + ((x + u * (int)blockDim.x) >> pl));
+    }
+    __device__ __forceinline__ void open(const ChipParams& p, int k0, int kn, int pl) {
+        const bool all = kn == p.K;
+        x = (all ? 0 : __ldg(p.kind_slot + k0) << pl) + (int)threadIdx.x;
+        end = (all ? p.P : __ldg(p.kind_slot + k0 + kn)) << pl;
+        load(p, pl);
+    }
+};
+
+// V doubles from shared memory, two per access.
+template <int V>
+__device__ __forceinline__ VecT<double, V> load_pair(const double* x) {
+    VecT<double, V> r;
+    if constexpr (V == 1) {
+        r.v[0] = x[0];
+    } else {
+#pragma unroll
+        for (int v = 0; v < V; v += 2) {
+            const double2 d = *reinterpret_cast<const double2*>(x + v);
+            r.v[v] = d.x;
+            r.v[v + 1] = d.y;
+        }
+    }
+    return r;
+}
+// A scratch value that holds a float-float pair.
+__device__ __forceinline__ float2 as_ff(double x) {
+    return make_float2(__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x)));
+}
+
+// Propagators of the slots of kinds [k0, k0 + kn); a thread forms V samples of a slot.
+template <int MODE, int V>
+__device__ __forceinline__ void chip_slots(const ChipParams& p, unsigned char* sm, int k0, int kn, bool in_double, SlotRange& r) {
+    using Tr = Traits<MODE>;
+    using Prop = typename Tr::Prop;
+    constexpr bool kMixed = Tr::kBase == COS_MODE_FP32_MIXED;
+    constexpr int VL = V == 4 ? 2 : V == 2 ? 1 : 0;
+    const int sl = p.s_log2, D = p.D, pitch = chip_pitch(1 << sl), np = kn * D * pitch;
+    const int pl = sl - VL, T = blockDim.x;   // pl: log2 pieces per slot
+    const Consts c(sm, p.coef_off, p.K);
+    const unsigned* pair = reinterpret_cast<const unsigned*>(sm + kScratchAt);
+    const double* fa = reinterpret_cast<const double*>(sm + kScratchAt + chip_pair_bytes(D));
+    const double* fb = fa + np;
+    const double* fc = fb + np;
+    Prop* G = reinterpret_cast<Prop*>(sm + p.g_off);
+    const int ahi = p.abs_weights ? 0x7fffffff : -1;
+    while (r.x < r.end) {
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const int x = r.x + u * T;
+            if (x >= r.end) break;
+            const uint2 sd = r.sd[u];
+            const int smp = (x & ((1 << pl) - 1)) << VL;
+            const unsigned ge = pair[sd.y & 0xffffu] >> smp;   // tau = t_i - t_j >= 0 ?
+            const int shi = (int)(sd.y & 0x80000000u);
+            const int xi = ((int)(sd.x & 0xffffu) - k0 * D) * pitch + smp;
+            const int xj = ((int)(sd.x >> 16) - k0 * D) * pitch + smp;
+            // V values of 8 bytes, aligned to 16 when there are more than one; neighbouring
+            // slots share (kind, i), so fetching both prefactors' rows costs few wavefronts
+            const VecT<double, V> vp = load_pair<V>(fa + xi), vn = load_pair<V>(fb + xi), ve = load_pair<V>(fc + xj);
+            VecT<Prop, V> out;
+            if (kMixed && !in_double && c.ff[(sd.y >> 16) & 0x7fff]) {
+#pragma unroll
+                for (int v = 0; v < V; ++v) {
+                    const float g = mul_ff(as_ff((ge >> v) & 1u ? vp.v[v] : vn.v[v]), as_ff(ve.v[v]));
+                    out.v[v] = (Prop)__uint_as_float((__float_as_uint(g) ^ (unsigned)shi) & (unsigned)ahi);
+                }
+            } else {
+#pragma unroll
+                for (int v = 0; v < V; ++v)
+                    out.v[v] = (Prop)sign_ops(((ge >> v) & 1u ? vp.v[v] : vn.v[v]) * ve.v[v], shi, ahi);
+            }
+            *reinterpret_cast<VecT<Prop, V>*>(G + ((size_t)x << VL)) = out;
+        }
+        r.x += kAhead * T;
+        r.load(p, pl);
+    }
+}
+
+// As chip_slots for user-tabulated propagators (see item_props).
+template <int MODE>
+__device__ __forceinline__ void chip_slots_table(const ChipParams& p, unsigned char* sm) {
+    using Prop = typename Traits<MODE>::Prop;
+    const int sl = p.s_log2, D = p.D, PT = p.ptab_T, n = p.P << sl, T = blockDim.x;
+    const double* st = reinterpret_cast<const double*>(sm + p.times_off);
+    Prop* G = reinterpret_cast<Prop*>(sm + p.g_off);
+    const int ahi = p.abs_weights ? 0x7fffffff : -1;
+    int x = threadIdx.x;
+    uint2 sd = x < n ? __ldg(p.g.slots + (x >> sl)) : make_uint2(0, 0);
+    while (x < n) {
+        uint2 next = sd;
+        if (x + T < n) next = __ldg(p.g.slots + ((x + T) >> sl));
+        const int smp = x & ((1 << sl) - 1);
+        const int k = (sd.y >> 16) & 0x7fff, i = (int)(sd.x & 0xffffu) - k * D, j = (int)(sd.x >> 16) - k * D;
+        const int shi = (int)(sd.y & 0x80000000u);
+        const double2* tk = reinterpret_cast<const double2*>(p.ptab) + (int64_t)k * 2 * PT;
+        const double tau = st[(i << sl) + smp] - st[(j << sl) + smp];
+        const bool pos = tau >= 0.0;
+        const double u = __dadd_rn(__dmul_rn(tau, p.ptab_inv_h), pos ? 0.0 : (double)PT);
+        int m = (int)u;
+        double f = __dsub_rn(u, (double)m);
+        if (u < 0.0) {
+            m = 0;
+            f = 0.0;
+        } else if (m >= PT) {
+            m = PT - 1;
+            f = 1.0;
+        }
+        const double2 as = __ldg(tk + (pos ? 0 : PT) + m);
+        G[x] = (Prop)sign_ops(__dadd_rn(as.x, __dmul_rn(f, as.y)), shi, ahi);
+        x += T;
+        sd = next;
+    }
+}
+
+// ---------------------------------------------------------------- rows
+
+// This lane's words (two rows) of a block with n words per row left (see cos_chip.h).
+struct Words {
+    uint4 a, b;
+};
+__device__ __forceinline__ void load_words(Words& m, const uint32_t* block, unsigned n, int r32) {
+    if (n == 1) {
+        const uint2 q = __ldg(reinterpret_cast<const uint2*>(block) + r32);
+        m.a.x = q.x;
+        m.a.y = q.y;
+    } else {
+        m.a = __ldg(reinterpret_cast<const uint4*>(block) + r32);
+        if (n > 2) m.b = __ldg(reinterpret_cast<const uint4*>(block) + 32 + r32);
+    }
+}
+
+// A lane's pieces of two destination rows: the in-edges in order, one multiply-add each.
+// par and pro: byte offsets in shared memory of this lane's piece of place 0 and slot 0.
+template <int MODE, int LB>
+struct RowSum {
+    using Tr = Traits<MODE>;
+    using Val = typename Tr::Val;
+    using Prop = typename Tr::Prop;
+    static constexpr int V = LB / (int)sizeof(Val);
+    using VecV = VecT<Val, V>;
+    using VecG = VecT<Prop, V>;
+
+    int par, pro;
+    int rb, gb;                       // row bytes of a node and of a slot
+    bool use_abs;                     // this lane sums A (|G|)
+    VecV acc[2];
+
+    __device__ __forceinline__ VecV parent(const unsigned char* sm, unsigned m) const {
+        return *reinterpret_cast<const VecV*>(sm + ((int)(m & 0xffffu) * rb + par));
+    }
+    __device__ __forceinline__ VecG factor(const unsigned char* sm, unsigned m) const {
+        if constexpr (Tr::kCount) return VecG{};
+        else return *reinterpret_cast<const VecG*>(sm + ((int)(m >> 16) * gb + pro));
+    }
+    __device__ __forceinline__ void add(VecV& s, const VecV& a, const VecG& g) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            if constexpr (Tr::kCount) s.v[v] += a.v[v];
+            else if constexpr (Tr::kAbs) s.v[v] = fmaf(a.v[v], use_abs ? abs_to_float(g.v[v]) : g.v[v], s.v[v]);
+            else s.v[v] = madd(a.v[v], g.v[v], s.v[v]);
+        }
+    }
+    // the next N in-edges of both rows, their loads ahead of the multiply-adds
+    template <int N>
+    __device__ __forceinline__ void steps(const unsigned char* sm, const unsigned (&w0)[N], const unsigned (&w1)[N]) {
+        VecV a0[N], a1[N];
+        VecG g0[N], g1[N];
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            a0[e] = parent(sm, w0[e]);
+            g0[e] = factor(sm, w0[e]);
+            a1[e] = parent(sm, w1[e]);
+            g1[e] = factor(sm, w1[e]);
+        }
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            add(acc[0], a0[e], g0[e]);
+            add(acc[1], a1[e], g1[e]);
+        }
+    }
+    __device__ __forceinline__ void block(const unsigned char* sm, const Words& m, unsigned n) {
+        const uint4 &a = m.a, &b = m.b;
+        if (n == 1) {
+            const unsigned w0[1] = {a.x}, w1[1] = {a.y};
+            steps<1>(sm, w0, w1);
+        } else if (n == 2) {
+            const unsigned w0[2] = {a.x, a.y}, w1[2] = {a.z, a.w};
+            steps<2>(sm, w0, w1);
+        } else if (n == 3) {
+            const unsigned w0[3] = {a.x, a.y, a.z}, w1[3] = {b.x, b.y, b.z};
+            steps<3>(sm, w0, w1);
+        } else {
+            const unsigned w0[2] = {a.x, a.y}, w1[2] = {b.x, b.y};
+            steps<2>(sm, w0, w1);
+            const unsigned w2[2] = {a.z, a.w}, w3[2] = {b.z, b.w};
+            steps<2>(sm, w2, w3);
+        }
+    }
+    // n in-edges whose first words are m and whose first block is b
+    __device__ __forceinline__ void rows(const unsigned char* sm, const Words& m, unsigned n, const uint32_t* b, int r32) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[0].v[v] = acc[1].v[v] = (Val)0;
+        block(sm, m, n);
+        while (n > 4) {
+            n -= 4;
+            b += 4 * kChipGroup;
+            Words q;
+            load_words(q, b, n, r32);
+            block(sm, q, n);
+        }
+    }
+};
+
+// ---------------------------------------------------------------- sample reduction
+
+__device__ __forceinline__ double ld_cg_f64(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ double ld_cg_f64(const long long* p) { return (double)__ldcg(p); }
+
+// One compensated addition as neumaier_add, without branches: the error of sum + y from
+// the larger operand (chosen by 32-bit comparison) is the same number.
+__device__ __forceinline__ bool bigger(double sum, double y) {   // |sum| >= |y|
+    const unsigned sh = (unsigned)__double2hiint(sum) & 0x7fffffffu, yh = (unsigned)__double2hiint(y) & 0x7fffffffu;
+    return sh > yh || (sh == yh && (unsigned)__double2loint(sum) >= (unsigned)__double2loint(y));
+}
+__device__ __forceinline__ void compensated_add(double& sum, double& comp, double y) {
+    const double u = sum + y;
+    const bool ge = bigger(sum, y);
+    comp += ((ge ? sum : y) - u) + (ge ? y : sum);
+    sum = u;
+}
+
+// As block_sum and partials_sum of the general kernels (same order, same result), with
+// L2 loads: the values come from other CTAs of this launch.  All loads are issued first
+// and the additions have no branches, so that the running sum is the only serial chain.
+template <typename T>
+__device__ __forceinline__ double chip_block_sum(const T* x, int64_t S, int64_t b, int lane) {
+    constexpr int per_lane = kReduceBlock / 32;
+    const int64_t s0 = b * kReduceBlock + lane;
+    double v[per_lane];
+#pragma unroll
+    for (int u = 0; u < per_lane; ++u) v[u] = s0 + u * 32 < S ? ld_cg_f64(x + s0 + u * 32) : 0.0;
+    double sum = 0.0, comp = 0.0;
+#pragma unroll
+    for (int u = 0; u < per_lane; ++u) compensated_add(sum, comp, v[u]);
+    warp_sum(sum, comp);
+    return sum + comp;
+}
+__device__ __forceinline__ void chip_partials_sum(const double* x, int64_t n, int lane, double& sum, double& comp) {
+    sum = 0.0;
+    comp = 0.0;
+    if (n == 1) {   // one finite partial sum is the sum: the tree would add zeros to it
+        const double v = __ldcg(x);
+        if (((unsigned)__double2hiint(v) & 0x7fffffffu) < 0x7ff00000u) {
+            sum += v;
+            return;
+        }
+    }
+    for (int64_t b = lane; b < n; b += 32) compensated_add(sum, comp, __ldcg(x + b));
+    warp_sum(sum, comp);
+}
+
+// Blocks of an evaluation that has few of them, by teams of four warps: one FP64
+// operation takes 64 cycles of an SM quarter whatever its lanes do, so the four chains of
+// a block's compensated sum run on four quarters -- running sums, rounding errors (two
+// warps), sum of errors -- in chunks of eight values, each a phase behind the other
+// (one warp: 15,800 cycles per block).  Same numbers as chip_block_sum.  Uses kTeamBytes of shared memory per team; called by the whole CTA.
+constexpr int kTeamBytes = (33 + 32 + 1) * 32 * 8;
+template <typename T>
+__device__ __noinline__ void team_sums(const T* x, double* partials, int64_t S, unsigned char* sm) {
+    const int lane = threadIdx.x & 31, role = (threadIdx.x >> 5) & 3, team = threadIdx.x >> 7;
+    const int teams = min((int)blockDim.x >> 7, (int)(dynamic_smem_bytes() / kTeamBytes));
+    const int nblk = (int)((S + kReduceBlock - 1) / kReduceBlock);
+    double(*U)[32] = reinterpret_cast<double(*)[32]>(sm + team * kTeamBytes);   // running sums before each value
+    double(*E)[32] = U + 33;                                                    // rounding errors
+    for (int b0 = 0; b0 < nblk; b0 += teams) {
+        const bool mine = team < teams && b0 + team < nblk;
+        const int64_t s0 = (int64_t)(b0 + team) * kReduceBlock + lane;
+        double acc = 0.0, y[32];   // the values this warp needs: all, or every other one
+        if (mine && role != 3) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+                const int64_t s = s0 + (role == 0 ? i : 2 * i + role - 1) * 32;
+                if (role == 0 || i < 16) y[i] = s < S ? ld_cg_f64(x + s) : 0.0;
+            }
+        }
+        if (mine && role == 0) U[0][lane] = 0.0;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            __syncthreads();
+            if (!mine) continue;
+            if (role == 0) {
+                if (c < 4)
+#pragma unroll
+                    for (int i = 8 * c; i < 8 * c + 8 && i < 32; ++i) U[i + 1][lane] = acc = acc + y[i];
+            } else if (role == 3) {
+                if (c >= 2)
+#pragma unroll
+                    for (int i = 8 * c - 16; i < 8 * c - 8; ++i)
+                        if (i >= 0) acc += E[i][lane];
+            } else if (c >= 1 && c < 5) {
+#pragma unroll
+                for (int h = 4 * c - 4; h < 4 * c; ++h) {
+                    if (h < 0 || h >= 16) continue;
+                    const int i = 2 * h + role - 1;
+                    const double sum = U[i][lane], u = U[i + 1][lane], v = y[h];
+                    const bool ge = bigger(sum, v);
+                    E[i][lane] = ((ge ? sum : v) - u) + (ge ? v : sum);
+                }
+            }
+        }
+        __syncthreads();
+        if (mine && role == 3) E[32][lane] = acc;   // (one row behind the errors)
+        __syncthreads();
+        if (mine && role == 0) {
+            double comp = E[32][lane];
+            warp_sum(acc, comp);
+            if (lane == 0) partials[b0 + team] = acc + comp;
+        }
+    }
+    __syncthreads();
+}
+template <int MODE>
+__device__ __forceinline__ void chip_sum_few(const ChipParams& p, unsigned char* sm) {
+    if constexpr (Traits<MODE>::kCount) team_sums(static_cast<const long long*>(p.R), p.partials, p.S, sm);
+    else team_sums(static_cast<const double*>(p.R), p.partials, p.S, sm);
+    if constexpr (Traits<MODE>::kAbs) team_sums(p.Rabs, p.partials_abs, p.S, sm);
+}
+
+constexpr unsigned kBlockSummed = 0xffffffffu;   // arrival word of a block whose partial sum is written
+
+// Count a chunk's results in (one thread; they were written by its warp).  Called a
+// phase after the writes, when the release has nothing left to wait for.
+__device__ __forceinline__ void chip_arrive(const ChipParams& p, int chunk) {
+    const int64_t s0 = (int64_t)chunk << p.s_log2;
+    const unsigned mine = (unsigned)min((int64_t)1 << p.s_log2, p.S - s0);
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.arrive + s0 / kReduceBlock), "r"(mine) : "memory");
+}
+
+// Partial sum of block b by one warp.
+template <int MODE>
+__device__ __noinline__ void chip_sum_block(const ChipParams& p, int64_t b, int lane) {
+    double v, va = 0.0;
+    if constexpr (Traits<MODE>::kCount) v = chip_block_sum(static_cast<const long long*>(p.R), p.S, b, lane);
+    else v = chip_block_sum(static_cast<const double*>(p.R), p.S, b, lane);
+    if constexpr (Traits<MODE>::kAbs) va = chip_block_sum(p.Rabs, p.S, b, lane);
+    if (lane == 0) {
+        p.partials[b] = v;
+        if constexpr (Traits<MODE>::kAbs) p.partials_abs[b] = va;
+    }
+}
+
+// A CTA that has no chunk left sums its share of the evaluation's blocks, as far as
+// they are complete; `first`: number of this evaluation's block 0 in the launch.
+template <int MODE>
+__device__ __forceinline__ void chip_sum_own(const ChipParams& p, int first) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nblk = (int)((p.S + kReduceBlock - 1) / kReduceBlock), grid = gridDim.x;
+    const int b0 = (int)((blockIdx.x + grid - first % grid) % grid);
+    for (int b = b0 + warp * grid; b < nblk; b += nw * grid) {
+        const unsigned full = (unsigned)min((int64_t)kReduceBlock, p.S - (int64_t)b * kReduceBlock);
+        const unsigned got = lane == 0 ? ld_acquire_gpu_u32(p.arrive + b) : 0u;
+        if (__shfl_sync(0xffffffffu, got, 0) != full) continue;
+        chip_sum_block<MODE>(p, b, lane);
+        __syncwarp();
+        if (lane == 0) p.arrive[b] = kBlockSummed;   // (read by the last CTA, after this one's release)
+    }
+}
+
+// The last CTA of the launch: the blocks nobody has summed, then the means.  The
+// arrival words are left at zero.
+template <int MODE>
+__device__ __forceinline__ void chip_sum_rest(const ChipParams& p) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nblk = (int)((p.S + kReduceBlock - 1) / kReduceBlock);
+    for (int b = warp; b < nblk; b += nw) {
+        const unsigned got = __shfl_sync(0xffffffffu, lane == 0 ? __ldcg(p.arrive + b) : 0u, 0);
+        if (got != kBlockSummed) chip_sum_block<MODE>(p, b, lane);
+        if (lane == 0) p.arrive[b] = 0;
+    }
+}
+template <int MODE>
+__device__ __noinline__ void chip_mean(const ChipParams& p, int lane) {
+    const int64_t nblk = (p.S + kReduceBlock - 1) / kReduceBlock;
+    double sum, comp, sa = 0.0, ca = 0.0;
+    chip_partials_sum(p.partials, nblk, lane, sum, comp);
+    if constexpr (Traits<MODE>::kAbs) chip_partials_sum(p.partials_abs, nblk, lane, sa, ca);
+    if (lane == 0) {
+        const double mean = (sum + comp) / (double)p.S, mean_abs = (sa + ca) / (double)p.S;
+        p.ctrl->sum = sum;
+        p.ctrl->comp = comp;
+        p.ctrl->mean = mean;
+        p.ctrl->mean_abs = mean_abs;
+        if (p.clear_err) {
+            p.ctrl->err = 0;
+            p.ctrl->err_detail = 0;
+        }
+        if (p.mean_out) {
+            p.mean_out[0] = mean;
+            if constexpr (Traits<MODE>::kAbs) p.mean_out[1] = mean_abs;
+        }
+    }
+}
+
+// ---------------------------------------------------------------- kernel
+
+// Sink of chunk `chunk` by one warp: one lane per sample, in-edges in order; parents at
+// byte `base` of shared memory.
+template <int MODE>
+__device__ __forceinline__ void chip_sink(const ChipParams& p, unsigned char* sm, int base, int chunk, unsigned word) {
+    using Tr = Traits<MODE>;
+    using Val = typename Tr::Val;
+    using Prop = typename Tr::Prop;
+    using Out = typename Tr::SinkAcc;
+    const int lane = threadIdx.x & 31, s = 1 << p.s_log2, smp = lane & (s - 1);
+    const int rb = 1 << p.rb_log2, gb = Tr::kAbs ? rb / 2 : rb;
+    const unsigned char* G = sm + p.g_off;
+    Out acc = (Out)0, acca = (Out)0;
+    for (int e = 0; e < p.g.nsink; ++e) {
+        const unsigned m = e < 32 ? __shfl_sync(0xffffffffu, word, e) : __ldg(p.g.sink + e);
+        const Val* pr = reinterpret_cast<const Val*>(sm + base + (int)(m & 0xffffu) * rb);
+        if constexpr (Tr::kCount) {
+            acc += pr[smp];
+        } else {
+            const Prop g = reinterpret_cast<const Prop*>(G + (int)(m >> 16) * gb)[smp];
+            if constexpr (Tr::kBase == COS_MODE_FP32_MIXED) {
+                acc += (double)pr[smp] * (double)g;   // exact product
+                if constexpr (Tr::kAbs) acca += (double)pr[s + smp] * (double)abs_to_float(g);
+            } else {
+                acc = madd(pr[smp], g, acc);
+            }
+        }
+    }
+    const int64_t at = ((int64_t)chunk << p.s_log2) + lane;
+    if (lane < s && at < p.S) {
+        static_cast<Out*>(p.R)[at] = acc;
+        if constexpr (Tr::kAbs) p.Rabs[at] = acca;
+    }
+}
+
+// State of a CTA between chunks.
+struct ChipState {
+    int pending;        // chunk whose sink has not been summed (-1: none); its tail level is in place
+    int written;        // chunk whose results are written but not counted in (warp 0)
+    unsigned word;      // this lane's sink word
+    bool counts;        // results are counted in block by block
+};
+
+// One chunk of samples: propagators (and the previous chunk's sink), then every level.
+// The chunk's times are in the times buffer; those of chunk `next` (< 0: none) follow.
+// `next_of` is called after a block barrier.
+template <int MODE, int LB, class Next>
+__device__ __forceinline__ void chip_chunk(const ChipParams& p, int chunk, unsigned char* sm, unsigned tmem, ChipState& cs,
+                                           const Next& next_of) {
+    using Tr = Traits<MODE>;
+    using Val = typename Tr::Val;
+    using RS = RowSum<MODE, LB>;
+    constexpr int V = RS::V;
+    constexpr bool kMixed = Tr::kBase == COS_MODE_FP32_MIXED;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int RB = 1 << p.rb_log2;
+    // the previous chunk's sink beside the exponentials
+    if (warp == 0 && cs.pending >= 0) {
+        chip_sink<MODE>(p, sm, p.tail_off, cs.pending, cs.word);
+        cs.written = cs.pending;
+    }
+    int cur = p.L == 2 ? p.tail_off : 0;   // where the current level is
+    if (tid * 4 < RB) reinterpret_cast<unsigned*>(sm + cur)[tid] = 0u;                        // the zero row
+    if (tid * (int)sizeof(Val) < RB) reinterpret_cast<Val*>(sm + cur + RB)[tid] = (Val)1;     // the root holds 1
+    if constexpr (Tr::kCount) {
+        __syncthreads();
+    } else if (p.ptab) {
+        __syncthreads();   // the previous sink has read its propagators
+        chip_slots_table<MODE>(p, sm);
+        __syncthreads();
+    } else {
+        for (int k0 = 0; k0 < p.K; k0 += p.kinds_per_pass) {
+            const int kn = min(p.kinds_per_pass, p.K - k0);
+            SlotRange range;
+            range.open(p, k0, kn, p.s_log2 - (V == 4 ? 2 : V == 2 ? 1 : 0));
+            bool far = chip_exps<MODE>(p, sm, k0, kn, false);
+            if (k0 == 0) chip_pairs(p, sm);
+            if constexpr (kMixed) {
+                far = __syncthreads_or(far);
+                if (far) {
+                    chip_exps<MODE>(p, sm, k0, kn, true);
+                    __syncthreads();
+                }
+            } else {
+                far = true;
+                __syncthreads();
+            }
+            chip_slots<MODE, V>(p, sm, k0, kn, far, range);
+            __syncthreads();   // the propagators are complete, the scratch is free
+        }
+    }
+    const int next = next_of();
+    if (next >= 0) chip_times<MODE>(p, sm, next);
+
+    const int lsh = p.rb_log2 - (LB == 16 ? 4 : LB == 8 ? 3 : 2);   // log2 lanes per row
+    const int lanes = 1 << lsh, piece = lane & (lanes - 1);
+    const int r32 = ((warp & (lanes - 1)) << (5 - lsh)) + (lane >> lsh);   // rows r32, r32 + 32 of a group
+    const int g0 = warp >> lsh, gstep = T >> (5 + lsh);
+    RS rs;
+    rs.rb = RB;
+    rs.gb = Tr::kAbs ? RB / 2 : RB;
+    rs.pro = p.g_off + (Tr::kAbs ? piece & (lanes / 2 - 1) : piece) * LB;
+    rs.use_abs = Tr::kAbs && piece >= lanes / 2;
+    const int mine = RB + r32 * RB + piece * LB;   // this lane's first piece in a level's rows
+    const int4* levt = reinterpret_cast<const int4*>(sm + p.tab_off);
+    const unsigned* grp = reinterpret_cast<const unsigned*>(levt + p.L);
+    const uint32_t* words = p.g.words;
+    int4 lv = make_int4(0, 0, 0, 0);   // width, groups, first group, place | staged
+    unsigned d = 0;                    // descriptor of this warp's next group, and this lane's words
+    Words m{};
+    auto open = [&](int l) {
+        lv = levt[l];
+        if (g0 >= lv.y) return;
+        d = __shfl_sync(0xffffffffu, grp[lv.z + g0], 0);
+        load_words(m, words + (d >> 11 << 6), d & 0x7ffu, r32);
+    };
+    if (p.L > 2) open(1);
+    if (cs.counts && tid == 0 && cs.written >= 0) chip_arrive(p, cs.written);
+    cs.written = -1;
+    for (int l = 1; l + 1 < p.L; ++l) {
+        const int W = lv.x, groups = lv.y, dst = lv.w & 0x7fffffff;
+        const bool staged = lv.w < 0;
+        const unsigned* gd = grp + lv.z;
+        rs.par = cur + piece * LB;
+        unsigned col = tmem;
+        for (int g = g0; g < groups; g += gstep) {
+            const unsigned dc = d;
+            const Words mc = m;
+            if (g + gstep < groups) {   // the next group's words, a round ahead
+                d = __shfl_sync(0xffffffffu, gd[g + gstep], 0);   // (uniform, known to be)
+                load_words(m, words + (d >> 11 << 6), d & 0x7ffu, r32);
+            }
+            rs.rows(sm, mc, dc & 0x7ffu, words + (dc >> 11 << 6), r32);
+            if (staged) {
+                Pair<LB> x;
+                memcpy(&x, &rs.acc, 2 * LB);
+                __syncwarp();
+                tmem_put<LB>(col, x);
+                col += LB / 2;
+            } else {
+                const int row = g * kChipGroup + r32, at = dst + g * (kChipGroup * RB) + mine;
+                if (row < W) *reinterpret_cast<typename RS::VecV*>(sm + at) = rs.acc[0];
+                if (row + 32 < W) *reinterpret_cast<typename RS::VecV*>(sm + (at + 32 * RB)) = rs.acc[1];
+            }
+        }
+        const int first = g0 * kChipGroup + r32, step = gstep * kChipGroup;
+        if (l + 2 < p.L) open(l + 1);   // ahead of the barriers
+        else cp_async_wait<0>();        // the next chunk's times
+        if (staged) {
+            tmem_wait_st();
+            __syncthreads();   // every row has read its parents
+            constexpr int U = 2;   // rounds per wait (a warp's 128 columns hold a multiple)
+            unsigned from = tmem;
+            const int warp_first = g0 * kChipGroup;
+            for (int row = first, wrow = warp_first; wrow < W; row += U * step, wrow += U * step) {
+                Pair<LB> x[U];
+                __syncwarp();
+#pragma unroll
+                for (int u = 0; u < U; ++u) tmem_get<LB>(from + (unsigned)u * (LB / 2), x[u]);
+                from += U * (LB / 2);
+#pragma unroll
+                for (int u = 0; u < U; ++u) tmem_wait_ld<LB>(x[u]);
+                const int at = dst + RB + row * RB + piece * LB;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    typename RS::VecV v[2];
+                    memcpy(&v, &x[u], 2 * LB);
+                    if (row + u * step < W) *reinterpret_cast<typename RS::VecV*>(sm + (at + u * step * RB)) = v[0];
+                    if (row + u * step + 32 < W) *reinterpret_cast<typename RS::VecV*>(sm + (at + (u * step + 32) * RB)) = v[1];
+                }
+            }
+        }
+        if (tid * 4 < RB) reinterpret_cast<unsigned*>(sm + dst)[tid] = 0u;   // its zero row
+        __syncthreads();
+        cur = dst;
+    }
+    if (p.L == 2) {
+        cp_async_wait<0>();
+        __syncthreads();
+    }
+    if (p.tail_off >= 0) {
+        cs.pending = chunk;   // its sink is summed beside the next chunk's exponentials
+    } else {
+        if (warp == 0) {
+            chip_sink<MODE>(p, sm, cur, chunk, cs.word);
+            cs.written = chunk;
+        }
+        __syncthreads();
+    }
+}
+
+// After the last chunk of a graph: its sink, and the results counted in.
+template <int MODE>
+__device__ __forceinline__ void chip_finish(const ChipParams& p, unsigned char* sm, ChipState& cs) {
+    if ((threadIdx.x >> 5) == 0) {
+        if (cs.counts && cs.written >= 0 && threadIdx.x == 0) chip_arrive(p, cs.written);
+        if (cs.pending >= 0) {
+            chip_sink<MODE>(p, sm, p.tail_off, cs.pending, cs.word);
+            __syncwarp();
+            if (cs.counts && threadIdx.x == 0) chip_arrive(p, cs.pending);
+        }
+    }
+    cs.pending = cs.written = -1;
+    __syncthreads();
+}
+
+template <int MODE, int LB>
+__global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ ChipArgs a) {
+    extern __shared__ __align__(128) unsigned char sm[];
+    __shared__ unsigned s_tmem;
+    __shared__ int s_next[2];
+    __shared__ int s_last;
+    __shared__ ChipParams s_p;
+    const int warp = threadIdx.x >> 5;
+    if (warp == 0) tmem_alloc(&s_tmem, (unsigned)a.tmem_cols);
+    if (a.list && threadIdx.x == 0) s_next[0] = (int)atomicAdd(a.ticket, 1u);
+    __syncthreads();
+    const unsigned base = s_tmem;
+    // a warp reaches the TMEM lanes of its number mod 4; the warps that share them take
+    // 128 columns each
+    const unsigned tmem = base + ((unsigned)(warp & 3) << 21) + (unsigned)(warp >> 2) * 128u;
+    const int lane = threadIdx.x & 31;
+    ChipState cs{-1, -1, 0u, !a.few};
+    if (!a.list) {
+        chip_setup<MODE>(a.one, sm);
+        cs.word = lane < a.one.g.nsink ? __ldg(a.one.g.sink + lane) : 0u;
+        chip_times<MODE>(a.one, sm, blockIdx.x);   // (the grid has no CTA without a chunk)
+        cp_async_wait<0>();
+        __syncthreads();
+        for (int c = blockIdx.x; c < a.one.nchunks; c += gridDim.x)
+            chip_chunk<MODE, LB>(a.one, c, sm, tmem, cs, [&] {
+                const int n = c + (int)gridDim.x;
+                return n < a.one.nchunks ? n : -1;
+            });
+        chip_finish<MODE>(a.one, sm, cs);
+        if (!a.few) chip_sum_own<MODE>(a.one, 0);
+    } else {
+        int g = -1;
+        for (int buf = 0;; buf ^= 1) {
+            const int c = s_next[buf];
+            if (c >= a.total) break;
+            if (threadIdx.x == 0) s_next[buf ^ 1] = (int)atomicAdd(a.ticket, 1u);   // read after a barrier
+            int h = max(g, 0);
+            while (h + 1 < a.n && a.list[h + 1].first_chunk <= c) ++h;
+            if (h != g) {
+                if (g >= 0) chip_finish<MODE>(s_p, sm, cs);
+                g = h;
+                static_assert(sizeof(ChipParams) % 4 == 0, "copied as words");
+                for (int q = threadIdx.x; q < (int)(sizeof(ChipParams) / 4); q += blockDim.x)
+                    reinterpret_cast<unsigned*>(&s_p)[q] = __ldg(reinterpret_cast<const unsigned*>(a.list + h) + q);
+                __syncthreads();
+                chip_setup<MODE>(s_p, sm);
+                cs.word = lane < s_p.g.nsink ? __ldg(s_p.g.sink + lane) : 0u;
+                chip_times<MODE>(s_p, sm, c - s_p.first_chunk);
+                cp_async_wait<0>();
+                __syncthreads();
+            }
+            chip_chunk<MODE, LB>(s_p, c - s_p.first_chunk, sm, tmem, cs, [&] {
+                const int n = s_next[buf ^ 1] - s_p.first_chunk;
+                return n < s_p.nchunks ? n : -1;
+            });
+        }
+        if (g >= 0) chip_finish<MODE>(s_p, sm, cs);
+        int first = 0;
+        for (int h = 0; h < a.n && !a.few; ++h) {
+            chip_sum_own<MODE>(a.list[h], first);
+            first += (int)((a.list[h].S + kReduceBlock - 1) / kReduceBlock);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(a.exits, 1u) + 1u == gridDim.x;
+        __threadfence();
+    }
+    __syncthreads();
+    if (s_last) {   // every other CTA has counted its chunks in and left
+        const int n = a.list ? a.n : 1;
+        for (int h = 0; h < n; ++h) {
+            const ChipParams& p = a.list ? a.list[h] : a.one;
+            if (a.few) chip_sum_few<MODE>(p, sm);
+            else chip_sum_rest<MODE>(p);
+        }
+        __syncthreads();
+        for (int h = warp; h < n; h += blockDim.x >> 5) chip_mean<MODE>(a.list ? a.list[h] : a.one, threadIdx.x & 31);
+        if (threadIdx.x == 0) *a.exits = 0;
+    }
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(base, (unsigned)a.tmem_cols);
+}
+
+template <int MODE, int LB>
+const void* ck() {
+    return reinterpret_cast<const void*>(&chip_kernel<MODE, LB>);
+}
+
+const void* select_chip(int kmode, int lb) {
+    switch (kmode * 32 + lb) {
+        case COS_MODE_FP64 * 32 + 16: return ck<COS_MODE_FP64, 16>();
+        case COS_MODE_FP64 * 32 + 8: return ck<COS_MODE_FP64, 8>();
+        case COS_MODE_FP32_MIXED * 32 + 16: return ck<COS_MODE_FP32_MIXED, 16>();
+        case COS_MODE_FP32_MIXED * 32 + 8: return ck<COS_MODE_FP32_MIXED, 8>();
+        case COS_MODE_FP32_MIXED * 32 + 4: return ck<COS_MODE_FP32_MIXED, 4>();
+        case COS_MODE_COUNT_I64 * 32 + 16: return ck<COS_MODE_COUNT_I64, 16>();
+        case COS_MODE_COUNT_I64 * 32 + 8: return ck<COS_MODE_COUNT_I64, 8>();
+        case kModeMixedAbs * 32 + 16: return ck<kModeMixedAbs, 16>();
+        case kModeMixedAbs * 32 + 8: return ck<kModeMixedAbs, 8>();
+        case kModeMixedAbs * 32 + 4: return ck<kModeMixedAbs, 4>();
+        default: return nullptr;
+    }
+}
+
+// Bytes of one sample in a node's row and in a slot's row.
+int node_bytes(int kmode) { return kmode == COS_MODE_FP32_MIXED ? 4 : 8; }
+int slot_bytes(int kmode) {
+    return kmode == COS_MODE_COUNT_I64 ? 0 : base_mode(kmode) == COS_MODE_FP32_MIXED ? 4 : 8;
+}
+
+// Shared memory of one CTA when `ctas` share an SM (1 KB of 228 KB reserved per CTA, and
+// the kernel's static shared memory).
+int smem_limit(int ctas) { return 228 * 1024 / ctas - 1024 - 512; }
+
+struct ChipLayout {
+    int lev_bytes, g_off, times_off, tab_off, coef_off, tail_off, total, kinds;
+};
+
+// Shared-memory layout of a CTA; total > limit when it does not fit.
+ChipLayout chip_layout(const ChipGraph& g, int kmode, int P, int K, int D, bool table, int rb, int limit) {
+    ChipLayout y;
+    const bool count = kmode == COS_MODE_COUNT_I64;
+    const int s = rb / node_bytes(kmode);
+    const int64_t gbytes = count ? 0 : round128((int64_t)(P + 1) * s * slot_bytes(kmode));
+    const int64_t times = count ? 0 : round128(8LL * D * s), tab = round128(16LL * g.tables);
+    const int64_t coef = count ? 0 : round128(chip_coef_bytes(K));
+    const int64_t tail = g.tail_width <= kTailRows ? round128((int64_t)(g.tail_width + 1) * rb) : 0;
+    const int64_t level = std::max<int64_t>(round128((int64_t)(g.max_width + 1) * rb), kScratchAt);
+    const int64_t rest = gbytes + times + tab + coef + tail;
+    int64_t lev = level;
+    y.kinds = K;
+    if (!count && !table) {
+        const int64_t fixed = kScratchAt + chip_pair_bytes(D), kind = 24LL * D * chip_pitch(s);
+        y.kinds = (int)std::max<int64_t>(1, std::min<int64_t>(K, (std::max<int64_t>(level, limit - rest) - fixed) / kind));
+        lev = std::max<int64_t>(level, round128(fixed + kind * y.kinds));
+    }
+    // room for a level and the next beside it, where there is some: no staging
+    lev = std::max<int64_t>(lev, std::min<int64_t>(2 * level, (limit - rest) / 128 * 128));
+    y.lev_bytes = (int)std::min<int64_t>(lev, 1 << 28);
+    y.g_off = y.lev_bytes;
+    y.times_off = y.g_off + (int)gbytes;
+    y.tab_off = y.times_off + (int)times;
+    y.coef_off = y.tab_off + (int)tab;
+    y.tail_off = tail ? y.coef_off + (int)coef : -1;
+    y.total = (int)(y.lev_bytes + rest);
+    return y;
+}
+
+}  // namespace
+
+int chip_phase_rows(int64_t max_width, int64_t P, int32_t K, int32_t D) {
+    ChipGraph g;
+    g.max_width = (int32_t)std::min<int64_t>(max_width, INT32_MAX - 1);
+    g.tail_width = kTailRows;
+    if (max_width > 65534 || P > 65534) return 0;
+    for (int rb = 128; rb >= 4; rb /= 2)
+        if (chip_layout(g, COS_MODE_FP32_MIXED, (int)P, K, D, false, rb, smem_limit(1)).total <= smem_limit(1)) return 128 / rb;
+    return 0;
+}
+
+// Model of the time of an evaluation in microseconds, within about 10 % of what 19 graphs
+// (1,000 to 117,000 nodes, 300 to 65,536 samples, every mode) took in every shape that
+// fits them.  Per chunk: the busiest of the shared-memory pipe (128 bytes per cycle, times
+// the passes per phase that the row order leaves), the issue slots and the FP64 pipe, then
+// the propagators, then what a chunk waits for by itself -- barriers, fetch and L2 latency,
+// mostly per level -- which CTAs that share an SM hide less than their number suggests
+// (medium graph, FP32: one CTA with 8 samples 1.66 ms, two with 4 samples 1.99 ms).
+double chip_time_us(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, int32_t D, bool table, int64_t S, int sms,
+                    int rb, int lane, int ctas) {
+    const int s = rb / node_bytes(kmode), mode = base_mode(kmode);
+    const double B = 128.0 / rb;
+    double conf = B <= 1 ? 1.0 : B <= 2 ? 1.15 : B <= 4 ? 1.45 : B <= 8 ? 1.9 : B <= 16 ? 2.2 : 2.4;
+    const double tables = mode == COS_MODE_COUNT_I64 ? 1.0 : kmode == kModeMixedAbs ? 1.5 : 2.0;
+    const double lds = (double)g.edges * rb / 128.0 * conf * tables + (double)g.rows * rb / 128.0 * 1.3;
+    const double issue = ((double)g.edges * 14 + (double)g.rows * 40) * rb / lane / 32.0 / 4.0;
+    const double f64 = mode == COS_MODE_FP64 ? (double)g.edges * s / 2.0 * 1.1 : 0.0;
+    double props = 0.0;
+    if (table) props = (double)P * s * 4.0;
+    else if (mode == COS_MODE_FP64) props = ((double)K * D * s * 17 + (double)P * s) / 2.0 * 1.1;
+    else if (mode == COS_MODE_FP32_MIXED) props = (double)K * D * s * 2.0 + (double)P * s * 0.25;
+    const double busy = std::max(lds, std::max(issue, f64)) + props, alone = 5000.0 + 900.0 * L;
+    const int64_t chunks = (S + s - 1) / s, slots = (int64_t)ctas * sms;
+    return (double)((chunks + slots - 1) / slots) * (ctas * busy + alone * (1.0 + 0.1 * (ctas - 1))) / 1930.0 + 12.0;
+}
+
+// The same for the general kernels: launch and barriers or task planning, edges at the
+// rate they reach on graphs of this kind, propagator slots (through L2, and back).
+double general_time_us(const ChipGraph& g, int kmode, int32_t L, int32_t P, int64_t S) {
+    const double es = (double)g.edges * (double)S, ps = (double)P * (double)S, fixed = 45.0 + 3.0 * L;
+    if (kmode == COS_MODE_COUNT_I64) return fixed + es / 9.5e5;
+    if (kmode == COS_MODE_FP64) return fixed + es / 5.4e5 + ps / 1.5e5;
+    return fixed + es / (kmode == kModeMixedAbs ? 8.5e5 : 1.65e6) + ps / 3e5;
+}
+
+// The shape with the least model time; on chip when that is below the general kernels'.
+// Measured on both sides of the line, general / on-chip: medium graph 2.35 / 1.66 ms
+// (FP32), 3.00 / 2.26 ms (with A), 3.2 / 2.2 ms (count), FP64 6.34 / 6.89 ms (both held
+// by the FP64 pipe; general); 117,000 nodes, levels of 11,500 (FP32, two samples per
+// chunk) 7.69 / 7.61 ms, levels of 19,500 5.44 / 5.80 ms (general), but 3,000 samples of
+// the latter 0.48 / 0.42 ms and 300 samples of levels of 30,000 102 / 63 us.
+bool chip_plan(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, int32_t D, bool table, int64_t S, int sms,
+               ChipPlan* out) {
+    if (g.max_width <= 0 || S <= 0 || sms <= 0 || kmode == kModeFp64Abs) return false;
+    const int nb = node_bytes(kmode);
+    bool found = false;
+    for (int rb = std::max(nb, 4); rb <= 128; rb *= 2) {
+        const int lane = std::min(kmode == kModeMixedAbs ? rb / 2 : rb, 16);   // (a piece is wholly R or wholly A)
+        for (int ctas = 1; ctas <= 4; ctas *= 2) {
+            const ChipLayout y = chip_layout(g, kmode, P, K, D, table, rb, smem_limit(ctas));
+            if (y.total > smem_limit(ctas) || 512 / ctas / 32 < rb / lane) continue;   // (a group needs rb / lane warps)
+            const double cost = chip_time_us(g, kmode, L, P, K, D, table, S, sms, rb, lane, ctas);
+            if (found && cost >= out->cost) continue;
+            found = true;
+            out->rb_log2 = 31 - __builtin_clz((unsigned)rb);
+            out->lane_bytes = lane;
+            out->threads = 512 / ctas;
+            out->ctas = ctas;
+            out->smem = y.total;
+            out->cost = cost;
+        }
+    }
+    return found && out->cost < 0.97 * general_time_us(g, kmode, L, P, S);
+}
+
+void chip_shape(int kmode, const ChipPlan& plan, ChipParams* p) {
+    const int rb = 1 << plan.rb_log2, s = rb / node_bytes(kmode);
+    const ChipLayout y = chip_layout(p->g, kmode, p->P, p->K, p->D, p->ptab != nullptr, rb, smem_limit(plan.ctas));
+    p->rb_log2 = plan.rb_log2;
+    p->s_log2 = 31 - __builtin_clz((unsigned)s);
+    p->kinds_per_pass = y.kinds;
+    p->lev_bytes = y.lev_bytes;
+    p->g_off = y.g_off;
+    p->times_off = y.times_off;
+    p->tab_off = y.tab_off;
+    p->coef_off = y.coef_off;
+    p->tail_off = y.tail_off;
+    p->d_magic = p->D > 1 ? (uint32_t)(((1ull << 32) + (uint64_t)p->D - 1) / (uint64_t)p->D) : 0;
+    p->nchunks = (int32_t)((p->S + s - 1) / s);
+}
+
+namespace {
+
+// Blocks of samples up to which the last CTA sums them all, two rounds of its teams.
+int few_blocks(int threads) { return 2 * (threads / 128); }
+
+int launch(int kmode, int lane_bytes, int threads, int smem, ChipArgs& a, int chunks, int sms, cudaStream_t st) {
+    const void* k = select_chip(kmode, lane_bytes);
+    if (!k) return set_error(COS_ERR_INVALID, "no on-chip kernel for mode %d, %d bytes per lane", kmode, lane_bytes);
+    // (always the same limit: calls of other threads may come between this one and the launch)
+    if (prepare_kernel_attrs(k, smem_limit(1)) != COS_OK) return set_error(COS_ERR_CUDA, "cannot set dynamic shared memory");
+    const int ctas = 512 / threads;
+    a.tmem_cols = 512 / ctas;
+    void* args[] = {&a};
+    const int grid = std::min(chunks, sms * ctas);
+    const cudaError_t e = cudaLaunchKernel(k, dim3((unsigned)grid), dim3((unsigned)threads), args, (size_t)smem, st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return set_error(COS_ERR_CUDA, "on-chip walk launch: %s", cudaGetErrorString(e));
+    }
+    return COS_OK;
+}
+
+}  // namespace
+
+int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, cudaStream_t st) {
+    ChipArgs a{};
+    a.one = p;
+    const int64_t blocks = (p.S + kReduceBlock - 1) / kReduceBlock;
+    a.exits = p.arrive + blocks;
+    a.few = blocks <= few_blocks(plan.threads);
+    const int smem = a.few ? std::max(plan.smem, kTeamBytes * (int)std::min<int64_t>(plan.threads / 128, blocks)) : plan.smem;
+    return launch(kmode, plan.lane_bytes, plan.threads, smem, a, p.nchunks, sms, st);
+}
+
+int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const ChipParams* list, int n, int total,
+                     unsigned* ticket, unsigned* exits, int sms, cudaStream_t st) {
+    ChipArgs a{};
+    a.exits = exits;
+    a.list = list;
+    a.n = n;
+    a.total = total;
+    a.ticket = ticket;
+    return launch(kmode, lane_bytes, threads, smem, a, total, sms, st);
+}
+
+}  // namespace cosgpu

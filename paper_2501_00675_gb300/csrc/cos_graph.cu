@@ -11,6 +11,8 @@
 #include <string>
 #include <vector>
 
+#include "cos_chip.cuh"
+#include "cos_chip.h"
 #include "cos_internal.cuh"
 
 using namespace cosgpu;
@@ -90,6 +92,7 @@ struct SharedArrays {
     int32_t* slot_kij = nullptr;
     int32_t* kind_slot = nullptr;
     double* exp_tab = nullptr;
+    char* chip = nullptr;            // row schedule of the on-chip walk (the arrays of ChipGraph), when the graph has one
     ~SharedArrays() {
         DeviceGuard dg(device);
         dfree(levels);
@@ -98,6 +101,7 @@ struct SharedArrays {
         dfree(slot_kij);
         dfree(kind_slot);
         dfree(exp_tab);
+        dfree(chip);
     }
 };
 
@@ -133,6 +137,8 @@ struct cos_graph {
     size_t arena_bytes = 0;
     double* d_partials = nullptr;
     int64_t partial_cap = 0;
+    unsigned* d_arrive = nullptr;   // on-chip walk: arrival counters [partial_cap + 1] behind the partials, zero between launches
+    ChipGraph chip;                 // on-chip walk: row schedule (max_width 0: none)
     void* d_R = nullptr;            // internal per-sample output when the caller passes none
     int64_t R_cap = 0;
     cos_tuning tuning{};
@@ -201,6 +207,68 @@ bool carve(cos_graph* g, int kmode, int64_t tile, WalkParams& p) {
     p.gtab = (mode != COS_MODE_COUNT_I64) ? (void*)(base + gt) : nullptr;
     p.coef = (double*)(base + cf);
     return true;
+}
+
+// Row schedule of the on-chip walk for a graph whose levels fit shared memory (none
+// otherwise: the graph is evaluated by the general kernels alone).
+cudaError_t upload_chip(cos_graph* g, const std::vector<int32_t>& row_ptr, const std::vector<int2>& csr,
+                        const std::vector<int32_t>& slot_kij, SharedArrays& a) {
+    int64_t wmax = 1;
+    for (int32_t l = 0; l + 1 < g->L; ++l) wmax = std::max(wmax, g->widths[(size_t)l]);
+    if ((int64_t)g->K * g->D > 65535 || g->K > 32767 || g->D > kChipMaxTimes) return cudaSuccess;   // 16-bit slot factors
+    const int phase = chip_phase_rows(wmax, g->P, g->K, g->D);
+    if (phase == 0) return cudaSuccess;
+    ChipSchedule cs;
+    if (!build_chip(g->L, g->off.data(), row_ptr.data(), g->P, phase, [&](int32_t q) { return csr[(size_t)q].x; },
+                    [&](int32_t q) { return csr[(size_t)q].y; }, cs))
+        return cudaSuccess;
+    // one allocation: levels and group descriptors, edge words, slots, sink
+    static_assert(sizeof(ChipLevel) == sizeof(int4), "read as int4");
+    const size_t units = cs.lev.size() + (cs.grp.size() + 3) / 4;
+    const size_t words_at = units * sizeof(int4), slots_at = words_at + (cs.words.size() * 4 + 15) / 16 * 16,
+                 sink_at = slots_at + (size_t)g->P * sizeof(uint2), bytes = sink_at + cs.sink.size() * 4;
+    std::vector<char> h(bytes + 16);
+    memcpy(h.data(), cs.lev.data(), cs.lev.size() * sizeof(int4));
+    if (!cs.grp.empty()) memcpy(h.data() + cs.lev.size() * sizeof(int4), cs.grp.data(), cs.grp.size() * 4);
+    if (!cs.words.empty()) memcpy(h.data() + words_at, cs.words.data(), cs.words.size() * 4);
+    if (!cs.sink.empty()) memcpy(h.data() + sink_at, cs.sink.data(), cs.sink.size() * 4);
+    uint2* slots = reinterpret_cast<uint2*>(h.data() + slots_at);
+    for (int64_t q = 0; q < g->P; ++q) {
+        const uint32_t k = (uint32_t)slot_kij[(size_t)(3 * q)], i = (uint32_t)slot_kij[(size_t)(3 * q + 1)],
+                       jw = (uint32_t)slot_kij[(size_t)(3 * q + 2)], j = jw & (uint32_t)kKindMask, D = (uint32_t)g->D;
+        slots[q] = make_uint2((k * D + i) | (k * D + j) << 16, (i * D + j) | k << 16 | ((jw & (uint32_t)kSignBit) << 1));
+    }
+    cudaError_t e = cudaMalloc(&a.chip, h.size());
+    if (e == cudaErrorMemoryAllocation) {   // the general kernels need none of this
+        cudaGetLastError();
+        a.chip = nullptr;
+        return cudaSuccess;
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(a.chip, h.data(), h.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+    ChipGraph& c = g->chip;
+    c.lev = reinterpret_cast<const int4*>(a.chip);
+    c.words = reinterpret_cast<const uint32_t*>(a.chip + words_at);
+    c.slots = reinterpret_cast<const uint2*>(a.chip + slots_at);
+    c.sink = reinterpret_cast<const uint32_t*>(a.chip + sink_at);
+    c.nsink = (int32_t)cs.sink.size();
+    c.max_width = cs.max_width;
+    c.tail_width = (int32_t)g->widths[(size_t)g->L - 2];
+    c.tables = (int32_t)units;
+    c.phase_rows = cs.phase_rows;
+    c.edges = g->E;
+    c.rows = g->N;
+    return cudaSuccess;
+}
+
+// The on-chip walk serves evaluations whose launch shape is left to the library; a
+// field that names a shape of the general kernels, a phase trace or a test hook of
+// their waits selects those.
+bool chip_allowed(const cos_graph* g) {
+    const cos_tuning& t = g->tuning;
+    return g->chip.max_width > 0 && t.samples_per_lane <= 0 && t.rows_per_warp <= 0 && t.blocks_per_sm <= 0 && t.layout <= 0 &&
+           t.schedule <= 0 && t.window_chunks <= 0 && t.prefetch <= 0 && !g->d_trace &&
+           !getenv("COS_TEST_SKIP_BARRIER_PHASE") && !getenv("COS_TEST_STALL_TASK");
 }
 
 }  // namespace
@@ -408,6 +476,7 @@ int cos_create_graph(int32_t num_levels, const int64_t* level_width, const int64
     if ((e = cudaMemset(g->d_ctrl, 0, sizeof(Ctrl))) != cudaSuccess) return cleanup_fail(e, "memset ctrl");
     auto arr = std::make_shared<SharedArrays>();
     arr->device = g->device;
+    if ((e = upload_chip(g, row_ptr, csr, slot_kij, *arr)) != cudaSuccess) return cleanup_fail(e, "on-chip row schedule");
     arr->levels = g->d_levels;
     arr->row_ptr = g->d_row_ptr;
     arr->edges = g->d_edges;
@@ -438,6 +507,7 @@ int cos_graph_share(cos_graph_t src, cos_graph_t* out) {
     g->d_kind_slot = src->d_kind_slot;
     g->d_exp_tab = src->d_exp_tab;
     g->arrays = src->arrays;
+    g->chip = src->chip;
     g->tuning = src->tuning;
     DeviceGuard dg(g->device);
     cudaError_t e = cudaMalloc(&g->d_ctrl, sizeof(Ctrl));
@@ -497,6 +567,17 @@ int cos_graph_info(cos_graph_t g, int64_t* info, int32_t n) {
     const int64_t v[10] = {g->L, g->N, g->E, g->P, g->Wmax, g->count_wrapped, g->count_overflow ? 1 : 0,
                            g->K, g->D, g->device};
     for (int32_t q = 0; q < n && q < 10; ++q) info[q] = v[q];
+    if (n > 10) {   // kernel modes whose automatic evaluation runs on chip, one bit each
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
+        info[10] = 0;
+        for (int km = 0; km <= kModeMixedAbs; ++km) {
+            ChipPlan plan;
+            if (chip_allowed(g) && chip_plan(g->chip, km, g->L, (int32_t)g->P, g->K, g->D, g->d_ptab != nullptr,
+                                             std::max<int64_t>(g->S, 1), sms, &plan))
+                info[10] |= 1LL << km;
+        }
+    }
     return COS_OK;
 }
 
@@ -620,14 +701,18 @@ int cos_autotune(cos_graph_t g, int32_t mode, void* per_sample_out, void* stream
     int rc = COS_OK;
     for (int sc : scheds)
         for (int r : rpws)
-            for (int vi = 0; vi < 2 && rc == COS_OK; ++vi) {
+            for (int vi = -1; vi < 2 && rc == COS_OK; ++vi) {
                 cos_tuning t = base;
-                if (base.schedule <= 0) t.schedule = sc;
-                else if (sc != scheds[0]) continue;
-                if (base.rows_per_warp <= 0) t.rows_per_warp = r;
-                else if (r != rpws[0]) continue;
-                if (base.samples_per_lane <= 0) t.samples_per_lane = vecs[vi];
-                else if (vi > 0) continue;
+                if (vi < 0) {   // the base tuning itself, where it selects the on-chip walk
+                    if (sc != scheds[0] || r != rpws[0] || !chip_allowed(g)) continue;
+                } else {
+                    if (base.schedule <= 0) t.schedule = sc;
+                    else if (sc != scheds[0]) continue;
+                    if (base.rows_per_warp <= 0) t.rows_per_warp = r;
+                    else if (r != rpws[0]) continue;
+                    if (base.samples_per_lane <= 0) t.samples_per_lane = vecs[vi];
+                    else if (vi > 0) continue;
+                }
                 g->tuning = t;
                 float ms_best = 1e30f;
                 for (int rep = 0; rep < 3 && rc == COS_OK; ++rep) {   // the first run warms up
@@ -641,6 +726,7 @@ int cos_autotune(cos_graph_t g, int32_t mode, void* per_sample_out, void* stream
                     cudaEventElapsedTime(&ms, e0, e1);
                     if (rep > 0) ms_best = std::min(ms_best, ms);
                 }
+                g->tuning = base;
                 if (rc == COS_OK && ms_best < best_ms) {
                     best_ms = ms_best;
                     best = t;
@@ -688,8 +774,12 @@ int cos_set_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t
     if (nblk > g->partial_cap) {
         dfree(g->d_partials);
         const int64_t cap = std::max<int64_t>(nblk, 4096);   // room for 4M samples without regrowth
-        // two arrays: partial sums of R, then of A (when the walk also sums |path| values)
-        COS_CUDA(cudaMalloc(&g->d_partials, 2 * sizeof(double) * cap), "cudaMalloc partials");
+        // two arrays: partial sums of R, then of A (when the walk also sums |path| values),
+        // and the arrival counters of the on-chip walk
+        g->partial_cap = 0;
+        COS_CUDA(cudaMalloc(&g->d_partials, 2 * sizeof(double) * cap + sizeof(unsigned) * (cap + 1)), "cudaMalloc partials");
+        g->d_arrive = reinterpret_cast<unsigned*>(g->d_partials + 2 * cap);
+        COS_CUDA(cudaMemsetAsync(g->d_arrive, 0, sizeof(unsigned) * (cap + 1), st), "clear arrival counters");
         g->partial_cap = cap;
     }
     // Workspace arena: enough for the FP64 mode over all samples, up to the budget.
@@ -819,6 +909,21 @@ int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean
     if (km < 0) return fail(COS_ERR_INVALID, "bad mode %d", mode);
     if (mode_has_abs(km) && g->abs_next)
         return fail(COS_ERR_INVALID, "COS_EVAL_ABS and cos_evaluate_abs do not combine");
+    {
+        ChipParams cp;
+        ChipPlan plan;
+        int sms = 0;
+        int on_chip = 0;
+        int rc = prepare_chip(g, km, per_sample_out, &cp, &plan, &sms, &on_chip);
+        if (rc == COS_OK && on_chip) rc = launch_chip(km, plan, cp, sms, st);
+        if (rc != COS_OK) return rc;
+        if (on_chip) {
+            g->last_wave = 0;
+            g->last_mode = km;
+            g->last_status_pending = 1;
+            return mean_out ? collect(g, mean_out, st) : COS_OK;
+        }
+    }
     WalkParams p;
     cos_tuning tn;
     int rc = cosgpu::prepare_walk(g, km, nullptr, per_sample_out, &p, &tn);
@@ -987,6 +1092,60 @@ int graph_view(cos_graph_t g, GraphView* out) {
     return COS_OK;
 }
 
+// The internal per-sample buffer holds nout values (allocated on first need).
+static int ensure_result_buffer(cos_graph_t g, int64_t nout) {
+    if (nout <= g->R_cap) return COS_OK;
+    if (g->d_R) cudaFree(g->d_R);
+    g->d_R = nullptr;
+    g->R_cap = 0;
+    COS_CUDA(cudaMalloc(&g->d_R, sizeof(double) * nout), "cudaMalloc R");
+    g->R_cap = nout;
+    g->generation++;
+    return COS_OK;
+}
+
+void chip_view(cos_graph_t g, ChipGraph* out) { *out = g->chip; }
+
+int prepare_chip(cos_graph_t g, int kmode, void* per_sample_out, ChipParams* out, ChipPlan* plan, int* sms, int* on_chip) {
+    *on_chip = 0;
+    if (!g->has_samples || !chip_allowed(g)) return COS_OK;   // (the general path reports missing samples)
+    if (cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess) return COS_OK;
+    if (!chip_plan(g->chip, kmode, g->L, (int32_t)g->P, g->K, g->D, g->d_ptab != nullptr, g->S, *sms, plan)) return COS_OK;
+    const bool abs2 = mode_has_abs(kmode);
+    if (!per_sample_out) {
+        const int rc = ensure_result_buffer(g, std::max<int64_t>(g->S, 1) * (abs2 ? 2 : 1));
+        if (rc != COS_OK) return rc;
+    }
+    ChipParams& p = *out;
+    memset(&p, 0, sizeof(p));
+    p.g = g->chip;
+    p.kind_slot = g->d_kind_slot;
+    p.exp_tab = g->d_exp_tab;
+    p.t = g->t_borrowed ? g->t_borrowed : g->d_t;
+    p.eps = g->d_eps;
+    p.ptab = g->d_ptab;
+    p.R = per_sample_out ? per_sample_out : g->d_R;
+    p.Rabs = abs2 ? static_cast<double*>(p.R) + g->S : nullptr;
+    p.partials = g->d_partials;
+    p.partials_abs = abs2 ? g->d_partials + g->partial_cap : nullptr;
+    p.ctrl = g->d_ctrl;
+    p.arrive = g->d_arrive;
+    p.beta = g->beta;
+    p.ptab_inv_h = g->d_ptab ? (double)g->ptab_T / g->ptab_tau_max : 0.0;
+    p.S = g->S;
+    p.t_ld = g->t_ld;
+    p.L = g->L;
+    p.P = (int32_t)g->P;
+    p.K = g->K;
+    p.D = g->D;
+    p.ptab_T = g->ptab_T;
+    p.abs_weights = g->abs_next;
+    p.clear_err = 1;
+    chip_shape(kmode, *plan, &p);
+    *on_chip = 1;
+    return COS_OK;
+}
+
 int prepare_walk(cos_graph_t g, int mode, const cos_tuning* force, void* per_sample_out, WalkParams* out,
                  cos_tuning* tn_out) {
     if (!g) return fail(COS_ERR_INVALID, "graph is NULL");
@@ -1045,14 +1204,9 @@ int prepare_walk(cos_graph_t g, int mode, const cos_tuning* force, void* per_sam
     p.S = g->S;
     p.t_ld = g->t_ld;
     const int64_t nout = std::max<int64_t>(g->S, 1) * (abs2 ? 2 : 1);   // R, then A
-    if (!per_sample_out && nout > g->R_cap) {
-        // no caller buffer: the per-sample values go to an internal buffer (allocated on first need)
-        if (g->d_R) cudaFree(g->d_R);
-        g->d_R = nullptr;
-        g->R_cap = 0;
-        COS_CUDA(cudaMalloc(&g->d_R, sizeof(double) * nout), "cudaMalloc R");
-        g->R_cap = nout;
-        g->generation++;
+    if (!per_sample_out) {   // no caller buffer: the per-sample values go to an internal buffer
+        const int rcb = ensure_result_buffer(g, nout);
+        if (rcb != COS_OK) return rcb;
     }
     p.R = per_sample_out ? per_sample_out : g->d_R;
     p.partials = g->d_partials;

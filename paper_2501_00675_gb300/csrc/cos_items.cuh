@@ -393,7 +393,7 @@ __device__ __forceinline__ void item_coef(const WalkParams& p) {
 // e^{+-x} = 2^{+-m} 2^{+-j/64} e^{+-r}; e^{+-r} = 1 + E +- O with the even and odd parts
 // of the Taylor series through r^5 (truncation below 4e-17 relative).  The 64 values
 // 2^{j/64} (and 2^{-j/64}) are read from `tab` ([0..63] = 2^{j/64}, [64..127] = 2^{-j/64}).
-__device__ __forceinline__ void exp_pair(double x, const double* __restrict__ tab, double& em, double& ep) {
+__device__ __forceinline__ void exp_pair_from(double x, const double* tab, bool ldg, double& em, double& ep) {
     const double inv = 92.33248261689366;                  // 64 / ln 2 (only rounds n)
     const double c_hi = 0.01083042469326756;               // ln2/64 to 32 significant bits: n*c_hi is exact
     const double c_lo = 2.9815858269852933e-12;            // ln2/64 - c_hi
@@ -407,11 +407,18 @@ __device__ __forceinline__ void exp_pair(double x, const double* __restrict__ ta
     const int j = n & 63;
     const int m = n >> 6;                                                       // floor(n / 64)
     // e^{+x} = 2^m 2^{j/64} (1 + even + odd);  e^{-x} = 2^{-m} 2^{-j/64} (1 + even - odd)
-    const double tp = __ldg(tab + j), tm = __ldg(tab + 64 + j);
+    const double tp = ldg ? __ldg(tab + j) : tab[j], tm = ldg ? __ldg(tab + 64 + j) : tab[64 + j];
     const double vp = fma(tp, even + odd, tp);
     const double vm = fma(tm, even - odd, tm);
     ep = __hiloint2double(__double2hiint(vp) + (m << 20), __double2loint(vp));
     em = __hiloint2double(__double2hiint(vm) - (m << 20), __double2loint(vm));
+}
+__device__ __forceinline__ void exp_pair(double x, const double* __restrict__ tab, double& em, double& ep) {
+    exp_pair_from(x, tab, true, em, ep);
+}
+// The table in shared memory.
+__device__ __forceinline__ void exp_pair_at(double x, const double* tab, double& em, double& ep) {
+    exp_pair_from(x, tab, false, em, ep);
 }
 
 // ---------------------------------------------------------------- float-float helpers
@@ -482,7 +489,7 @@ __device__ __forceinline__ float2 ldexp_ff(float2 v, int m) {
 // `tff` ([0..63] = 2^{j/64}, [64..127] = 2^{-j/64}, each as (hi, lo)).
 __device__ __forceinline__ void exp_pair_ff(double x, const float2* __restrict__ tff, float2& em, float2& ep) {
     const float nf = rintf(trunc_to_float(x) * 92.33248261689366f);
-    const double nd = (double)(int)nf;
+    const double nd = float_to_double_exact(nf);   // (an integer: no conversion on the FP64 pipe)
     double r = fma(-nd, 0.01083042469326756, x);
     r = fma(-nd, 2.9815858269852933e-12, r);
     const int n = (int)nf;

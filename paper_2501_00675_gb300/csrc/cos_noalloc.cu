@@ -26,6 +26,7 @@
 #include <cstdint>
 #include <cuda.h>
 
+#include "cos_chip.cuh"
 #include "cos_internal.cuh"
 
 namespace cosgpu {
@@ -33,11 +34,17 @@ namespace {
 
 static __device__ __align__(256) unsigned char g_static_scratch[COS_STATIC_SCRATCH_BYTES];
 
+// Arrival counters of the on-chip walk, zero between launches (its other working memory
+// is on chip; the partial sums and the control block are in the scratch array).
+constexpr int kStaticBlocks = 4096;
+static __device__ unsigned g_static_arrive[kStaticBlocks + 1];
+
 constexpr int kMaxDevices = 64;
 std::mutex g_addr_mutex;
 struct ScratchAddr {
     void* ctx;    // the context the address belongs to
     void* ptr;    // device address of g_static_scratch in that context
+    void* arrive; // ... and of g_static_arrive
 };
 ScratchAddr g_scratch_addr[kMaxDevices] = {};
 
@@ -64,7 +71,7 @@ void* current_context() {
 // is kept together with the context it was taken in and looked up again when the
 // device's context differs (after cudaDeviceReset, a new primary context may load
 // the module elsewhere).
-int scratch_address(int device, void** out) {
+int scratch_address(int device, void** out, void** arrive) {
     if (device < 0 || device >= kMaxDevices) return set_error(COS_ERR_INVALID, "device ordinal %d not supported", device);
     void* ctx = current_context();
     std::lock_guard<std::mutex> lock(g_addr_mutex);
@@ -72,6 +79,7 @@ int scratch_address(int device, void** out) {
     if (!a.ptr || !ctx || a.ctx != ctx) {
         void* ptr = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&ptr, g_static_scratch);
+        if (e == cudaSuccess) e = cudaGetSymbolAddress(&a.arrive, g_static_arrive);
         if (e != cudaSuccess || !ptr) {
             a.ptr = nullptr;
             return set_error(COS_ERR_CUDA, "cudaGetSymbolAddress(static scratch) failed: %s", cudaGetErrorString(e));
@@ -80,10 +88,36 @@ int scratch_address(int device, void** out) {
         a.ctx = ctx;
     }
     *out = a.ptr;
+    *arrive = a.arrive;
     return COS_OK;
 }
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+
+// Wait for the stream, report (and clear) a recorded failure, else store the mean.
+int static_result(const GraphView& gv, int mode, Ctrl* ctrl, double* mean_out, cudaStream_t st) {
+    char* cb = reinterpret_cast<char*>(ctrl);
+    Ctrl c;
+    cudaError_t e = cudaMemcpyAsync(&c, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return set_error(COS_ERR_CUDA, "read result: %s", cudaGetErrorString(e));
+    if (c.err != 0) {
+        // report once: clear the recorded failure so that the next call starts clean
+        e = cudaMemsetAsync(cb + offsetof(Ctrl, err), 0, 2 * sizeof(int), st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return set_error(COS_ERR_CUDA, "clear error word: %s", cudaGetErrorString(e));
+        if (c.err == KERR_BARRIER_TIMEOUT)
+            return set_error(COS_ERR_TIMEOUT,
+                             "a grid barrier timed out (phase %d) in this call or in a call since the last one that "
+                             "passed mean_out; the results of those calls are invalid",
+                             c.err_detail);
+        return set_error(COS_ERR_CUDA, "kernel reported error %d", c.err);
+    }
+    *mean_out = c.mean;
+    if (mode == COS_MODE_COUNT_I64 && gv.count_overflow)
+        return set_error(COS_ERR_OVERFLOW, "path count exceeds 2^63-1; results wrap modulo 2^64");
+    return COS_OK;
+}
 
 }  // namespace
 }  // namespace cosgpu
@@ -109,8 +143,8 @@ extern "C" int cos_evaluate_static(cos_graph_t g, int32_t mode, int64_t num_samp
     int cur = -1;
     if (cudaGetDevice(&cur) != cudaSuccess || cur != gv.device)
         return set_error(COS_ERR_INVALID, "the graph's device (%d) must be current", gv.device);
-    void* base = nullptr;
-    rc = scratch_address(gv.device, &base);
+    void *base = nullptr, *arrive = nullptr;
+    rc = scratch_address(gv.device, &base, &arrive);
     if (rc != COS_OK) return rc;
 
     // Carve the static array: control block, partial sums, coefficients, then one tile's working set.
@@ -180,11 +214,45 @@ extern "C" int cos_evaluate_static(cos_graph_t g, int32_t mode, int64_t num_samp
     if (const char* env = getenv("COS_TEST_SKIP_BARRIER_PHASE")) p.skip_barrier_phase = atoi(env);
 
     int per_sm = 0, sms = 0;
-    const int dev_max = max_coresident_blocks(mode, vec, 1, gv.D, gv.device);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, gv.device);
+    cudaStream_t st = (cudaStream_t)stream;
+    // Graphs that fit on chip: one launch that waits for nothing and leaves the error
+    // word alone (the general kernel's test hook keeps the general kernel).
+    ChipGraph cg;
+    ChipPlan plan;
+    chip_view(g, &cg);
+    const bool on_chip = S > 0 && nblk <= kStaticBlocks && !p.skip_barrier_phase &&
+                         chip_plan(cg, mode, gv.L, gv.P, gv.K, gv.D, gv.ptab != nullptr, S, sms, &plan);
+    if (on_chip) {
+        ChipParams q;
+        memset(&q, 0, sizeof(q));
+        q.g = cg;
+        q.kind_slot = gv.kind_slot;
+        q.exp_tab = gv.exp_tab;
+        q.t = t;
+        q.eps = eps;
+        q.ptab = gv.ptab;
+        q.R = per_sample_out;
+        q.partials = reinterpret_cast<double*>(b + part_at);
+        q.ctrl = p.ctrl;
+        q.arrive = static_cast<unsigned*>(arrive);
+        q.beta = beta;
+        q.ptab_inv_h = p.ptab_inv_h;
+        q.S = S;
+        q.t_ld = t_ld;
+        q.L = gv.L;
+        q.P = gv.P;
+        q.K = gv.K;
+        q.D = gv.D;
+        q.ptab_T = gv.ptab_T;
+        chip_shape(mode, plan, &q);
+        rc = launch_chip(mode, plan, q, sms, st);
+        if (rc != COS_OK) return rc;
+        return mean_out ? static_result(gv, mode, p.ctrl, mean_out, st) : COS_OK;
+    }
+    const int dev_max = max_coresident_blocks(mode, vec, 1, gv.D, gv.device);
     if (dev_max <= 0 || sms <= 0) return set_error(COS_ERR_CUDA, "cannot query occupancy");
     per_sm = dev_max / sms;
-    cudaStream_t st = (cudaStream_t)stream;
     // The barrier counter and the result fields start at zero on every call.  The error
     // word and its detail are not cleared here: a failure of a call made without
     // mean_out stays recorded until a call with mean_out reports (and clears) it.
@@ -197,25 +265,5 @@ extern "C" int cos_evaluate_static(cos_graph_t g, int32_t mode, int64_t num_samp
     char msg[256] = {0};
     rc = launch_walk(mode, vec, 1, p, sms * per_sm, st, msg, sizeof(msg));
     if (rc != COS_OK) return set_error(rc, "walker launch failed: %s", msg);
-    if (!mean_out) return COS_OK;
-    Ctrl c;
-    e = cudaMemcpyAsync(&c, p.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return set_error(COS_ERR_CUDA, "read result: %s", cudaGetErrorString(e));
-    if (c.err != 0) {
-        // report once: clear the recorded failure so that the next call starts clean
-        e = cudaMemsetAsync(cb + offsetof(Ctrl, err), 0, 2 * sizeof(int), st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return set_error(COS_ERR_CUDA, "clear error word: %s", cudaGetErrorString(e));
-        if (c.err == KERR_BARRIER_TIMEOUT)
-            return set_error(COS_ERR_TIMEOUT,
-                             "a grid barrier timed out (phase %d) in this call or in a call since the last one that "
-                             "passed mean_out; the results of those calls are invalid",
-                             c.err_detail);
-        return set_error(COS_ERR_CUDA, "kernel reported error %d", c.err);
-    }
-    *mean_out = c.mean;
-    if (mode == COS_MODE_COUNT_I64 && gv.count_overflow)
-        return set_error(COS_ERR_OVERFLOW, "path count exceeds 2^63-1; results wrap modulo 2^64");
-    return COS_OK;
+    return mean_out ? static_result(gv, mode, p.ctrl, mean_out, st) : COS_OK;
 }
