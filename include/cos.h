@@ -59,7 +59,7 @@ enum cos_status {
 enum cos_mode {
     COS_MODE_FP64 = 0,        /* propagators, products and sums in IEEE double */
     COS_MODE_FP32_MIXED = 1,  /* propagators (formed in double, rounded once) and per-level products
-                                 in float; sink node and cross-sample sums in double, compensated */
+                                 in float; sink node and cross-sample sums exact or compensated */
     COS_MODE_COUNT_I64 = 2,   /* unit edge weights, int64 sums modulo 2^64: the number of paths */
     COS_EVAL_ABS = 16         /* flag, with modes 0 and 1: the same walk also accumulates
                                  A(s) = sum over paths of |path value| (every factor replaced by
@@ -171,8 +171,9 @@ int cos_copy_times(cos_graph_t g, double* dst, void* stream);
  *                   int64[S] (COUNT_I64), index = sample index; with COS_EVAL_ABS
  *                   double[2*S]: R(s) at s, A(s) at S + s
  *   mean_out        host pointer or NULL.  If non-NULL the call waits for the
- *                   stream and stores the mean over samples (Neumaier-compensated
- *                   double; in count mode the mean of the counts), and reports
+ *                   stream and stores the mean over samples (summed in 128-bit
+ *                   integers or, beyond their range, with Neumaier compensation,
+ *                   and rounded to double; in count mode the mean of the counts), and reports
  *                   kernel-side errors; with COS_EVAL_ABS mean_out[0] = mean R and
  *                   mean_out[1] = mean A (two doubles).  If NULL the call returns
  *                   at once; use cos_get_result to wait and collect.

@@ -17,7 +17,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libcosgpu.so")
 SOURCES = ["cos_graph.cu", "cos_walk.cu", "cos_batch.cu", "cos_noalloc.cu", "cos_mc.cu", "cos_serve.cu", "cos_chip.cu"]
-HEADERS = ["cos_internal.cuh", "cos_items.cuh", "cos_tasks.cuh", "cos_feed.h", "cos_chip.h", "cos_chip.cuh"]
+HEADERS = ["cos_internal.cuh", "cos_items.cuh", "cos_tasks.cuh", "cos_feed.h", "cos_chip.h", "cos_fixed.h", "cos_chip.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -28,9 +28,11 @@
 //
 // CTAs never wait for one another: a CTA that has no chunk left sums its share of the
 // blocks of kReduceBlock samples that are complete, the last CTA the others, and it forms
-// the mean, in the fixed order of the general kernels (summing a block as soon as it is
-// complete put every sum, 8 us of dependent FP64 additions, on the one CTA that was
-// already last: 130 us per 16 blocks).
+// the mean.  A block is summed by the whole CTA in 128-bit integers (cos_fixed.h): 2,800
+// cycles from the first load to the partial sum, most of them latency, against 15,800 for
+// one warp's compensated additions, which the end of every launch waits for.  Tiny graph,
+// 1,000 samples, mixed, one launch: 20.5 -> 14.4 us; order 2, 1,000 nodes, 10,007 samples:
+// 96 -> 84 us.
 #include <algorithm>
 #include <cstdio>
 #include <type_traits>
@@ -514,120 +516,125 @@ struct RowSum {
 
 // ---------------------------------------------------------------- sample reduction
 
-__device__ __forceinline__ double ld_cg_f64(const double* p) { return __ldcg(p); }
-__device__ __forceinline__ double ld_cg_f64(const long long* p) { return (double)__ldcg(p); }
-
-// One compensated addition as neumaier_add, without branches: the error of sum + y from
-// the larger operand (chosen by 32-bit comparison) is the same number.
-__device__ __forceinline__ bool bigger(double sum, double y) {   // |sum| >= |y|
-    const unsigned sh = (unsigned)__double2hiint(sum) & 0x7fffffffu, yh = (unsigned)__double2hiint(y) & 0x7fffffffu;
-    return sh > yh || (sh == yh && (unsigned)__double2loint(sum) >= (unsigned)__double2loint(y));
-}
-__device__ __forceinline__ void compensated_add(double& sum, double& comp, double y) {
-    const double u = sum + y;
-    const bool ge = bigger(sum, y);
-    comp += ((ge ? sum : y) - u) + (ge ? y : sum);
-    sum = u;
-}
-
-// As block_sum and partials_sum of the general kernels (same order, same result), with
-// L2 loads: the values come from other CTAs of this launch.  All loads are issued first
-// and the additions have no branches, so that the running sum is the only serial chain.
+// For values outside the integers' range.
 template <typename T>
-__device__ __forceinline__ double chip_block_sum(const T* x, int64_t S, int64_t b, int lane) {
+__device__ __noinline__ double block_sum_compensated(const T* x, int64_t S, int64_t b, int lane) {
     constexpr int per_lane = kReduceBlock / 32;
+    constexpr int AHEAD = 8;
     const int64_t s0 = b * kReduceBlock + lane;
-    double v[per_lane];
-#pragma unroll
-    for (int u = 0; u < per_lane; ++u) v[u] = s0 + u * 32 < S ? ld_cg_f64(x + s0 + u * 32) : 0.0;
     double sum = 0.0, comp = 0.0;
+#pragma unroll 1
+    for (int u0 = 0; u0 < per_lane; u0 += AHEAD) {
+        double v[AHEAD];
 #pragma unroll
-    for (int u = 0; u < per_lane; ++u) compensated_add(sum, comp, v[u]);
+        for (int u = 0; u < AHEAD; ++u) {
+            const int64_t s = s0 + (int64_t)(u0 + u) * 32;
+            v[u] = s < S ? load_value(x + s) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < AHEAD; ++u) neumaier_add(sum, comp, v[u]);
+    }
     warp_sum(sum, comp);
     return sum + comp;
 }
-__device__ __forceinline__ void chip_partials_sum(const double* x, int64_t n, int lane, double& sum, double& comp) {
-    sum = 0.0;
-    comp = 0.0;
-    if (n == 1) {   // one finite partial sum is the sum: the tree would add zeros to it
-        const double v = __ldcg(x);
-        if (((unsigned)__double2hiint(v) & 0x7fffffffu) < 0x7ff00000u) {
-            sum += v;
-            return;
-        }
-    }
-    for (int64_t b = lane; b < n; b += 32) compensated_add(sum, comp, __ldcg(x + b));
-    warp_sum(sum, comp);
-}
 
-// Blocks of an evaluation that has few of them, by teams of four warps: one FP64
-// operation takes 64 cycles of an SM quarter whatever its lanes do, so the four chains of
-// a block's compensated sum run on four quarters -- running sums, rounding errors (two
-// warps), sum of errors -- in chunks of eight values, each a phase behind the other
-// (one warp: 15,800 cycles per block).  Same numbers as chip_block_sum.  Uses kTeamBytes of shared memory per team; called by the whole CTA.
-constexpr int kTeamBytes = (33 + 32 + 1) * 32 * 8;
+// Sums of blocks of kReduceBlock samples by the whole CTA, its threads sharing a block's
+// values; same result as block_sum of the general kernels.
+static_assert(kScratchAt <= 320, "the level buffer has room for either");
+struct CtaSum {
+    unsigned mx[16];
+    Fixed f[16];
+};
+constexpr int kPerThread = 8;   // values of a thread, 128 threads
+
 template <typename T>
-__device__ __noinline__ void team_sums(const T* x, double* partials, int64_t S, unsigned char* sm) {
-    const int lane = threadIdx.x & 31, role = (threadIdx.x >> 5) & 3, team = threadIdx.x >> 7;
-    const int teams = min((int)blockDim.x >> 7, (int)(dynamic_smem_bytes() / kTeamBytes));
-    const int nblk = (int)((S + kReduceBlock - 1) / kReduceBlock);
-    double(*U)[32] = reinterpret_cast<double(*)[32]>(sm + team * kTeamBytes);   // running sums before each value
-    double(*E)[32] = U + 33;                                                    // rounding errors
-    for (int b0 = 0; b0 < nblk; b0 += teams) {
-        const bool mine = team < teams && b0 + team < nblk;
-        const int64_t s0 = (int64_t)(b0 + team) * kReduceBlock + lane;
-        double acc = 0.0, y[32];   // the values this warp needs: all, or every other one
-        if (mine && role != 3) {
+__device__ __forceinline__ void cta_load(double (&v)[kPerThread], const T* x, int64_t S, int64_t b) {
+    const int64_t s0 = b * kReduceBlock + threadIdx.x;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int64_t s = s0 + (role == 0 ? i : 2 * i + role - 1) * 32;
-                if (role == 0 || i < 16) y[i] = s < S ? ld_cg_f64(x + s) : 0.0;
-            }
-        }
-        if (mine && role == 0) U[0][lane] = 0.0;
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            __syncthreads();
-            if (!mine) continue;
-            if (role == 0) {
-                if (c < 4)
-#pragma unroll
-                    for (int i = 8 * c; i < 8 * c + 8 && i < 32; ++i) U[i + 1][lane] = acc = acc + y[i];
-            } else if (role == 3) {
-                if (c >= 2)
-#pragma unroll
-                    for (int i = 8 * c - 16; i < 8 * c - 8; ++i)
-                        if (i >= 0) acc += E[i][lane];
-            } else if (c >= 1 && c < 5) {
-#pragma unroll
-                for (int h = 4 * c - 4; h < 4 * c; ++h) {
-                    if (h < 0 || h >= 16) continue;
-                    const int i = 2 * h + role - 1;
-                    const double sum = U[i][lane], u = U[i + 1][lane], v = y[h];
-                    const bool ge = bigger(sum, v);
-                    E[i][lane] = ((ge ? sum : v) - u) + (ge ? v : sum);
-                }
-            }
-        }
-        __syncthreads();
-        if (mine && role == 3) E[32][lane] = acc;   // (one row behind the errors)
-        __syncthreads();
-        if (mine && role == 0) {
-            double comp = E[32][lane];
-            warp_sum(acc, comp);
-            if (lane == 0) partials[b0 + team] = acc + comp;
-        }
+    for (int u = 0; u < kPerThread; ++u) {
+        const int at = u * (int)blockDim.x;
+        v[u] = at < kReduceBlock && s0 + at < S ? load_value(x + s0 + at) : 0.0;
     }
+}
+// (two barriers; the partial sum is written by thread 0)
+template <typename T>
+__device__ __forceinline__ void cta_sum(double (&v)[kPerThread], const T* x, double* partials, int64_t S, int64_t b,
+                                        CtaSum& c) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, T_ = blockDim.x;
+    unsigned mx = 0;
+#pragma unroll
+    for (int u = 0; u < kPerThread; ++u) mx = max(mx, magnitude_word(v[u]));
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0) c.mx[warp] = mx;
     __syncthreads();
+    const int emax = warp_exponent(lane < nw ? c.mx[lane] : 0u);
+    if (!fixed_in_range(emax)) {
+        if (warp == 0) {
+            const double sum = block_sum_compensated(x, S, b, lane);
+            if (lane == 0) partials[b] = sum;
+        }
+        __syncthreads();
+        return;
+    }
+    Fixed f{{0u, 0u, 0u, 0u}};
+#pragma unroll 1
+    for (int u = 0; u * T_ < kReduceBlock; ++u) {   // (one copy of the code: it runs cold)
+        fixed_add_value(f, v[0], emax);
+#pragma unroll
+        for (int h = 0; h + 1 < kPerThread; ++h) v[h] = v[h + 1];
+    }
+    f = warp_fixed_sum(f);
+    if (lane == 0) c.f[warp] = f;
+    __syncthreads();
+    if (warp == 0) {
+        f = lane < nw ? c.f[lane] : Fixed{{0u, 0u, 0u, 0u}};
+        const double sum = fixed_value(warp_fixed_sum(f), emax);
+        if (lane == 0) partials[b] = sum;
+    }
+}
+constexpr unsigned kBlockSummed = 0xffffffffu;   // arrival word of a block whose partial sum is written
+
+// Partial sums of blocks [b, nblk) whose arrival word is not kBlockSummed (arrive
+// nullptr: of all).
+template <typename T>
+__device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S, int b, int nblk, const unsigned* arrive, CtaSum& c) {
+    // the next block to sum: 32 arrival words at a time (they change no more, so that every
+    // warp finds the same)
+    int base = -1;
+    unsigned open = 0;
+    auto skip = [&](int q) {
+        while (arrive && q < nblk) {
+            if ((q & ~31) != base) {
+                base = q & ~31;
+                const int at = base + (int)(threadIdx.x & 31);
+                open = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != kBlockSummed);
+            }
+            const unsigned left = open >> (q - base);
+            if (left) return q + __ffs((int)left) - 1;
+            q = base + 32;
+        }
+        return min(q, nblk);
+    };
+    double v[kPerThread], next[kPerThread];
+    b = skip(b);
+    if (b < nblk) cta_load(v, x, S, b);
+    while (b < nblk) {
+        const int n = skip(b + 1);
+        if (n < nblk) cta_load(next, x, S, n);   // a block ahead
+        cta_sum(v, x, partials, S, b, c);
+#pragma unroll
+        for (int u = 0; u < kPerThread; ++u) v[u] = next[u];
+        b = n;
+    }
 }
 template <int MODE>
-__device__ __forceinline__ void chip_sum_few(const ChipParams& p, unsigned char* sm) {
-    if constexpr (Traits<MODE>::kCount) team_sums(static_cast<const long long*>(p.R), p.partials, p.S, sm);
-    else team_sums(static_cast<const double*>(p.R), p.partials, p.S, sm);
-    if constexpr (Traits<MODE>::kAbs) team_sums(p.Rabs, p.partials_abs, p.S, sm);
+__device__ __noinline__ void chip_sums(const ChipParams& p, unsigned char* sm, int b, int nblk, const unsigned* arrive) {
+    CtaSum& c = *reinterpret_cast<CtaSum*>(sm);   // (the level buffer, free by now)
+    if constexpr (Traits<MODE>::kCount) cta_sums(static_cast<const long long*>(p.R), p.partials, p.S, b, nblk, arrive, c);
+    else cta_sums(static_cast<const double*>(p.R), p.partials, p.S, b, nblk, arrive, c);
+    if constexpr (Traits<MODE>::kAbs) cta_sums(p.Rabs, p.partials_abs, p.S, b, nblk, arrive, c);
 }
 
-constexpr unsigned kBlockSummed = 0xffffffffu;   // arrival word of a block whose partial sum is written
 
 // Count a chunk's results in (one thread; they were written by its warp).  Called a
 // phase after the writes, when the release has nothing left to wait for.
@@ -637,54 +644,42 @@ __device__ __forceinline__ void chip_arrive(const ChipParams& p, int chunk) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.arrive + s0 / kReduceBlock), "r"(mine) : "memory");
 }
 
-// Partial sum of block b by one warp.
-template <int MODE>
-__device__ __noinline__ void chip_sum_block(const ChipParams& p, int64_t b, int lane) {
-    double v, va = 0.0;
-    if constexpr (Traits<MODE>::kCount) v = chip_block_sum(static_cast<const long long*>(p.R), p.S, b, lane);
-    else v = chip_block_sum(static_cast<const double*>(p.R), p.S, b, lane);
-    if constexpr (Traits<MODE>::kAbs) va = chip_block_sum(p.Rabs, p.S, b, lane);
-    if (lane == 0) {
-        p.partials[b] = v;
-        if constexpr (Traits<MODE>::kAbs) p.partials_abs[b] = va;
-    }
-}
+__device__ __forceinline__ int chip_blocks(const ChipParams& p) { return (int)((p.S + kReduceBlock - 1) / kReduceBlock); }
 
 // A CTA that has no chunk left sums its share of the evaluation's blocks, as far as
 // they are complete; `first`: number of this evaluation's block 0 in the launch.
 template <int MODE>
-__device__ __forceinline__ void chip_sum_own(const ChipParams& p, int first) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int nblk = (int)((p.S + kReduceBlock - 1) / kReduceBlock), grid = gridDim.x;
-    const int b0 = (int)((blockIdx.x + grid - first % grid) % grid);
-    for (int b = b0 + warp * grid; b < nblk; b += nw * grid) {
-        const unsigned full = (unsigned)min((int64_t)kReduceBlock, p.S - (int64_t)b * kReduceBlock);
-        const unsigned got = lane == 0 ? ld_acquire_gpu_u32(p.arrive + b) : 0u;
-        if (__shfl_sync(0xffffffffu, got, 0) != full) continue;
-        chip_sum_block<MODE>(p, b, lane);
-        __syncwarp();
-        if (lane == 0) p.arrive[b] = kBlockSummed;   // (read by the last CTA, after this one's release)
+__device__ __forceinline__ void chip_sum_own(const ChipParams& p, unsigned char* sm, int first) {
+    __shared__ int s_full;
+    const int nblk = chip_blocks(p), grid = gridDim.x;
+    for (int b = (int)((blockIdx.x + grid - first % grid) % grid); b < nblk; b += grid) {
+        if (threadIdx.x == 0)
+            s_full = ld_acquire_gpu_u32(p.arrive + b) == (unsigned)min((int64_t)kReduceBlock, p.S - (int64_t)b * kReduceBlock);
+        __syncthreads();
+        const bool full = s_full != 0;
+        __syncthreads();
+        if (!full) continue;
+        chip_sums<MODE>(p, sm, b, b + 1, nullptr);
+        if (threadIdx.x == 0) p.arrive[b] = kBlockSummed;   // (read by the last CTA, after this one's release)
     }
 }
 
 // The last CTA of the launch: the blocks nobody has summed, then the means.  The
 // arrival words are left at zero.
 template <int MODE>
-__device__ __forceinline__ void chip_sum_rest(const ChipParams& p) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int nblk = (int)((p.S + kReduceBlock - 1) / kReduceBlock);
-    for (int b = warp; b < nblk; b += nw) {
-        const unsigned got = __shfl_sync(0xffffffffu, lane == 0 ? __ldcg(p.arrive + b) : 0u, 0);
-        if (got != kBlockSummed) chip_sum_block<MODE>(p, b, lane);
-        if (lane == 0) p.arrive[b] = 0;
-    }
+__device__ __forceinline__ void chip_sum_rest(const ChipParams& p, unsigned char* sm, bool all) {
+    const int nblk = chip_blocks(p);
+    chip_sums<MODE>(p, sm, 0, nblk, all ? nullptr : p.arrive);
+    if (all) return;
+    __syncthreads();
+    for (int b = threadIdx.x; b < nblk; b += blockDim.x) p.arrive[b] = 0;
 }
 template <int MODE>
 __device__ __noinline__ void chip_mean(const ChipParams& p, int lane) {
     const int64_t nblk = (p.S + kReduceBlock - 1) / kReduceBlock;
     double sum, comp, sa = 0.0, ca = 0.0;
-    chip_partials_sum(p.partials, nblk, lane, sum, comp);
-    if constexpr (Traits<MODE>::kAbs) chip_partials_sum(p.partials_abs, nblk, lane, sa, ca);
+    partials_sum(p.partials, nblk, lane, sum, comp);
+    if constexpr (Traits<MODE>::kAbs) partials_sum(p.partials_abs, nblk, lane, sa, ca);
     if (lane == 0) {
         const double mean = (sum + comp) / (double)p.S, mean_abs = (sa + ca) / (double)p.S;
         p.ctrl->sum = sum;
@@ -938,7 +933,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
                 return n < a.one.nchunks ? n : -1;
             });
         chip_finish<MODE>(a.one, sm, cs);
-        if (!a.few) chip_sum_own<MODE>(a.one, 0);
+        if (!a.few) chip_sum_own<MODE>(a.one, sm, 0);
     } else {
         int g = -1;
         for (int buf = 0;; buf ^= 1) {
@@ -968,7 +963,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
         if (g >= 0) chip_finish<MODE>(s_p, sm, cs);
         int first = 0;
         for (int h = 0; h < a.n && !a.few; ++h) {
-            chip_sum_own<MODE>(a.list[h], first);
+            chip_sum_own<MODE>(a.list[h], sm, first);
             first += (int)((a.list[h].S + kReduceBlock - 1) / kReduceBlock);
         }
     }
@@ -983,8 +978,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
         const int n = a.list ? a.n : 1;
         for (int h = 0; h < n; ++h) {
             const ChipParams& p = a.list ? a.list[h] : a.one;
-            if (a.few) chip_sum_few<MODE>(p, sm);
-            else chip_sum_rest<MODE>(p);
+            chip_sum_rest<MODE>(p, sm, a.few != 0);
         }
         __syncthreads();
         for (int h = warp; h < n; h += blockDim.x >> 5) chip_mean<MODE>(a.list ? a.list[h] : a.one, threadIdx.x & 31);
@@ -1038,7 +1032,7 @@ ChipLayout chip_layout(const ChipGraph& g, int kmode, int P, int K, int D, bool 
     const int64_t times = count ? 0 : round128(8LL * D * s), tab = round128(16LL * g.tables);
     const int64_t coef = count ? 0 : round128(chip_coef_bytes(K));
     const int64_t tail = g.tail_width <= kTailRows ? round128((int64_t)(g.tail_width + 1) * rb) : 0;
-    const int64_t level = std::max<int64_t>(round128((int64_t)(g.max_width + 1) * rb), kScratchAt);
+    const int64_t level = std::max<int64_t>(round128((int64_t)(g.max_width + 1) * rb), round128(sizeof(CtaSum)));
     const int64_t rest = gbytes + times + tab + coef + tail;
     int64_t lev = level;
     y.kinds = K;
@@ -1181,8 +1175,7 @@ int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, c
     const int64_t blocks = (p.S + kReduceBlock - 1) / kReduceBlock;
     a.exits = p.arrive + blocks;
     a.few = blocks <= few_blocks(plan.threads);
-    const int smem = a.few ? std::max(plan.smem, kTeamBytes * (int)std::min<int64_t>(plan.threads / 128, blocks)) : plan.smem;
-    return launch(kmode, plan.lane_bytes, plan.threads, smem, a, p.nchunks, sms, st);
+    return launch(kmode, plan.lane_bytes, plan.threads, plan.smem, a, p.nchunks, sms, st);
 }
 
 int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const ChipParams* list, int n, int total,

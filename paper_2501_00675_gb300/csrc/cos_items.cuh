@@ -18,6 +18,7 @@
 // Either way a lane moves V values per access (16 B for float with V = 4).
 #pragma once
 
+#include "cos_fixed.h"
 #include <cstdint>
 
 #include "cos_internal.cuh"
@@ -1401,33 +1402,87 @@ __device__ __forceinline__ void warp_sum(double& s, double& c) {
     for (int o = 16; o >= 1; o >>= 1) add_pair(s, c, __shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o));
 }
 
-// Compensated partial sums of R over blocks of kReduceBlock samples in a fixed order:
-// lane q adds samples q, q+32, q+64, ... of the block with Neumaier compensation
-// (coalesced loads, all issued ahead of the adds), then the lanes are combined by an
-// error-free pairwise tree.  Item = kWarps consecutive blocks (one per warp).
+// Partial sums of R over blocks of kReduceBlock samples: in 128-bit integers (cos_fixed.h),
+// or, for values outside their range, lane q adds samples q, q+32, q+64, ... of the block
+// with Neumaier compensation and the lanes are combined by an error-free pairwise tree.
+// Either way the result depends on the values only, not on the kernel that forms it.
+// Item = kWarps consecutive blocks (one per warp).
 __device__ __forceinline__ int partial_items(const WalkParams& p) {
     const int64_t nblk = (p.S + kReduceBlock - 1) / kReduceBlock;
     return (int)((nblk + kWarps - 1) / kWarps);
 }
 
-// Compensated sum of block b (kReduceBlock samples) of x, returned on every lane.
+// R(s) as a double, from L2: it comes from other CTAs of the launch.
+__device__ __forceinline__ double load_value(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ double load_value(const long long* p) { return (double)__ldcg(p); }
+
+__device__ __forceinline__ bool fixed_in_range(int emax) { return emax >= kFixedMin && emax <= kFixedMax; }
+
+// Largest exponent field over a warp of the largest high word with the sign cleared.
+__device__ __forceinline__ int warp_exponent(unsigned mx) { return (int)(__reduce_max_sync(0xffffffffu, mx) >> 20); }
+
+// Sum of one Fixed per lane, on every lane: 16-bit halves by redux.
+__device__ __forceinline__ Fixed warp_fixed_sum(const Fixed& f) {
+    unsigned h[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        h[2 * i] = __reduce_add_sync(0xffffffffu, f.w[i] & 0xffffu);
+        h[2 * i + 1] = __reduce_add_sync(0xffffffffu, f.w[i] >> 16);
+    }
+    Fixed a{{h[0], h[2], h[4], h[6]}};
+    const Fixed b{{h[1] << 16, h[1] >> 16 | h[3] << 16, h[3] >> 16 | h[5] << 16, h[5] >> 16 | h[7] << 16}};
+    fixed_add(a, b, 0u);
+    return a;
+}
+__device__ __forceinline__ double fixed_value(const Fixed& f, int top) {
+    uint32_t hi, lo;
+    fixed_to_double(f, top, hi, lo);
+    return __hiloint2double((int)hi, (int)lo);
+}
+__device__ __forceinline__ unsigned magnitude_word(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
+__device__ __forceinline__ void fixed_add_value(Fixed& f, double v, int top) {
+    fixed_add_double(f, (unsigned)__double2hiint(v), (unsigned)__double2loint(v), top);
+}
+
+// Sum of block b by one warp, returned on every lane.  (Inlined: a call would cost the
+// FP64 kernels registers, 4 % of their time.)
 template <typename T>
 __device__ __forceinline__ double block_sum(const T* __restrict__ x, int64_t S, int64_t b, int lane) {
-    constexpr int per_lane = kReduceBlock / 32;
-    constexpr int AHEAD = 8;
+    constexpr int per_lane = kReduceBlock / 32, AHEAD = 8;
     const int64_t s0 = b * kReduceBlock + lane;
+    unsigned mx = 0;
+    Fixed f{{0u, 0u, 0u, 0u}};
     double sum = 0.0, comp = 0.0;
+    int emax = 0;
+    bool fixed = false;
 #pragma unroll 1
-    for (int u0 = 0; u0 < per_lane; u0 += AHEAD) {
+    for (int u0 = 0; u0 < 2 * per_lane; u0 += AHEAD) {   // the exponents, then the values again
         double v[AHEAD];
 #pragma unroll
         for (int u = 0; u < AHEAD; ++u) {
-            const int64_t s = s0 + (int64_t)(u0 + u) * 32;
-            v[u] = s < S ? (double)x[s] : 0.0;
+            const int64_t s = s0 + (int64_t)((u0 + u) & (per_lane - 1)) * 32;
+            v[u] = s < S ? load_value(x + s) : 0.0;
         }
+        if (u0 < per_lane) {
 #pragma unroll
-        for (int u = 0; u < AHEAD; ++u) neumaier_add(sum, comp, v[u]);
+            for (int u = 0; u < AHEAD; ++u) mx = max(mx, magnitude_word(v[u]));
+            if (u0 + AHEAD == per_lane) {
+                emax = warp_exponent(mx);
+                fixed = fixed_in_range(emax);
+            }
+        } else if (fixed) {
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) fixed_add_value(f, v[u], emax);
+        } else {
+#pragma unroll 1
+            for (int u = 0; u < AHEAD; ++u) {
+                neumaier_add(sum, comp, v[0]);
+#pragma unroll
+                for (int h = 0; h + 1 < AHEAD; ++h) v[h] = v[h + 1];
+            }
+        }
     }
+    if (fixed) return fixed_value(warp_fixed_sum(f), emax);
     warp_sum(sum, comp);
     return sum + comp;
 }
@@ -1448,15 +1503,41 @@ __device__ __forceinline__ void item_partials(const WalkParams& p, int item) {
     }
 }
 
-// Compensated sum of n block partials (lane-strided Neumaier, then the lane tree).
+// Sum of n block partials by one warp, on every lane, as sum + comp.
 __device__ __forceinline__ void partials_sum(const double* x, int64_t n, int lane, double& sum, double& comp) {
-    sum = 0.0;
     comp = 0.0;
-    for (int64_t b = lane; b < n; b += 32) neumaier_add(sum, comp, x[b]);
-    warp_sum(sum, comp);
+    if (n == 1) {   // one finite partial sum is the sum
+        sum = 0.0 + __ldcg(x);
+        if (magnitude_word(sum) < 0x7ff00000u) return;
+    }
+    constexpr int HELD = 4, EXTRA = 20;   // (room for 2^30 partial sums)
+    double v[HELD];
+    unsigned mx = 0;
+#pragma unroll
+    for (int u = 0; u < HELD; ++u) {
+        v[u] = lane + u * 32 < n ? __ldcg(x + lane + u * 32) : 0.0;
+        mx = max(mx, magnitude_word(v[u]));
+    }
+    for (int64_t b = lane + HELD * 32; b < n; b += 32) mx = max(mx, magnitude_word(__ldcg(x + b)));
+    const int emax = warp_exponent(mx), top = emax + EXTRA;
+    if (!fixed_in_range(emax)) {
+        sum = 0.0;
+        for (int64_t b = lane; b < n; b += 32) neumaier_add(sum, comp, __ldcg(x + b));
+        warp_sum(sum, comp);
+        return;
+    }
+    Fixed f{{0u, 0u, 0u, 0u}};
+#pragma unroll 1
+    for (int u = 0; u < HELD; ++u) {
+        fixed_add_value(f, v[0], top);
+#pragma unroll
+        for (int h = 0; h + 1 < HELD; ++h) v[h] = v[h + 1];
+    }
+    for (int64_t b = lane + HELD * 32; b < n; b += 32) fixed_add_value(f, __ldcg(x + b), top);
+    sum = fixed_value(warp_fixed_sum(f), top);
 }
 
-// Final compensated sum of the block partials by warp 0 of one CTA; the mean over
+// Final sum of the block partials by warp 0 of one CTA; the mean over
 // samples (and the mean of A(s) when the walk accumulated it).
 __device__ __forceinline__ void item_final(const WalkParams& p) {
     if (threadIdx.x >= 32) return;
