@@ -744,8 +744,26 @@ int cos_autotune(cos_graph_t g, int32_t mode, void* per_sample_out, void* stream
     return COS_OK;
 }
 
-int cos_set_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t t_flags, const double* eps,
-                    double beta, void* stream) {
+// The energies as parameters of the launch that places the times, or (more of them than
+// travel that way, or a capturing stream, whose replays read the host's array) by a copy.
+static int stage_energies(cos_graph_t g, const double* eps, cudaStream_t st, Energies* e) {
+    e->dst = nullptr;
+    e->n = 0;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (g->K <= kInlineEnergies && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+        e->dst = g->d_eps;
+        e->n = g->K;
+        memcpy(e->v, eps, sizeof(double) * g->K);
+        return COS_OK;
+    }
+    COS_CUDA(cudaMemcpyAsync(g->d_eps, eps, sizeof(double) * g->K, cudaMemcpyHostToDevice, st), "copy eps");
+    return COS_OK;
+}
+
+// cos_set_samples; with `rest` the caller's launch writes the energies (left in *rest) and
+// the times.
+static int attach_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t t_flags, const double* eps,
+                          double beta, void* stream, Energies* rest) {
     if (!g) return fail(COS_ERR_INVALID, "graph is NULL");
     if (num_samples < 0) return fail(COS_ERR_INVALID, "num_samples must be >= 0");
     if (num_samples > 0 && !t) return fail(COS_ERR_INVALID, "t is NULL");
@@ -800,18 +818,20 @@ int cos_set_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t
             g->arena_bytes = bytes;
         }
     }
-    COS_CUDA(cudaMemcpyAsync(g->d_eps, eps, sizeof(double) * g->K, cudaMemcpyHostToDevice, st), "copy eps");
+    Energies energies;
+    int rc = stage_energies(g, eps, st, &energies);
+    if (rc != COS_OK) return rc;
     g->t_borrowed = borrow ? t : nullptr;
-    if (!borrow) COS_CUDA(cudaMemsetAsync(g->d_t, 0, sizeof(double) * t_ld * D, st), "clear t");
+    PlaceFrom from = borrow ? PLACE_NOTHING : PLACE_PADDING;
+    const double* src = t;
     if (S > 0 && !borrow) {
         const bool host = (t_flags & COS_T_HOST) != 0;
-        const bool smaj = (t_flags & COS_T_SAMPLE_MAJOR) != 0;
-        if (!smaj) {
+        if (!(t_flags & COS_T_SAMPLE_MAJOR)) {
             COS_CUDA(cudaMemcpy2DAsync(g->d_t, sizeof(double) * t_ld, t, sizeof(double) * S, sizeof(double) * S, D,
                                        host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st),
                      "copy t");
         } else {
-            const double* src = t;
+            from = PLACE_SAMPLE_MAJOR;
             if (host) {
                 if (S * D > g->stage_cap) {
                     dfree(g->d_stage);
@@ -821,9 +841,13 @@ int cos_set_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t
                 COS_CUDA(cudaMemcpyAsync(g->d_stage, t, sizeof(double) * S * D, cudaMemcpyHostToDevice, st), "copy t");
                 src = g->d_stage;
             }
-            int rc = launch_transpose(src, S, D, g->d_t, t_ld, st);
-            if (rc != COS_OK) return fail(rc, "transpose launch failed: %s", cudaGetErrorString(cudaGetLastError()));
         }
+    }
+    if (rest) {
+        *rest = energies;
+    } else {
+        rc = launch_place(from, src, S, D, g->d_t, t_ld, energies, st);
+        if (rc != COS_OK) return fail(rc, "launch of the time layout failed: %s", cudaGetErrorString(cudaGetLastError()));
     }
     g->S = S;
     g->t_ld = t_ld;
@@ -831,6 +855,11 @@ int cos_set_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t
     g->has_samples = true;
     g->generation++;
     return COS_OK;
+}
+
+int cos_set_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t t_flags, const double* eps,
+                    double beta, void* stream) {
+    return attach_samples(g, num_samples, t, t_flags, eps, beta, stream, nullptr);
 }
 
 int cos_set_samples_uniform(cos_graph_t g, int64_t num_samples, uint64_t seed, int64_t first_sample,
@@ -847,16 +876,14 @@ int cos_set_samples_uniform(cos_graph_t g, int64_t num_samples, uint64_t seed, i
         COS_CUDA(cudaMalloc(&g->d_t, sizeof(double) * t_ld * g->D), "cudaMalloc t");
         g->t_cap = t_ld * g->D;
     }
-    int rc = cos_set_samples(g, num_samples, g->d_t, COS_T_BORROW, eps, beta, stream);
+    Energies energies;
+    int rc = attach_samples(g, num_samples, g->d_t, COS_T_BORROW, eps, beta, stream, &energies);
     if (rc != COS_OK) return rc;
     // ... then fill the graph's own time buffer with the counter-based draws
     g->t_borrowed = nullptr;
     g->generation++;
-    COS_CUDA(cudaMemsetAsync(g->d_t, 0, sizeof(double) * t_ld * g->D, st), "clear t");
-    if (num_samples > 0) {
-        rc = launch_uniform_times(seed, first_sample, num_samples, g->D, beta, g->d_t, t_ld, st);
-        if (rc != COS_OK) return fail(rc, "sampler launch failed");
-    }
+    rc = launch_uniform_times(seed, first_sample, num_samples, g->D, beta, g->d_t, t_ld, energies, st);
+    if (rc != COS_OK) return fail(rc, "sampler launch failed");
     return COS_OK;
 }
 

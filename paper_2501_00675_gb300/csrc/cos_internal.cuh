@@ -169,10 +169,20 @@ int prepare_kernel_attrs(const void* kernel, int smem_bytes);
 int probe_fma_rate(int precision, double* per_second, char* msg, size_t msglen);
 // e^{-x} and e^{+x} with the evaluator's table-driven exponentials (self test).
 int launch_exp_pair(const double* x, int64_t n, const double* tab, double* em, double* ep, cudaStream_t stream);
+// Times in sample-major order into the handle's [D][t_ld] layout (or only the zeros behind
+// sample S), and the energies, in one launch.
+enum PlaceFrom { PLACE_NOTHING, PLACE_PADDING, PLACE_SAMPLE_MAJOR };
+constexpr int kInlineEnergies = 64;   // energies that travel as kernel parameters
+struct Energies {
+    double* dst;                      // nullptr: none to write
+    int32_t n;
+    double v[kInlineEnergies];
+};
 // Counter-based uniform times t[i][s] in [0, beta) for samples first..first+S-1.
 int launch_uniform_times(uint64_t seed, int64_t first, int64_t S, int32_t D, double beta, double* t, int64_t t_ld,
-                         cudaStream_t stream);
+                         const Energies& eps, cudaStream_t stream);
 // Transpose t from [S][D] (src_ld = D) into [D][t_ld].
-int launch_transpose(const double* src, int64_t S, int32_t D, double* dst, int64_t t_ld, cudaStream_t stream);
+int launch_place(PlaceFrom from, const double* src, int64_t S, int32_t D, double* dst, int64_t t_ld, const Energies& eps,
+                 cudaStream_t stream);
 
 }  // namespace cosgpu

@@ -100,28 +100,57 @@ __global__ void __launch_bounds__(kThreads, min_blocks<MODE, V, LAYOUT>()) walk_
     if (blockIdx.x == 0) item_final(p);
 }
 
-__global__ void transpose_kernel(const double* __restrict__ src, int64_t S, int32_t D, double* __restrict__ dst,
-                                 int64_t t_ld) {
-    const int64_t total = S * D;
-    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = idx / S, s = idx % S;
-        dst[i * t_ld + s] = src[s * D + i];
+__device__ __forceinline__ void write_energies(const Energies& e) {
+    if (blockIdx.x == 0 && e.dst)
+        for (int k = threadIdx.x; k < e.n; k += blockDim.x) e.dst[k] = e.v[k];
+}
+
+// The times of a call in the layout of the walks.  Replaces a copy of the energies, a
+// memset and a kernel whose writes were D strides apart: with S = 1,024, D = 6 the three took
+// 8.3 us on the device, one after another, for 50 KB; what is left is one launch.  A block
+// moves 64 samples through shared memory, 32 times at a time, so that both sides are read and
+// written in whole sectors.
+constexpr int kPlaceSamples = 64, kPlaceTimes = 32;
+__global__ void __launch_bounds__(256) place_kernel(int from, const double* __restrict__ src, int64_t S, int32_t D,
+                                                    double* __restrict__ dst, int64_t t_ld, const __grid_constant__ Energies eps) {
+    __shared__ double tile[kPlaceTimes][kPlaceSamples + 1];
+    write_energies(eps);
+    if (from == PLACE_SAMPLE_MAJOR) {
+        for (int64_t s0 = (int64_t)blockIdx.x * kPlaceSamples; s0 < t_ld; s0 += (int64_t)gridDim.x * kPlaceSamples)
+            for (int i0 = 0; i0 < D; i0 += kPlaceTimes) {
+                const int dn = min(kPlaceTimes, D - i0);
+                __syncthreads();
+                for (int x = threadIdx.x; x < kPlaceSamples * dn; x += blockDim.x) {
+                    const int s = x / dn, i = x - s * dn;
+                    tile[i][s] = s0 + s < S ? src[(s0 + s) * D + i0 + i] : 0.0;
+                }
+                __syncthreads();
+                for (int x = threadIdx.x; x < kPlaceSamples * dn; x += blockDim.x) {
+                    const int i = x / kPlaceSamples, s = x % kPlaceSamples;
+                    dst[(i0 + i) * t_ld + s0 + s] = tile[i][s];
+                }
+            }
+    } else if (from == PLACE_PADDING) {
+        const int64_t n = t_ld - S;
+        for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n * D; x += (int64_t)gridDim.x * blockDim.x)
+            dst[x / n * t_ld + S + x % n] = 0.0;
     }
 }
 
 // t[2m][s], t[2m+1][s] for sample n = first + s: counter (n lo, n hi, m, 0), key = seed;
 // 53 bits of each word pair scaled to [0, beta).
+// Zeros behind sample S.
 __global__ void uniform_times_kernel(unsigned long long seed, long long first, long long S, int D, double beta,
-                                     double* __restrict__ t, long long t_ld) {
+                                     double* __restrict__ t, long long t_ld, const __grid_constant__ Energies eps) {
+    write_energies(eps);
     const int pairs = (D + 1) / 2;
-    const long long total = S * pairs;
+    const long long total = t_ld * pairs;
     for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
          q += (long long)gridDim.x * blockDim.x) {
-        const int m = (int)(q / S);
-        const long long s = q - (long long)m * S;
-        double a, b;
-        uniform_time_pair(seed, (unsigned long long)(first + s), m, beta, a, b);
+        const int m = (int)(q / t_ld);
+        const long long s = q - (long long)m * t_ld;
+        double a = 0.0, b = 0.0;
+        if (s < S) uniform_time_pair(seed, (unsigned long long)(first + s), m, beta, a, b);
         t[(long long)(2 * m) * t_ld + s] = a;
         if (2 * m + 1 < D) t[(long long)(2 * m + 1) * t_ld + s] = b;
     }
@@ -311,18 +340,22 @@ int launch_exp_pair(const double* x, int64_t n, const double* tab, double* em, d
 }
 
 int launch_uniform_times(uint64_t seed, int64_t first, int64_t S, int32_t D, double beta, double* t, int64_t t_ld,
-                         cudaStream_t stream) {
-    const int64_t total = S * ((D + 1) / 2);
+                         const Energies& eps, cudaStream_t stream) {
+    const int64_t total = t_ld * ((D + 1) / 2);
     const int64_t blocks = std::min<int64_t>((total + 255) / 256, 152LL * 16);
-    uniform_times_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, stream>>>(seed, first, S, D, beta, t, t_ld);
+    uniform_times_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), 256, 0, stream>>>(seed, first, S, D, beta, t, t_ld, eps);
     return cudaGetLastError() == cudaSuccess ? COS_OK : COS_ERR_CUDA;
 }
 
-int launch_transpose(const double* src, int64_t S, int32_t D, double* dst, int64_t t_ld, cudaStream_t stream) {
-    const int64_t total = S * D;
-    const int threads = 256;
-    const int64_t blocks = std::min<int64_t>((total + threads - 1) / threads, 152LL * 16);
-    transpose_kernel<<<(unsigned)std::max<int64_t>(blocks, 1), threads, 0, stream>>>(src, S, D, dst, t_ld);
+int launch_place(PlaceFrom from, const double* src, int64_t S, int32_t D, double* dst, int64_t t_ld, const Energies& eps,
+                 cudaStream_t stream) {
+    if (from == PLACE_PADDING && t_ld == S) from = PLACE_NOTHING;
+    if (from == PLACE_NOTHING && !eps.dst) return COS_OK;
+    int64_t blocks = 1;
+    if (from == PLACE_SAMPLE_MAJOR) blocks = t_ld / kPlaceSamples;   // (t_ld is a multiple of 128)
+    if (from == PLACE_PADDING) blocks = ((t_ld - S) * D + 255) / 256;
+    blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, 152LL * 8));
+    place_kernel<<<(unsigned)blocks, 256, 0, stream>>>(from, src, S, D, dst, t_ld, eps);
     return cudaGetLastError() == cudaSuccess ? COS_OK : COS_ERR_CUDA;
 }
 
