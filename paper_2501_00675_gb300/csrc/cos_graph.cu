@@ -152,6 +152,9 @@ struct cos_graph {
     int32_t ptab_T = 0;
     double ptab_tau_max = 0.0;
     int last_wave = 0;              // the last evaluate ran the windowed schedule
+    // page-locked (mean R, mean A), written by the on-chip walk of a call that waits for its
+    // mean: reading the control block takes a copy after the kernel (nullptr: no such memory)
+    double* h_means = nullptr;
     // Bumped whenever something a batch plan copies from the handle may change: the
     // sample buffers, sample count or layout, the workspace, the internal result
     // buffer, the propagator tables or the tuning.  A batch re-plans when it differs.
@@ -207,6 +210,14 @@ bool carve(cos_graph* g, int kmode, int64_t tile, WalkParams& p) {
     p.gtab = (mode != COS_MODE_COUNT_I64) ? (void*)(base + gt) : nullptr;
     p.coef = (double*)(base + cf);
     return true;
+}
+
+void alloc_means(cos_graph* g) {
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, 2 * sizeof(double), cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess)
+        g->h_means = static_cast<double*>(p);
+    else
+        cudaGetLastError();   // the control block serves without it
 }
 
 // Row schedule of the on-chip walk for a graph whose levels fit shared memory (none
@@ -445,6 +456,7 @@ int cos_create_graph(int32_t num_levels, const int64_t* level_width, const int64
     if ((e = cudaMalloc(&g->d_edges, sizeof(int2) * std::max<int64_t>(E, 1))) != cudaSuccess) return cleanup_fail(e, "cudaMalloc edges");
     if ((e = cudaMalloc(&g->d_slot_kij, sizeof(int32_t) * std::max<int64_t>(3 * P, 3))) != cudaSuccess) return cleanup_fail(e, "cudaMalloc slots");
     if ((e = cudaMalloc(&g->d_ctrl, sizeof(Ctrl))) != cudaSuccess) return cleanup_fail(e, "cudaMalloc ctrl");
+    alloc_means(g);
     {
         // slots are numbered in (kind, i, j) order, so every kind owns one contiguous range
         std::vector<int32_t> ks((size_t)num_kinds + 1, 0);
@@ -526,6 +538,7 @@ int cos_graph_share(cos_graph_t src, cos_graph_t* out) {
         cos_destroy(g);
         return rc;
     }
+    alloc_means(g);
     *out = g;
     return COS_OK;
 }
@@ -548,6 +561,7 @@ int cos_destroy(cos_graph_t g) {
             dfree(g->d_exp_tab);
         }
         dfree(g->d_ctrl);
+        if (g->h_means) cudaFreeHost(g->h_means);
         dfree(g->d_t);
         dfree(g->d_eps);
         dfree(g->d_stage);
@@ -899,6 +913,8 @@ int cos_copy_times(cos_graph_t g, double* dst, void* stream) {
     return COS_OK;
 }
 
+static const char kOverflowText[] = "path count exceeds 2^63-1; results wrap modulo 2^64";
+
 static int collect(cos_graph_t g, double* mean_out, cudaStream_t st) {
     const bool abs2 = mode_has_abs(g->last_mode);   // mean_out holds (mean R, mean A)
     if (g->last_wave && g->wave) {   // windowed schedule: errors are in the batch's control block
@@ -923,7 +939,7 @@ static int collect(cos_graph_t g, double* mean_out, cudaStream_t st) {
         if (abs2) mean_out[1] = c.mean_abs;
     }
     if (g->last_mode == COS_MODE_COUNT_I64 && g->count_overflow)
-        return fail(COS_ERR_OVERFLOW, "path count exceeds 2^63-1; results wrap modulo 2^64");
+        return fail(COS_ERR_OVERFLOW, kOverflowText);
     return COS_OK;
 }
 
@@ -942,9 +958,21 @@ int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean
         int sms = 0;
         int on_chip = 0;
         int rc = prepare_chip(g, km, per_sample_out, &cp, &plan, &sms, &on_chip);
-        if (rc == COS_OK && on_chip) rc = launch_chip(km, plan, cp, sms, st);
+        if (rc == COS_OK && on_chip) {
+            if (mean_out) cp.mean_out = g->h_means;
+            rc = launch_chip(km, plan, cp, sms, st);
+        }
         if (rc != COS_OK) return rc;
         if (on_chip) {
+            if (mean_out && g->h_means) {   // (the on-chip walk reports no errors of its own)
+                g->last_wave = 0;
+                g->last_mode = km;
+                COS_CUDA(cudaStreamSynchronize(st), "synchronize");
+                g->last_status_pending = 0;
+                mean_out[0] = g->h_means[0];
+                if (mode_has_abs(km)) mean_out[1] = g->h_means[1];
+                return km == COS_MODE_COUNT_I64 && g->count_overflow ? fail(COS_ERR_OVERFLOW, kOverflowText) : COS_OK;
+            }
             g->last_wave = 0;
             g->last_mode = km;
             g->last_status_pending = 1;
