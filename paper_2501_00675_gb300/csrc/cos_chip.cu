@@ -21,10 +21,10 @@
 // What bounds it (ncu, medium graph, FP32, 16,384 samples): the shared-memory pipe, two
 // 16-byte reads per edge and lane, 68 % of all cycles busy, a third of that bank conflicts
 // that the row order of cos_chip.h leaves; issue slots 38 %, DRAM 0.  A chunk of 8 samples
-// takes 66,000 cycles, 43,000 of them in its four levels of 4,096 rows, 10,000 in the
+// takes 64,600 cycles, 43,000 of them in its four levels of 4,096 rows, 9,000 in the
 // propagators; a small level costs some 900 cycles whatever it holds.  Medium graph, 65,536
-// samples, before (general kernels) and after: FP32 2.35 -> 1.66 ms, with A 3.00 -> 2.24,
-// count 3.2 -> 1.91.  The FP64 walk is bound by the FP64 pipe on both paths (6.3 / 6.9 ms).
+// samples, before (general kernels) and after: FP32 2.35 -> 1.61 ms, with A 3.00 -> 2.20,
+// count 3.2 -> 1.87.  The FP64 walk is bound by the FP64 pipe on both paths (6.3 / 6.9 ms).
 //
 // CTAs never wait for one another: a CTA that has no chunk left sums its share of the
 // blocks of kReduceBlock samples that are complete, the last CTA the others, and it forms
@@ -217,6 +217,12 @@ __device__ __forceinline__ bool within_30(double x) {
     return hi < 0x403e0000u || (hi == 0x403e0000u && __double2loint(x) == 0);
 }
 
+// What bounds the propagators is the instructions of the exponentials (some 115 each, one of
+// them FP64; 38 % of the issue slots used) and fetching them: the loops have one copy of
+// their code, and a graph whose kinds need no double arithmetic never enters its loop.  Order
+// 2, 32 kinds, 32 samples a chunk: exponentials 18,000 -> 14,000 cycles, slots 15,700 ->
+// 10,900, of 50,000 -> 45,000 (84 -> 72 us for 10,007 samples).
+//
 // Exponentials of the kinds [k0, k0 + kn), times and samples of the chunk, with the
 // arithmetic of item_props of the general kernels.  Returns whether a time lies so far
 // outside [-beta, beta] that float-float arithmetic does not apply (then the caller
@@ -231,48 +237,69 @@ __device__ __forceinline__ bool chip_exps(const ChipParams& p, unsigned char* sm
     double* fb = fa + np;                                                           // coef- e^{-eps t}
     double* fc = fb + np;                                                           // e^{+eps t}
     const int T = blockDim.x;
-    bool far = false;
-    if (Tr::kBase == COS_MODE_FP32_MIXED && !in_double) {
-        // two independent chains per thread; warp 0, which has a sink to sum, comes last
+    constexpr bool kMixed = Tr::kBase == COS_MODE_FP32_MIXED;
+    bool far = false, rest = true;   // rest: this thread has exponentials to form in double
+    if (kMixed && !in_double) {
+        rest = false;
+        // two independent chains per thread, their arguments (the FP64 part) formed a round
+        // ahead; warp 0, which has a sink to sum, comes last
         const int half = (n + 1) / 2;
-        for (int x0 = T - 1 - (int)threadIdx.x; x0 < half; x0 += T) {
-            float2 em[2], ep[2];
-            int k[2], at[2];
-            bool ok[2];
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int x = x0 + u * half < n ? x0 + u * half : x0;
-                const unsigned r = (unsigned)x >> sl;
-                at[u] = (int)r * pitch + (x & (s - 1));
-                const int kk = D == 1 ? (int)r : (int)__umulhi(r, p.d_magic);
-                k[u] = k0 + kk;
-                const double arg = c.eps[k[u]] * st[x - kk * DS];
-                ok[u] = within_30(arg);
-                exp_pair_ff(ok[u] ? arg : 0.0, reinterpret_cast<const float2*>(c.tab), em[u], ep[u]);
+        struct Item {
+            int k, at;
+            double arg;
+        };
+        auto fetch = [&](int x) {
+            const unsigned r = (unsigned)x >> sl;
+            const int kk = D == 1 ? (int)r : (int)__umulhi(r, p.d_magic);
+            return Item{k0 + kk, (int)r * pitch + (x & (s - 1)), c.eps[k0 + kk] * st[x - kk * DS]};
+        };
+        auto second = [&](int x) { return x + half < n ? x + half : x; };
+        int x = T - 1 - (int)threadIdx.x;
+        Item next[2];
+        if (x < half) {
+            next[0] = fetch(x);
+            next[1] = fetch(second(x));
+        }
+        for (; x < half; x += T) {
+            const Item it[2] = {next[0], next[1]};
+            if (x + T < half) {
+                next[0] = fetch(x + T);
+                next[1] = fetch(second(x + T));
             }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                if (!c.ff[k[u]]) continue;   // (formed in double below)
-                if (!ok[u]) far = true;
-                reinterpret_cast<float2*>(fa)[at[u]] = mul_ff2(c.cff[k[u]], em[u]);
-                reinterpret_cast<float2*>(fb)[at[u]] = mul_ff2(c.cff[p.K + k[u]], em[u]);
-                reinterpret_cast<float2*>(fc)[at[u]] = ep[u];
+                const bool ok = within_30(it[u].arg);
+                float2 em, ep;
+                exp_pair_ff(ok ? it[u].arg : 0.0, reinterpret_cast<const float2*>(c.tab), em, ep);
+                if (!c.ff[it[u].k]) {
+                    rest = true;
+                    continue;
+                }
+                if (!ok) far = true;
+                reinterpret_cast<float2*>(fa)[it[u].at] = mul_ff2(c.cff[it[u].k], em);
+                reinterpret_cast<float2*>(fb)[it[u].at] = mul_ff2(c.cff[p.K + it[u].k], em);
+                reinterpret_cast<float2*>(fc)[it[u].at] = ep;
             }
         }
     }
-    for (int x = T - 1 - (int)threadIdx.x; x < n; x += T) {
-        const unsigned r = (unsigned)x >> sl;
-        const int kk = D == 1 ? (int)r : (int)__umulhi(r, p.d_magic), k = k0 + kk;
-        if (Tr::kBase == COS_MODE_FP32_MIXED && !in_double && c.ff[k]) continue;
-        const double arg = c.eps[k] * st[x - kk * DS];
-        double em, ep;
-        if constexpr (Tr::kBase == COS_MODE_FP32_MIXED) exp_pair(arg, p.exp_tab, em, ep);   // (rare: the table at hand is the other)
-        else exp_pair_at(arg, c.tab, em, ep);
-        const int at = (int)r * pitch + (x & (s - 1));
-        fa[at] = c.cf[k] * em;
-        fb[at] = c.cf[p.K + k] * em;
-        fc[at] = ep;
-    }
+    if (!rest) return far;
+    // (the same exponentials as above, one after another)
+    const int half = kMixed ? (n + 1) / 2 : n;
+    for (int x0 = T - 1 - (int)threadIdx.x; x0 < half; x0 += T)
+#pragma unroll 1
+        for (int x = x0; x < n; x += half) {
+            const unsigned r = (unsigned)x >> sl;
+            const int kk = D == 1 ? (int)r : (int)__umulhi(r, p.d_magic), k = k0 + kk;
+            if (kMixed && !in_double && c.ff[k]) continue;
+            const double arg = c.eps[k] * st[x - kk * DS];
+            double em, ep;
+            if constexpr (kMixed) exp_pair(arg, p.exp_tab, em, ep);   // (rare: the table at hand is the other)
+            else exp_pair_at(arg, c.tab, em, ep);
+            const int at = (int)r * pitch + (x & (s - 1));
+            fa[at] = c.cf[k] * em;
+            fb[at] = c.cf[p.K + k] * em;
+            fc[at] = ep;
+        }
     return far;
 }
 
@@ -291,34 +318,31 @@ __device__ __forceinline__ void chip_pairs(const ChipParams& p, unsigned char* s
 }
 
 // This thread's slots of the kinds [k0, k0 + kn): pieces x, x + T, ... below `end`, the
-// first kAhead descriptors loaded (ahead of the exponentials).
-constexpr int kAhead = 4;
+// next kAhead descriptors loaded (the first ahead of the exponentials).
+constexpr int kAhead = 2;
 struct SlotRange {
     int x, end;
     uint2 sd[kAhead];
-    __device__ __forceinline__ void load(const ChipParams& p, int pl) {
-#pragma unroll
-        for (int u = 0; u < kAhead; ++u)
-            if (x + u * (int)blockDim.x < end) sd[u] = __ldg(p.g.slots + ((x + u * (int)blockDim.x) >> pl));
-    }
     __device__ __forceinline__ void open(const ChipParams& p, int k0, int kn, int pl) {
         const bool all = kn == p.K;
         x = (all ? 0 : __ldg(p.kind_slot + k0) << pl) + (int)threadIdx.x;
         end = (all ? p.P : __ldg(p.kind_slot + k0 + kn)) << pl;
-        load(p, pl);
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+            if (x + u * (int)blockDim.x < end) sd[u] = __ldg(p.g.slots + ((x + u * (int)blockDim.x) >> pl));
     }
 };
 
-// V doubles from shared memory, two per access.
+// V doubles from shared memory, two per access, the second two `half` further.
 template <int V>
-__device__ __forceinline__ VecT<double, V> load_pair(const double* x) {
+__device__ __forceinline__ VecT<double, V> load_pair(const double* x, int half) {
     VecT<double, V> r;
     if constexpr (V == 1) {
         r.v[0] = x[0];
     } else {
 #pragma unroll
         for (int v = 0; v < V; v += 2) {
-            const double2 d = *reinterpret_cast<const double2*>(x + v);
+            const double2 d = *reinterpret_cast<const double2*>(x + (v ? half : 0));
             r.v[v] = d.x;
             r.v[v + 1] = d.y;
         }
@@ -346,36 +370,46 @@ __device__ __forceinline__ void chip_slots(const ChipParams& p, unsigned char* s
     const double* fc = fb + np;
     Prop* G = reinterpret_cast<Prop*>(sm + p.g_off);
     const int ahi = p.abs_weights ? 0x7fffffff : -1;
-    while (r.x < r.end) {
+    // a thread's samples: V = 4 takes two at smp and two half a row on, so that the threads
+    // of a row read 16 neighbouring bytes each (four in a row: two of eight threads in the
+    // same banks)
+    const int part = (int)threadIdx.x & ((1 << pl) - 1), smp = V == 4 ? part << 1 : part << VL, half = V == 4 ? 1 << (sl - 1) : 0;
+    fa += smp - k0 * D * pitch;
+    fb += smp - k0 * D * pitch;
+    fc += smp - k0 * D * pitch;
+    while (r.x < r.end) {   // (one copy of the code: unrolled, the warps wait for instructions)
+        const int x = r.x;
+        const uint2 d = r.sd[0];
 #pragma unroll
-        for (int u = 0; u < kAhead; ++u) {
-            const int x = r.x + u * T;
-            if (x >= r.end) break;
-            const uint2 sd = r.sd[u];
-            const int smp = (x & ((1 << pl) - 1)) << VL;
-            const unsigned ge = pair[sd.y & 0xffffu] >> smp;   // tau = t_i - t_j >= 0 ?
-            const int shi = (int)(sd.y & 0x80000000u);
-            const int xi = ((int)(sd.x & 0xffffu) - k0 * D) * pitch + smp;
-            const int xj = ((int)(sd.x >> 16) - k0 * D) * pitch + smp;
-            // V values of 8 bytes, aligned to 16 when there are more than one; neighbouring
-            // slots share (kind, i), so fetching both prefactors' rows costs few wavefronts
-            const VecT<double, V> vp = load_pair<V>(fa + xi), vn = load_pair<V>(fb + xi), ve = load_pair<V>(fc + xj);
-            VecT<Prop, V> out;
-            if (kMixed && !in_double && c.ff[(sd.y >> 16) & 0x7fff]) {
+        for (int u = 0; u + 1 < kAhead; ++u) r.sd[u] = r.sd[u + 1];
+        if (x + kAhead * T < r.end) r.sd[kAhead - 1] = __ldg(p.g.slots + ((x + kAhead * T) >> pl));
+        r.x += T;
+        unsigned ge = pair[d.y & 0xffffu] >> smp;   // tau = t_i - t_j >= 0 ?
+        if constexpr (V == 4) ge = (ge & 3u) | (ge >> half & 3u) << 2;
+        const int shi = (int)(d.y & 0x80000000u);
+        const int xi = (int)(d.x & 0xffffu) * pitch, xj = (int)(d.x >> 16) * pitch;
+        // V values of 8 bytes, aligned to 16 when there are more than one; neighbouring slots
+        // share (kind, i), so fetching both prefactors' rows costs few wavefronts
+        const VecT<double, V> vp = load_pair<V>(fa + xi, half), vn = load_pair<V>(fb + xi, half), ve = load_pair<V>(fc + xj, half);
+        VecT<Prop, V> out;
+        if (kMixed && !in_double && c.ff[(d.y >> 16) & 0x7fff]) {
 #pragma unroll
-                for (int v = 0; v < V; ++v) {
-                    const float g = mul_ff(as_ff((ge >> v) & 1u ? vp.v[v] : vn.v[v]), as_ff(ve.v[v]));
-                    out.v[v] = (Prop)__uint_as_float((__float_as_uint(g) ^ (unsigned)shi) & (unsigned)ahi);
-                }
-            } else {
-#pragma unroll
-                for (int v = 0; v < V; ++v)
-                    out.v[v] = (Prop)sign_ops(((ge >> v) & 1u ? vp.v[v] : vn.v[v]) * ve.v[v], shi, ahi);
+            for (int v = 0; v < V; ++v) {
+                const float g = mul_ff(as_ff((ge >> v) & 1u ? vp.v[v] : vn.v[v]), as_ff(ve.v[v]));
+                out.v[v] = (Prop)__uint_as_float((__float_as_uint(g) ^ (unsigned)shi) & (unsigned)ahi);
             }
-            *reinterpret_cast<VecT<Prop, V>*>(G + ((size_t)x << VL)) = out;
+        } else {
+#pragma unroll
+            for (int v = 0; v < V; ++v)
+                out.v[v] = (Prop)sign_ops(((ge >> v) & 1u ? vp.v[v] : vn.v[v]) * ve.v[v], shi, ahi);
         }
-        r.x += kAhead * T;
-        r.load(p, pl);
+        Prop* g = G + (((size_t)x - part) << VL) + smp;
+        if constexpr (V == 4) {
+            *reinterpret_cast<VecT<Prop, 2>*>(g) = VecT<Prop, 2>{{out.v[0], out.v[1]}};
+            *reinterpret_cast<VecT<Prop, 2>*>(g + half) = VecT<Prop, 2>{{out.v[2], out.v[3]}};
+        } else {
+            *reinterpret_cast<VecT<Prop, V>*>(g) = out;
+        }
     }
 }
 
@@ -699,6 +733,16 @@ __device__ __noinline__ void chip_mean(const ChipParams& p, int lane) {
 
 // ---------------------------------------------------------------- kernel
 
+// A float as a double, by 32-bit integer instructions but for subnormals, infinities and
+// NaN (a conversion takes as long as an FP64 operation, and the sink's in-edges are a
+// serial chain).
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+    if (e - 1u >= 254u && (u << 1) != 0) return (double)f;
+    const unsigned hi = (u & 0x80000000u) | (e ? ((u & 0x7fffffffu) >> 3) + (896u << 20) : 0u);
+    return __hiloint2double((int)hi, (int)(e ? u << 29 : 0u));
+}
+
 // Sink of chunk `chunk` by one warp: one lane per sample, in-edges in order; parents at
 // byte `base` of shared memory.
 template <int MODE>
@@ -719,8 +763,9 @@ __device__ __forceinline__ void chip_sink(const ChipParams& p, unsigned char* sm
         } else {
             const Prop g = reinterpret_cast<const Prop*>(G + (int)(m >> 16) * gb)[smp];
             if constexpr (Tr::kBase == COS_MODE_FP32_MIXED) {
-                acc += (double)pr[smp] * (double)g;   // exact product
-                if constexpr (Tr::kAbs) acca += (double)pr[s + smp] * (double)abs_to_float(g);
+                const double gd = widen(g);
+                acc = fma(widen(pr[smp]), gd, acc);   // exact product
+                if constexpr (Tr::kAbs) acca = fma(widen(pr[s + smp]), sign_ops(gd, 0, 0x7fffffff), acca);
             } else {
                 acc = madd(pr[smp], g, acc);
             }
@@ -773,17 +818,12 @@ __device__ __forceinline__ void chip_chunk(const ChipParams& p, int chunk, unsig
             const int kn = min(p.kinds_per_pass, p.K - k0);
             SlotRange range;
             range.open(p, k0, kn, p.s_log2 - (V == 4 ? 2 : V == 2 ? 1 : 0));
-            bool far = chip_exps<MODE>(p, sm, k0, kn, false);
-            if (k0 == 0) chip_pairs(p, sm);
-            if constexpr (kMixed) {
-                far = __syncthreads_or(far);
-                if (far) {
-                    chip_exps<MODE>(p, sm, k0, kn, true);
-                    __syncthreads();
-                }
-            } else {
+            bool far = !kMixed;
+            for (;;) {   // again in double, where a time lies too far outside [-beta, beta]
+                const bool again = chip_exps<MODE>(p, sm, k0, kn, far);
+                if (k0 == 0 && far == !kMixed) chip_pairs(p, sm);
+                if (!__syncthreads_or(again)) break;
                 far = true;
-                __syncthreads();
             }
             chip_slots<MODE, V>(p, sm, k0, kn, far, range);
             __syncthreads();   // the propagators are complete, the scratch is free

@@ -455,7 +455,7 @@ __device__ __forceinline__ float2 split_ff(double x) {
 // Product of two float-float numbers rounded to float: the exact leading product
 // hi*hi plus its rounding error (FMA) plus the cross terms, summed once.
 __device__ __forceinline__ float mul_ff(float2 a, float2 b) {
-    const float x = a.x * b.x;
+    const float x = __fmul_rn(a.x, b.x);   // (rounded: contracted into the sum below it would count its error twice)
     float e = fmaf(a.x, b.x, -x);
     e = fmaf(a.x, b.y, e);
     e = fmaf(a.y, b.x, e);
@@ -464,7 +464,7 @@ __device__ __forceinline__ float mul_ff(float2 a, float2 b) {
 
 // Float-float product of two float-float numbers (about 46 significant bits).
 __device__ __forceinline__ float2 mul_ff2(float2 a, float2 b) {
-    const float x = a.x * b.x;
+    const float x = __fmul_rn(a.x, b.x);   // (rounded: contracted into the sum below it would count its error twice)
     float e = fmaf(a.x, b.x, -x);
     e = fmaf(a.x, b.y, e);
     e = fmaf(a.y, b.x, e);
@@ -472,40 +472,52 @@ __device__ __forceinline__ float2 mul_ff2(float2 a, float2 b) {
     return make_float2(hi, e - (hi - x));
 }
 
-// 2^m * (hi, lo) by exponent arithmetic; hi must stay normal (the callers keep it
-// within 2^{+-100}); a lo that would leave the normal range becomes zero.
-__device__ __forceinline__ float2 ldexp_ff(float2 v, int m) {
-    const unsigned sh = (unsigned)m << 23;
-    const float hi = __uint_as_float(__float_as_uint(v.x) + sh);
-    const int elo = (int)((__float_as_uint(v.y) >> 23) & 0xffu) + m;
-    const float lo = (elo <= 0 || elo >= 255) ? 0.0f : __uint_as_float(__float_as_uint(v.y) + sh);
-    return make_float2(hi, lo);
+// The reduced argument of exp_pair_ff, x - n ln2/64 truncated to 24 bits, n != 0, |x| <= 30:
+// in fixed point with 70 fractional bits, modulo 2^-6, by 32-bit integer instructions.
+// (Two double FMAs, as before, occupy a quarter of an SM for 128 cycles per warp, twice the
+// issue slots of everything else here.)  ln2/64 = H 2^-38 + L 2^-70 to within 2^-72, so the
+// result is within 2^-59.5 of x - n ln2/64, where the rounding of x itself leaves 2^-49.
+__device__ __forceinline__ float reduced_argument(double x, int n) {
+    const unsigned H = 0xb17217f7u, L = 0xd1cf79acu;
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), na = (unsigned)abs(n);
+    const int sh = (int)((hi >> 20) & 0x7ffu) - 1005;   // 10 .. 22: |x| >= ln2/128
+    unsigned rh = __funnelshift_l(lo, (hi & 0xfffffu) | 0x100000u, sh) - na * H, rl = lo << sh;
+    asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %3;" : "+r"(rl), "+r"(rh) : "r"(na * L), "r"(__umulhi(na, L)));
+    const unsigned neg = (unsigned)((int)rh >> 31);
+    rl ^= neg;
+    rh ^= neg;
+    asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %2;" : "+r"(rl), "+r"(rh) : "r"(neg));
+    const bool top = rh != 0;
+    const int z = __clz((int)(top ? rh : rl));
+    const unsigned w = top ? __funnelshift_l(rl, rh, z) : rl << (z & 31);   // leading bit at 31
+    const unsigned mag = w ? ((unsigned)((top ? 120 : 88) - z) << 23) + ((w >> 8) & 0x7fffffu) : 0u;
+    return __uint_as_float(mag | ((hi ^ neg) & 0x80000000u));
 }
 
 // e^{-x} and e^{+x} as float-float values accurate to about 1e-10 relative, for
-// |x| <= 30: the reduction x = (64 m + j) ln2/64 + r is done in double (one rounding
-// of n, two FMAs), everything after it in FP32 -- r is below 0.0055, so its float
+// |x| <= 30: the reduction x = (64 m + j) ln2/64 + r is done to 2^-59 (see
+// reduced_argument), everything after it in FP32 -- r is below 0.0055, so its float
 // rounding and the float polynomial (even and odd parts through r^4 and r^3) change
 // e^{+-r} by less than 1e-9 relative; 2^{+-j/64} comes from a float-float table
 // `tff` ([0..63] = 2^{j/64}, [64..127] = 2^{-j/64}, each as (hi, lo)).
 __device__ __forceinline__ void exp_pair_ff(double x, const float2* __restrict__ tff, float2& em, float2& ep) {
-    const float nf = rintf(trunc_to_float(x) * 92.33248261689366f);
-    const double nd = float_to_double_exact(nf);   // (an integer: no conversion on the FP64 pipe)
-    double r = fma(-nd, 0.01083042469326756, x);
-    r = fma(-nd, 2.9815858269852933e-12, r);
+    const float xf = trunc_to_float(x);
+    const float nf = rintf(xf * 92.33248261689366f);
     const int n = (int)nf;
-    const float rf = trunc_to_float(r);
+    const float rf = n == 0 ? xf : reduced_argument(x, n);
     const float r2 = rf * rf;
-    const float even = r2 * fmaf(r2, 1.0f / 24.0f, 0.5f);
-    const float odd = rf * fmaf(r2, 1.0f / 6.0f, 1.0f);
+    const float ev = fmaf(r2, 1.0f / 24.0f, 0.5f), odd = __fmul_rn(rf, fmaf(r2, 1.0f / 6.0f, 1.0f));
     const int j = n & 63, m = n >> 6;
     const float2 tp = tff[j], tm = tff[64 + j];
     // T (1 + p) = T_hi + (T_lo + T_hi p), renormalised
-    const float pp = even + odd, pm = even - odd;
+    // (written out: left to the compiler, the contraction may differ from kernel to kernel)
+    const float pp = fmaf(r2, ev, odd), pm = fmaf(r2, ev, -odd);
     const float wp = fmaf(tp.x, pp, tp.y), wm = fmaf(tm.x, pm, tm.y);
     const float hp = tp.x + wp, hm = tm.x + wm;
-    ep = ldexp_ff(make_float2(hp, wp - (hp - tp.x)), m);
-    em = ldexp_ff(make_float2(hm, wm - (hm - tm.x)), -m);
+    // (|m| <= 44: exact)
+    const float up = __uint_as_float((unsigned)(127 + m) << 23), down = __uint_as_float((unsigned)(127 - m) << 23);
+    ep = make_float2(hp * up, (wp - (hp - tp.x)) * up);
+    em = make_float2(hm * down, (wm - (hm - tm.x)) * down);
 }
 
 // ---------------------------------------------------------------- phase: propagators
