@@ -433,7 +433,7 @@ __device__ __forceinline__ void chip_slots_table(const ChipParams& p, unsigned c
         const double tau = st[(i << sl) + smp] - st[(j << sl) + smp];
         const bool pos = tau >= 0.0;
         const double u = __dadd_rn(__dmul_rn(tau, p.ptab_inv_h), pos ? 0.0 : (double)PT);
-        int m = (int)u;
+        int m = max((int)u, 0);   // (NaN converts to the least integer)
         double f = __dsub_rn(u, (double)m);
         if (u < 0.0) {
             m = 0;

@@ -623,7 +623,7 @@ __device__ __forceinline__ void item_props(const WalkParams& p, const TileCtx& t
                     // grid coordinate: tau/h on the tau >= 0 half, (tau + tau_max)/h = tau/h + T
                     // below; every step rounded once (no contraction)
                     const double u = __dadd_rn(__dmul_rn(tau, p.ptab_inv_h), pos ? 0.0 : (double)T);
-                    int m = (int)u;
+                    int m = max((int)u, 0);   // (NaN converts to the least integer)
                     double f = __dsub_rn(u, (double)m);
                     if (u < 0.0) {   // before the grid: the first node's value
                         m = 0;
