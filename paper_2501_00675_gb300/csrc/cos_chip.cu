@@ -211,12 +211,6 @@ __device__ __forceinline__ void chip_times(const ChipParams& p, unsigned char* s
     }
 }
 
-// |x| <= 30 by 32-bit integer comparison (false for NaN).
-__device__ __forceinline__ bool within_30(double x) {
-    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
-    return hi < 0x403e0000u || (hi == 0x403e0000u && __double2loint(x) == 0);
-}
-
 // What bounds the propagators is the instructions of the exponentials (some 115 each, one of
 // them FP64; 38 % of the issue slots used) and fetching them: the loops have one copy of
 // their code, and a graph whose kinds need no double arithmetic never enters its loop.  Order
@@ -238,6 +232,7 @@ __device__ __forceinline__ bool chip_exps(const ChipParams& p, unsigned char* sm
     double* fc = fb + np;                                                           // e^{+eps t}
     const int T = blockDim.x;
     constexpr bool kMixed = Tr::kBase == COS_MODE_FP32_MIXED;
+    const FmaConst fma_ = fma_const(p.D);
     bool far = false, rest = true;   // rest: this thread has exponentials to form in double
     if (kMixed && !in_double) {
         rest = false;
@@ -291,13 +286,13 @@ __device__ __forceinline__ bool chip_exps(const ChipParams& p, unsigned char* sm
             const unsigned r = (unsigned)x >> sl;
             const int kk = D == 1 ? (int)r : (int)__umulhi(r, p.d_magic), k = k0 + kk;
             if (kMixed && !in_double && c.ff[k]) continue;
-            const double arg = c.eps[k] * st[x - kk * DS];
+            const double arg = fma_.mul(c.eps[k], st[x - kk * DS]);
             double em, ep;
-            if constexpr (kMixed) exp_pair(arg, p.exp_tab, em, ep);   // (rare: the table at hand is the other)
-            else exp_pair_at(arg, c.tab, em, ep);
+            if constexpr (kMixed) exp_pair(arg, p.exp_tab, fma_, em, ep);   // (rare: the table at hand is the other)
+            else exp_pair_at(arg, c.tab, fma_, em, ep);
             const int at = (int)r * pitch + (x & (s - 1));
-            fa[at] = c.cf[k] * em;
-            fb[at] = c.cf[p.K + k] * em;
+            fa[at] = fma_.mul(c.cf[k], em);
+            fb[at] = fma_.mul(c.cf[p.K + k], em);
             fc[at] = ep;
         }
     return far;
@@ -363,6 +358,7 @@ __device__ __forceinline__ void chip_slots(const ChipParams& p, unsigned char* s
     constexpr int VL = V == 4 ? 2 : V == 2 ? 1 : 0;
     const int sl = p.s_log2, D = p.D, pitch = chip_pitch(1 << sl), np = kn * D * pitch;
     const int pl = sl - VL, T = blockDim.x;   // pl: log2 pieces per slot
+    const FmaConst fma_ = fma_const(p.D);
     const Consts c(sm, p.coef_off, p.K);
     const unsigned* pair = reinterpret_cast<const unsigned*>(sm + kScratchAt);
     const double* fa = reinterpret_cast<const double*>(sm + kScratchAt + chip_pair_bytes(D));
@@ -401,7 +397,7 @@ __device__ __forceinline__ void chip_slots(const ChipParams& p, unsigned char* s
         } else {
 #pragma unroll
             for (int v = 0; v < V; ++v)
-                out.v[v] = (Prop)sign_ops(((ge >> v) & 1u ? vp.v[v] : vn.v[v]) * ve.v[v], shi, ahi);
+                out.v[v] = (Prop)sign_ops(fma_.mul((ge >> v) & 1u ? vp.v[v] : vn.v[v], ve.v[v]), shi, ahi);
         }
         Prop* g = G + (((size_t)x - part) << VL) + smp;
         if constexpr (V == 4) {
@@ -418,6 +414,7 @@ template <int MODE>
 __device__ __forceinline__ void chip_slots_table(const ChipParams& p, unsigned char* sm) {
     using Prop = typename Traits<MODE>::Prop;
     const int sl = p.s_log2, D = p.D, PT = p.ptab_T, n = p.P << sl, T = blockDim.x;
+    const FmaConst fc = fma_const(p.D);
     const double* st = reinterpret_cast<const double*>(sm + p.times_off);
     Prop* G = reinterpret_cast<Prop*>(sm + p.g_off);
     const int ahi = p.abs_weights ? 0x7fffffff : -1;
@@ -430,20 +427,7 @@ __device__ __forceinline__ void chip_slots_table(const ChipParams& p, unsigned c
         const int k = (sd.y >> 16) & 0x7fff, i = (int)(sd.x & 0xffffu) - k * D, j = (int)(sd.x >> 16) - k * D;
         const int shi = (int)(sd.y & 0x80000000u);
         const double2* tk = reinterpret_cast<const double2*>(p.ptab) + (int64_t)k * 2 * PT;
-        const double tau = st[(i << sl) + smp] - st[(j << sl) + smp];
-        const bool pos = tau >= 0.0;
-        const double u = __dadd_rn(__dmul_rn(tau, p.ptab_inv_h), pos ? 0.0 : (double)PT);
-        int m = max((int)u, 0);   // (NaN converts to the least integer)
-        double f = __dsub_rn(u, (double)m);
-        if (u < 0.0) {
-            m = 0;
-            f = 0.0;
-        } else if (m >= PT) {
-            m = PT - 1;
-            f = 1.0;
-        }
-        const double2 as = __ldg(tk + (pos ? 0 : PT) + m);
-        G[x] = (Prop)sign_ops(__dadd_rn(as.x, __dmul_rn(f, as.y)), shi, ahi);
+        G[x] = (Prop)sign_ops(table_value(st[(i << sl) + smp], st[(j << sl) + smp], tk, PT, p.ptab_inv_h, fc), shi, ahi);
         x += T;
         sd = next;
     }

@@ -151,6 +151,7 @@ struct cos_graph {
     double* d_ptab = nullptr;       // user-tabulated propagators [K][2][ptab_T+1], or none
     int32_t ptab_T = 0;
     double ptab_tau_max = 0.0;
+    bool capturing = false;         // during cos_evaluate: its stream is being captured
     int last_wave = 0;              // the last evaluate ran the windowed schedule
     // page-locked (mean R, mean A), written by the on-chip walk of a call that waits for its
     // mean: reading the control block takes a copy after the kernel (nullptr: no such memory)
@@ -626,9 +627,16 @@ static int resolve_tuning(cos_graph_t g, int kmode, cos_tuning* out, int64_t* ti
     // (with the FP32 work-queue walker at four CTAs per SM the FP32 walk of medium graphs
     // joined the FP64 one there: medium mixed 2.44 -> 2.36 ms; the level-synchronous
     // walker with six edges in flight per warp later matched it, 2.36 ms)
-    const bool big = (double)g->E * (double)g->S >= 1e9;
+    const double work = (double)g->E * (double)g->S;
+    const bool big = work >= 1e9;
+    // With tabulated propagators in FP64 the work queue, whose kernel has the registers for
+    // their integer arithmetic (see item_props), is ahead from fewer samples on: medium
+    // graph, level-synchronous / work queue, 4,096 samples (1.9e8) 630 / 660 us, 8,192 1,106 /
+    // 1,007, 16,384 2,063 / 1,865; 100,000 nodes, 1,024 (2.6e8) 853 / 870, 2,048 1,454 / 1,302.
+    // Not on a capturing stream, which the work queue's uploads do not suit.
+    const bool tables = g->d_ptab && kmode == COS_MODE_FP64 && work >= 3e8 && !g->capturing;
     if (t.schedule <= 0)
-        t.schedule = ((big && (mode == COS_MODE_FP64 || mode == COS_MODE_FP32_MIXED)) || g->Wmax >= 65536) ? 2 : 1;
+        t.schedule = ((big && (mode == COS_MODE_FP64 || mode == COS_MODE_FP32_MIXED)) || tables || g->Wmax >= 65536) ? 2 : 1;
     // level-synchronous: 8 rows per warp measured best for the FP32 walk (medium: 2.46 ms
     // against 2.50 with 16 and 2.88 with 31)
     if (t.rows_per_warp <= 0) {
@@ -981,7 +989,10 @@ int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean
     }
     WalkParams p;
     cos_tuning tn;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    g->capturing = g->d_ptab && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
     int rc = cosgpu::prepare_walk(g, km, nullptr, per_sample_out, &p, &tn);
+    g->capturing = false;
     if (rc != COS_OK) return rc;
     if (const char* env = getenv("COS_TEST_SKIP_BARRIER_PHASE")) p.skip_barrier_phase = atoi(env);
     if (g->d_trace) {

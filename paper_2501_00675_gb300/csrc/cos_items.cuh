@@ -389,40 +389,19 @@ __device__ __forceinline__ void item_coef(const WalkParams& p) {
 
 // ---------------------------------------------------------------- exponentials
 
-// e^{-x} and e^{+x} in double precision for |x| <= 708, by the table-driven method of
-// P. T. P. Tang (ACM TOMS 15, 1989): x = (64 m + j) ln2/64 + r with |r| <= ln2/128,
-// e^{+-x} = 2^{+-m} 2^{+-j/64} e^{+-r}; e^{+-r} = 1 + E +- O with the even and odd parts
-// of the Taylor series through r^5 (truncation below 4e-17 relative).  The 64 values
-// 2^{j/64} (and 2^{-j/64}) are read from `tab` ([0..63] = 2^{j/64}, [64..127] = 2^{-j/64}).
-__device__ __forceinline__ void exp_pair_from(double x, const double* tab, bool ldg, double& em, double& ep) {
-    const double inv = 92.33248261689366;                  // 64 / ln 2 (only rounds n)
-    const double c_hi = 0.01083042469326756;               // ln2/64 to 32 significant bits: n*c_hi is exact
-    const double c_lo = 2.9815858269852933e-12;            // ln2/64 - c_hi
-    const double nd = rint(x * inv);
-    const int n = (int)nd;
-    double r = fma(-nd, c_hi, x);
-    r = fma(-nd, c_lo, r);
-    const double r2 = r * r;
-    const double even = r2 * fma(r2, fma(r2, 1.0 / 720.0, 1.0 / 24.0), 0.5);      // cosh(r) - 1
-    const double odd = r * fma(r2, fma(r2, 1.0 / 120.0, 1.0 / 6.0), 1.0);         // sinh(r)
-    const int j = n & 63;
-    const int m = n >> 6;                                                       // floor(n / 64)
-    // e^{+x} = 2^m 2^{j/64} (1 + even + odd);  e^{-x} = 2^{-m} 2^{-j/64} (1 + even - odd)
-    const double tp = ldg ? __ldg(tab + j) : tab[j], tm = ldg ? __ldg(tab + 64 + j) : tab[64 + j];
-    const double vp = fma(tp, even + odd, tp);
-    const double vm = fma(tm, even - odd, tm);
-    ep = __hiloint2double(__double2hiint(vp) + (m << 20), __double2loint(vp));
-    em = __hiloint2double(__double2hiint(vm) - (m << 20), __double2loint(vm));
+// Products and sums of doubles as fused multiply-adds, with the same results: the FP64 pipe
+// takes 2.0 fused operations per cycle and SM, but only 1.68 plain additions or
+// multiplications.  The constants come from the kernel's parameters, or the compiler would
+// write the plain operations again.
+struct FmaConst {
+    double zero, one;   // -0.0 and 1.0
+    __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, zero); }
+    __device__ __forceinline__ double add(double a, double b) const { return fma(a, one, b); }
+};
+// x: any parameter that is never negative
+__device__ __forceinline__ FmaConst fma_const(int x) {
+    return FmaConst{__hiloint2double((int)0x80000000 ^ (x >> 31), 0), __hiloint2double(0x3ff00000 ^ (x >> 31), 0)};
 }
-__device__ __forceinline__ void exp_pair(double x, const double* __restrict__ tab, double& em, double& ep) {
-    exp_pair_from(x, tab, true, em, ep);
-}
-// The table in shared memory.
-__device__ __forceinline__ void exp_pair_at(double x, const double* tab, double& em, double& ep) {
-    exp_pair_from(x, tab, false, em, ep);
-}
-
-// ---------------------------------------------------------------- float-float helpers
 
 // Leading 24 significant bits of a double as a float, by truncation with 32-bit
 // integer operations on the double's two halves only (no FP64 conversion; 64-bit
@@ -445,6 +424,97 @@ __device__ __forceinline__ double float_to_double_exact(float f) {
     const unsigned hi = (u & 0x80000000u) | ((e - 127u + 1023u) << 20) | ((u & 0x7fffffu) >> 3);
     return __hiloint2double((int)hi, (int)((u & 0x7u) << 29));
 }
+
+// e^{-x} and e^{+x} in double precision for |x| <= 708, by the table-driven method of
+// P. T. P. Tang (ACM TOMS 15, 1989): x = (64 m + j) ln2/64 + r with |r| <= ln2/128,
+// e^{+-x} = 2^{+-m} 2^{+-j/64} e^{+-r}; e^{+-r} = 1 + E +- O with the even and odd parts
+// of the Taylor series through r^5 (truncation below 4e-17 relative).  The 64 values
+// 2^{j/64} (and 2^{-j/64}) are read from `tab` ([0..63] = 2^{j/64}, [64..127] = 2^{-j/64}).
+// The nearest n is found in FP32 (|r| may exceed ln2/128 by 2^-9 of it), so that of the
+// 16 FP64 operations a pair took, two prefactors included, three conversions and roundings
+// are gone and the others are fused ones.
+__device__ __forceinline__ void exp_pair_from(double x, const double* tab, bool ldg, const FmaConst& f, double& em, double& ep) {
+    const double c_hi = 0.01083042469326756;               // ln2/64 to 32 significant bits: n*c_hi is exact
+    const double c_lo = 2.9815858269852933e-12;            // ln2/64 - c_hi
+    const bool finite = ((unsigned)__double2hiint(x) & 0x7fffffffu) < 0x7ff00000u;
+    const float nf = rintf(trunc_to_float(x) * 92.33248261689366f);   // 64 / ln 2
+    const double nd = finite ? float_to_double_exact(nf) : x;
+    const int n = finite ? (int)nf : 0;
+    double r = fma(-nd, c_hi, x);
+    r = fma(-nd, c_lo, r);
+    const double r2 = f.mul(r, r);
+    const double ev = fma(r2, fma(r2, 1.0 / 720.0, 1.0 / 24.0), 0.5);
+    const double odd = f.mul(r, fma(r2, fma(r2, 1.0 / 120.0, 1.0 / 6.0), 1.0));   // sinh(r)
+    const double pp = fma(r2, ev, odd), pm = fma(r2, ev, -odd);                   // cosh(r) - 1 +- sinh(r)
+    const int j = n & 63;
+    const int m = n >> 6;                                                       // floor(n / 64)
+    // e^{+x} = 2^m 2^{j/64} (1 + even + odd);  e^{-x} = 2^{-m} 2^{-j/64} (1 + even - odd)
+    const double tp = ldg ? __ldg(tab + j) : tab[j], tm = ldg ? __ldg(tab + 64 + j) : tab[64 + j];
+    const double vp = fma(tp, pp, tp);
+    const double vm = fma(tm, pm, tm);
+    ep = __hiloint2double(__double2hiint(vp) + (m << 20), __double2loint(vp));
+    em = __hiloint2double(__double2hiint(vm) - (m << 20), __double2loint(vm));
+}
+__device__ __forceinline__ void exp_pair(double x, const double* __restrict__ tab, const FmaConst& f, double& em, double& ep) {
+    exp_pair_from(x, tab, true, f, em, ep);
+}
+// The table in shared memory.
+__device__ __forceinline__ void exp_pair_at(double x, const double* tab, const FmaConst& f, double& em, double& ep) {
+    exp_pair_from(x, tab, false, f, em, ep);
+}
+
+// |x| <= 30 by 32-bit integer comparison (false for NaN): a comparison of doubles
+// occupies the FP64 pipe.
+__device__ __forceinline__ bool within_30(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    return hi < 0x403e0000u || (hi == 0x403e0000u && __double2loint(x) == 0);
+}
+
+// Integer part (below 2^21) of u >= 1 and, exactly, the rest, by 32-bit instructions.
+__device__ __forceinline__ int split_integer(double u, double& frac) {
+    const unsigned hi = (unsigned)__double2hiint(u), lo = (unsigned)__double2loint(u);
+    const int e = (int)(hi >> 20), sh = 20 - (e - 1023);   // places of the high word behind the point
+    const unsigned mant = (hi & 0xfffffu) | 0x100000u, fh = mant & ((1u << sh) - 1u);
+    const int k = fh ? __clz((int)fh) - 11 : 21 + __clz((int)lo);   // to the left, for a leading bit at 20
+    const unsigned nh = k < 32 ? __funnelshift_l(lo, fh, k) : lo << (k - 32), nl = k < 32 ? lo << (k & 31) : 0u;
+    frac = (fh | lo) ? __hiloint2double((int)(((unsigned)(e - k) << 20) + (nh & 0xfffffu)), (int)nl) : 0.0;
+    return (int)(mant >> sh);
+}
+
+// User-tabulated G_k(t_i - t_j): linear interpolation on the half of the table that the sign
+// of tau selects (tau = 0 takes the tau >= 0 half), in double, every step rounded once; end
+// values outside the grid.  tk: (a_m, slope_m) of the kind, the tau >= 0 half first.  What
+// bounds it is the FP64 pipe: five fused operations (two sums, three products as they were;
+// the two conversions and two comparisons besides are integer work now).
+__device__ __forceinline__ double table_value(double ti, double tj, const double2* tk, int T, double inv_h, const FmaConst& c) {
+    const double tau = c.add(ti, -tj);
+    const int th = __double2hiint(tau);
+    const unsigned ta = (unsigned)th & 0x7fffffffu;
+    const bool nan_tau = ta > 0x7ff00000u || (ta == 0x7ff00000u && __double2loint(tau) != 0);
+    const bool pos = !nan_tau && (th >= 0 || (ta == 0 && __double2loint(tau) == 0));   // tau >= 0
+    // grid coordinate: tau/h on the tau >= 0 half, (tau + tau_max)/h = tau/h + T below
+    const double u = c.add(c.mul(tau, inv_h), pos ? 0.0 : (double)T);
+    const unsigned uh = (unsigned)__double2hiint(u);
+    int m = 0;
+    double f = u;                                  // below the second node
+    if (uh >= 0x80000000u) {                       // before the grid: the first node's value
+        const unsigned ua = uh & 0x7fffffffu;
+        if (!(ua > 0x7ff00000u || (ua == 0x7ff00000u && __double2loint(u) != 0))) f = 0.0;
+    } else if (uh >= (1023u + 21u) << 20) {        // 2^21 nodes or more, infinite or NaN
+        m = max((int)u, 0);                        // (NaN converts to the least integer)
+        f = __dsub_rn(u, (double)m);
+    } else if (uh >= 1023u << 20) {
+        m = split_integer(u, f);
+    }
+    if (m >= T) {                                  // at or past the last node: its value
+        m = T - 1;
+        f = 1.0;
+    }
+    const double2 as = __ldg(tk + (pos ? 0 : T) + m);
+    return c.add(c.mul(f, as.y), as.x);
+}
+
+// ---------------------------------------------------------------- float-float helpers
 
 // x = hi + lo with hi, lo floats (about 48 significant bits), one DADD.
 __device__ __forceinline__ float2 split_ff(double x) {
@@ -577,7 +647,10 @@ __host__ __device__ constexpr int prop_smem_bytes(int D, int chv) { return 4 * 8
 // fermion-loop edge, whose factor is negated.  The first kind also writes the
 // chunk's root values (node 0 holds 1, Fig. 1 caption).  The chunk's samples are
 // taken in passes of at most 64 (the shared memory holds one pass).
-template <int MODE, int CHV>
+// PLAIN_TABLE: tabulated propagators by plain conversions and comparisons (same numbers).  The
+// level-synchronous kernel has no registers left for the integer work of table_value: with it
+// its FP64 walk takes 5 % longer (medium graph, 16,384 samples: 1.66 / 1.75 ms), tables or not.
+template <int MODE, int CHV, bool PLAIN_TABLE = false>
 __device__ __forceinline__ void item_props(const WalkParams& p, const TileCtx& tc, int item, double* sm) {
     using Tr = Traits<MODE>;
     using Prop = typename Tr::Prop;
@@ -594,15 +667,14 @@ __device__ __forceinline__ void item_props(const WalkParams& p, const TileCtx& t
         }
     if constexpr (!Tr::kCount) {
         const int D = p.D;
+        const FmaConst fc = fma_const(p.D);
         const double eps = p.eps[k], cpos = p.coef[k], cneg = p.coef[p.K + k];
         const int q0 = __ldg(p.kind_slot + k), q1 = __ldg(p.kind_slot + k + 1);
         for (int h0 = 0; h0 < CHV; h0 += PCH) {   // pass: samples [h0, h0 + PCH) of the chunk
         const int64_t s0 = tc.base + (int64_t)c * CHV + h0;
         Prop* gt = static_cast<Prop*>(p.gtab) + (int64_t)c * p.P * CHV + h0;
         if (p.ptab) {
-            // user-tabulated G_k: linear interpolation on the half of the table that
-            // the sign of tau selects (tau = 0 takes the tau >= 0 half), in double,
-            // rounded once to the propagator type; end values outside the grid
+            // user-tabulated G_k, rounded once to the propagator type
             double* st = sm;   // [D][PCH] times
             for (int x = threadIdx.x; x < PCH * D; x += blockDim.x) {
                 const int i = x / PCH, s = x - i * PCH;
@@ -618,22 +690,29 @@ __device__ __forceinline__ void item_props(const WalkParams& p, const TileCtx& t
                 const int ahi = p.abs_weights ? 0x7fffffff : -1;            // |G| for A(s)
 #pragma unroll
                 for (int v = 0; v < PCH / 32; ++v) {
-                    const double tau = st[i * PCH + v * 32 + lane] - st[j * PCH + v * 32 + lane];
-                    const bool pos = tau >= 0.0;
-                    // grid coordinate: tau/h on the tau >= 0 half, (tau + tau_max)/h = tau/h + T
-                    // below; every step rounded once (no contraction)
-                    const double u = __dadd_rn(__dmul_rn(tau, p.ptab_inv_h), pos ? 0.0 : (double)T);
-                    int m = max((int)u, 0);   // (NaN converts to the least integer)
-                    double f = __dsub_rn(u, (double)m);
-                    if (u < 0.0) {   // before the grid: the first node's value
-                        m = 0;
-                        f = 0.0;
-                    } else if (m >= T) {   // at or past the last node: its value
-                        m = T - 1;
-                        f = 1.0;
+                    const double ti = st[i * PCH + v * 32 + lane], tj = st[j * PCH + v * 32 + lane];
+                    double g;
+                    if constexpr (PLAIN_TABLE) {
+                        const double tau = ti - tj;
+                        const bool pos = tau >= 0.0;
+                        // grid coordinate: tau/h on the tau >= 0 half, (tau + tau_max)/h = tau/h + T
+                        // below; every step rounded once (no contraction)
+                        const double u = __dadd_rn(__dmul_rn(tau, p.ptab_inv_h), pos ? 0.0 : (double)T);
+                        int m = max((int)u, 0);   // (NaN converts to the least integer)
+                        double f = __dsub_rn(u, (double)m);
+                        if (u < 0.0) {   // before the grid: the first node's value
+                            m = 0;
+                            f = 0.0;
+                        } else if (m >= T) {   // at or past the last node: its value
+                            m = T - 1;
+                            f = 1.0;
+                        }
+                        const double2 as = __ldg(tk + (pos ? 0 : T) + m);
+                        g = __dadd_rn(as.x, __dmul_rn(f, as.y));
+                    } else {
+                        g = table_value(ti, tj, tk, T, p.ptab_inv_h, fc);
                     }
-                    const double2 as = __ldg(tk + (pos ? 0 : T) + m);
-                    const double g = sign_ops(__dadd_rn(as.x, __dmul_rn(f, as.y)), shi, ahi);
+                    g = sign_ops(g, shi, ahi);
                     __stcg(gt + (int64_t)q * CHV + v * 32 + lane, (Prop)g);
                 }
             }
@@ -658,7 +737,7 @@ __device__ __forceinline__ void item_props(const WalkParams& p, const TileCtx& t
                 const int i = x / PCH, s = x - i * PCH;
                 const double t = p.t[(int64_t)i * p.t_ld + s0 + s];
                 const double arg = eps * t;
-                if (!(fabs(arg) <= 30.0)) {
+                if (!within_30(arg)) {
                     out_of_range = true;
                     continue;
                 }
@@ -695,10 +774,10 @@ __device__ __forceinline__ void item_props(const WalkParams& p, const TileCtx& t
                 const int i = x / PCH, s = x - i * PCH;
                 const double t = p.t[(int64_t)i * p.t_ld + s0 + s];
                 double em, ep;
-                exp_pair(eps * t, p.exp_tab, em, ep);
+                exp_pair(fc.mul(eps, t), p.exp_tab, fc, em, ep);
                 sk[x] = time_order_key(t);
-                sp[x] = cpos * em;
-                sn[x] = cneg * em;
+                sp[x] = fc.mul(cpos, em);
+                sn[x] = fc.mul(cneg, em);
                 se[x] = ep;
             }
             __syncthreads();
@@ -712,7 +791,7 @@ __device__ __forceinline__ void item_props(const WalkParams& p, const TileCtx& t
                 for (int v = 0; v < PCH / 32; ++v) {
                     const int xi = i * PCH + v * 32 + lane, xj = j * PCH + v * 32 + lane;
                     const double a = key_ge(sk[xi], sk[xj]) ? sp[xi] : sn[xi];   // tau = t_i - t_j >= 0 ?
-                    const double g = sign_ops(a * se[xj], shi, ahi);
+                    const double g = sign_ops(fc.mul(a, se[xj]), shi, ahi);
                     __stcg(gt + (int64_t)q * CHV + v * 32 + lane, (Prop)g);
                 }
             }

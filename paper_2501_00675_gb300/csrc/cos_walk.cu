@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kThreads, min_blocks<MODE, V, LAYOUT>()) walk_
     for (int64_t tix = 0; tix < ntiles; ++tix) {
         const TileCtx tc = tile_ctx<CHV>(p, tix);
         const int np = prop_items<MODE>(p, tc);
-        for (int it = blockIdx.x; it < np; it += gridDim.x) item_props<MODE, CHV>(p, tc, it, smem);
+        for (int it = blockIdx.x; it < np; it += gridDim.x) item_props<MODE, CHV, true>(p, tc, it, smem);
         if (!grid_sync(p, epoch, 2)) return;
         for (int l = 1; l < p.L; ++l) {
             const int n = level_items(p, p.levels[l], tc);
@@ -160,7 +160,7 @@ __global__ void exp_pair_kernel(const double* __restrict__ x, int64_t n, const d
                                 double* __restrict__ em, double* __restrict__ ep) {
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
         double a, b;
-        exp_pair(x[q], tab, a, b);
+        exp_pair(x[q], tab, fma_const((int)gridDim.x), a, b);
         em[q] = a;
         ep[q] = b;
     }
