@@ -144,7 +144,7 @@ struct ChipArgs {
     unsigned* ticket;
     unsigned* exits;          // CTAs that have left (zero between launches)
     int n, total;
-    int tmem_cols;
+    int tmem_cols;            // 0: no level goes through TMEM
     int few;                  // so few blocks of samples that the last CTA sums them all
 };
 
@@ -699,7 +699,7 @@ __device__ __noinline__ void chip_mean(const ChipParams& p, int lane) {
     partials_sum(p.partials, nblk, lane, sum, comp);
     if constexpr (Traits<MODE>::kAbs) partials_sum(p.partials_abs, nblk, lane, sa, ca);
     if (lane == 0) {
-        const double mean = (sum + comp) / (double)p.S, mean_abs = (sa + ca) / (double)p.S;
+        const double mean = (sum + comp) / (double)p.S, mean_abs = Traits<MODE>::kAbs ? (sa + ca) / (double)p.S : 0.0;
         p.ctrl->sum = sum;
         p.ctrl->comp = comp;
         p.ctrl->mean = mean;
@@ -936,10 +936,10 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
     __shared__ int s_last;
     __shared__ ChipParams s_p;
     const int warp = threadIdx.x >> 5;
-    if (warp == 0) tmem_alloc(&s_tmem, (unsigned)a.tmem_cols);
+    if (warp == 0 && a.tmem_cols) tmem_alloc(&s_tmem, (unsigned)a.tmem_cols);
     if (a.list && threadIdx.x == 0) s_next[0] = (int)atomicAdd(a.ticket, 1u);
     __syncthreads();
-    const unsigned base = s_tmem;
+    const unsigned base = a.tmem_cols ? s_tmem : 0u;
     // a warp reaches the TMEM lanes of its number mod 4; the warps that share them take
     // 128 columns each
     const unsigned tmem = base + ((unsigned)(warp & 3) << 21) + (unsigned)(warp >> 2) * 128u;
@@ -993,9 +993,10 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(a.exits, 1u) + 1u == gridDim.x;
-        __threadfence();
+        // (one atomic with both orders: between two fences it took 1,000 cycles longer)
+        unsigned before;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(a.exits) : "memory");
+        s_last = before + 1u == gridDim.x;
     }
     __syncthreads();
     if (s_last) {   // every other CTA has counted its chunks in and left
@@ -1009,7 +1010,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
         if (threadIdx.x == 0) *a.exits = 0;
     }
     __syncthreads();
-    if (warp == 0) tmem_dealloc(base, (unsigned)a.tmem_cols);
+    if (warp == 0 && a.tmem_cols) tmem_dealloc(base, (unsigned)a.tmem_cols);
 }
 
 template <int MODE, int LB>
@@ -1174,13 +1175,13 @@ namespace {
 // Blocks of samples up to which the last CTA sums them all, two rounds of its teams.
 int few_blocks(int threads) { return 2 * (threads / 128); }
 
-int launch(int kmode, int lane_bytes, int threads, int smem, ChipArgs& a, int chunks, int sms, cudaStream_t st) {
+int launch(int kmode, int lane_bytes, int threads, int smem, bool staged, ChipArgs& a, int chunks, int sms, cudaStream_t st) {
     const void* k = select_chip(kmode, lane_bytes);
     if (!k) return set_error(COS_ERR_INVALID, "no on-chip kernel for mode %d, %d bytes per lane", kmode, lane_bytes);
     // (always the same limit: calls of other threads may come between this one and the launch)
     if (prepare_kernel_attrs(k, smem_limit(1)) != COS_OK) return set_error(COS_ERR_CUDA, "cannot set dynamic shared memory");
     const int ctas = 512 / threads;
-    a.tmem_cols = 512 / ctas;
+    a.tmem_cols = staged ? 512 / ctas : 0;
     void* args[] = {&a};
     const int grid = std::min(chunks, sms * ctas);
     const cudaError_t e = cudaLaunchKernel(k, dim3((unsigned)grid), dim3((unsigned)threads), args, (size_t)smem, st);
@@ -1199,7 +1200,9 @@ int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, c
     const int64_t blocks = (p.S + kReduceBlock - 1) / kReduceBlock;
     a.exits = p.arrive + blocks;
     a.few = blocks <= few_blocks(plan.threads);
-    return launch(kmode, plan.lane_bytes, plan.threads, plan.smem, a, p.nchunks, sms, st);
+    // with room for any two levels none goes through TMEM, whose allocation takes 700 cycles
+    const bool staged = p.lev_bytes < 2 * round128(((int64_t)p.g.max_width + 1) << p.rb_log2);
+    return launch(kmode, plan.lane_bytes, plan.threads, plan.smem, staged, a, p.nchunks, sms, st);
 }
 
 int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const ChipParams* list, int n, int total,
@@ -1210,7 +1213,7 @@ int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const Chi
     a.n = n;
     a.total = total;
     a.ticket = ticket;
-    return launch(kmode, lane_bytes, threads, smem, a, total, sms, st);
+    return launch(kmode, lane_bytes, threads, smem, true, a, total, sms, st);
 }
 
 }  // namespace cosgpu
