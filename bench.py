@@ -320,6 +320,8 @@ def run_ours(args, rank, world, local):
     gr.get_result(stream)
     torch.cuda.synchronize()
     tuning = gr.get_tuning(emode)
+    # (the profiled DRAM traffic is the workspace kernels'; the on-chip walk has next to none)
+    on_chip = bool(gr.info()["on_chip"] >> (4 if mode == 1 and args.abs else mode) & 1) and not (mode == 0 and args.abs)
 
     uuid = None
     try:
@@ -360,8 +362,9 @@ def run_ours(args, rank, world, local):
     hbm = {"bound": "hbm", "achieved": alg_bytes / walk_s / 1e9, "peak": peak, "unit": "GB/s",
            "frac": alg_bytes / walk_s / 1e9 / peak, "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)"
            if peak_kind == "measured" else "fallback 6.8 TB/s",
-           "traffic": profiled_traffic(f"walk_{mode_name}{'_abs' if args.abs else ''}_{args.workload}",
-                                       S, tuning["schedule"], tuning["layout"]),
+           "traffic": None if on_chip else
+           profiled_traffic(f"walk_{mode_name}{'_abs' if args.abs else ''}_{args.workload}",
+                            S, tuning["schedule"], tuning["layout"]),
            "algorithmic_bytes_per_launch": alg_bytes}
     if mode == 0:
         tflops = 2.0 * E * S / walk_s / 1e12

@@ -215,9 +215,10 @@ class Graph:
         return self._h.value
 
     def info(self) -> dict:
-        arr = np.zeros(10, dtype=np.int64)
-        _check(load_library().cos_graph_info(self._h, _ptr(arr), 10))
-        keys = ["L", "N", "E", "P", "W_max", "count", "count_overflow", "K", "D", "device"]
+        arr = np.zeros(11, dtype=np.int64)
+        _check(load_library().cos_graph_info(self._h, _ptr(arr), 11))
+        # on_chip: bit k set when kernel mode k (4: FP32 mixed with A) runs on chip now
+        keys = ["L", "N", "E", "P", "W_max", "count", "count_overflow", "K", "D", "device", "on_chip"]
         return {k: int(v) for k, v in zip(keys, arr)}
 
     def set_samples(self, t, eps, beta: float, t_flags: int, num_samples: Optional[int] = None, stream=None):

@@ -47,8 +47,11 @@ namespace {
 // ---------------------------------------------------------------- tensor memory
 
 __device__ __forceinline__ void tmem_alloc(unsigned* smem_dst, unsigned cols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)), "r"(cols)
-                 : "memory");
+    if (cols)
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)), "r"(cols)
+                     : "memory");
+    // (also by a CTA that allocates nothing: while one holds the permit, no second CTA of the
+    // kernel runs on its SM -- order 2, two CTAs per SM: 66 / 105 us)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void tmem_dealloc(unsigned addr, unsigned cols) {
@@ -936,7 +939,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
     __shared__ int s_last;
     __shared__ ChipParams s_p;
     const int warp = threadIdx.x >> 5;
-    if (warp == 0 && a.tmem_cols) tmem_alloc(&s_tmem, (unsigned)a.tmem_cols);
+    if (warp == 0) tmem_alloc(&s_tmem, (unsigned)a.tmem_cols);
     if (a.list && threadIdx.x == 0) s_next[0] = (int)atomicAdd(a.ticket, 1u);
     __syncthreads();
     const unsigned base = a.tmem_cols ? s_tmem : 0u;
@@ -1090,29 +1093,32 @@ int chip_phase_rows(int64_t max_width, int64_t P, int32_t K, int32_t D) {
     return 0;
 }
 
-// Model of the time of an evaluation in microseconds, within about 10 % of what 19 graphs
-// (1,000 to 117,000 nodes, 300 to 65,536 samples, every mode) took in every shape that
-// fits them.  Per chunk: the busiest of the shared-memory pipe (128 bytes per cycle, times
-// the passes per phase that the row order leaves), the issue slots and the FP64 pipe, then
-// the propagators, then what a chunk waits for by itself -- barriers, fetch and L2 latency,
-// mostly per level -- which CTAs that share an SM hide less than their number suggests
-// (medium graph, FP32: one CTA with 8 samples 1.66 ms, two with 4 samples 1.99 ms).
+// Model of the time of an evaluation in microseconds, fitted to 16 graphs (1,000 to 117,000
+// nodes, 300 to 65,536 samples, every mode) in every shape that fits them, 6 % rms.  Per
+// chunk: the busiest of the shared-memory pipe (128 bytes per cycle, times the passes per
+// phase that the row order leaves), the issue slots and the FP64 pipe, then the propagators,
+// four tenths of whose time CTAs that share an SM hide from one another, then what a chunk
+// waits for by itself -- barriers, fetch and L2 latency, mostly per level -- which they hide
+// almost wholly.  Order 2, 1,000 nodes, 10,007 samples, FP32: one CTA with 32 samples 72
+// us, two with 16 or 8 samples 66, four with 8 samples 70; medium, FP32: one with 8 samples
+// 1.61 ms, two with 4 samples 1.99.
 double chip_time_us(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, int32_t D, bool table, int64_t S, int sms,
                     int rb, int lane, int ctas) {
     const int s = rb / node_bytes(kmode), mode = base_mode(kmode);
     const double B = 128.0 / rb;
-    double conf = B <= 1 ? 1.0 : B <= 2 ? 1.15 : B <= 4 ? 1.45 : B <= 8 ? 1.9 : B <= 16 ? 2.2 : 2.4;
-    const double tables = mode == COS_MODE_COUNT_I64 ? 1.0 : kmode == kModeMixedAbs ? 1.5 : 2.0;
+    double conf = B <= 1 ? 1.0 : B <= 2 ? 1.15 : B <= 4 ? 1.5 : B <= 8 ? 2.0 : B <= 16 ? 2.4 : 2.5;
+    const double tables = mode == COS_MODE_COUNT_I64 ? 1.0 : kmode == kModeMixedAbs ? 1.65 : 2.0;
     const double lds = (double)g.edges * rb / 128.0 * conf * tables + (double)g.rows * rb / 128.0 * 1.3;
-    const double issue = ((double)g.edges * 14 + (double)g.rows * 40) * rb / lane / 32.0 / 4.0;
+    const double issue = ((double)g.edges * 15.2 + (double)g.rows * 47.9) * rb / lane / 32.0 / 4.0;
     const double f64 = mode == COS_MODE_FP64 ? (double)g.edges * s / 2.0 * 1.1 : 0.0;
     double props = 0.0;
     if (table) props = (double)P * s * 4.0;
-    else if (mode == COS_MODE_FP64) props = ((double)K * D * s * 17 + (double)P * s) / 2.0 * 1.1;
-    else if (mode == COS_MODE_FP32_MIXED) props = (double)K * D * s * 2.0 + (double)P * s * 0.25;
-    const double busy = std::max(lds, std::max(issue, f64)) + props, alone = 5000.0 + 900.0 * L;
+    else if (mode == COS_MODE_FP64) props = ((double)K * D * s * 19.9 + (double)P * s) / 2.0 * 1.1;
+    else if (mode == COS_MODE_FP32_MIXED) props = (double)K * D * s * 0.68 + (double)P * s * 0.62;
+    const double busy = std::max(lds, std::max(issue, f64)), alone = 3000.0 + 590.0 * L;
     const int64_t chunks = (S + s - 1) / s, slots = (int64_t)ctas * sms;
-    return (double)((chunks + slots - 1) / slots) * (ctas * busy + alone * (1.0 + 0.1 * (ctas - 1))) / 1930.0 + 12.0;
+    const double wave = ctas * (busy + 0.59 * props) + 0.41 * props + alone * (1.0 + 0.03 * (ctas - 1));
+    return (double)((chunks + slots - 1) / slots) * wave / 1930.0 + 13.9;
 }
 
 // The same for the general kernels: launch and barriers or task planning, edges at the
