@@ -411,7 +411,7 @@ int plan(cos_batch* b) {
         if (chip_ok) {
             OnChip oc;
             int yes = 0;
-            rc = prepare_chip(b->graphs[(size_t)g], mode, b->outs[(size_t)g], &oc.p, &oc.plan, &b->sms, &yes);
+            rc = prepare_chip(b->graphs[(size_t)g], mode, b->outs[(size_t)g], b->n, &oc.p, &oc.plan, &b->sms, &yes);
             if (rc != COS_OK) return rc;
             if (yes) {
                 oc.g = g;

@@ -1103,7 +1103,7 @@ int chip_phase_rows(int64_t max_width, int64_t P, int32_t K, int32_t D) {
 // us, two with 16 or 8 samples 66, four with 8 samples 70; medium, FP32: one with 8 samples
 // 1.61 ms, two with 4 samples 1.99.
 double chip_time_us(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, int32_t D, bool table, int64_t S, int sms,
-                    int rb, int lane, int ctas) {
+                    int rb, int lane, int ctas, int members) {
     const int s = rb / node_bytes(kmode), mode = base_mode(kmode);
     const double B = 128.0 / rb;
     double conf = B <= 1 ? 1.0 : B <= 2 ? 1.15 : B <= 4 ? 1.5 : B <= 8 ? 2.0 : B <= 16 ? 2.4 : 2.5;
@@ -1118,26 +1118,30 @@ double chip_time_us(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t
     const double busy = std::max(lds, std::max(issue, f64)), alone = 3000.0 + 590.0 * L;
     const int64_t chunks = (S + s - 1) / s, slots = (int64_t)ctas * sms;
     const double wave = ctas * (busy + 0.59 * props) + 0.41 * props + alone * (1.0 + 0.03 * (ctas - 1));
-    return (double)((chunks + slots - 1) / slots) * wave / 1930.0 + 13.9;
+    // (the chunks of a batch's members fill one another's last rounds)
+    const double rounds = members > 1 ? (double)chunks / (double)slots : (double)((chunks + slots - 1) / slots);
+    return rounds * wave / 1930.0 + 13.9 / members;
 }
 
 // The same for the general kernels: launch and barriers or task planning, edges at the
 // rate they reach on graphs of this kind, propagator slots (through L2, and back).
-double general_time_us(const ChipGraph& g, int kmode, int32_t L, int32_t P, int64_t S) {
-    const double es = (double)g.edges * (double)S, ps = (double)P * (double)S, fixed = 45.0 + 3.0 * L;
+double general_time_us(const ChipGraph& g, int kmode, int32_t L, int32_t P, int64_t S, int members) {
+    const double es = (double)g.edges * (double)S, ps = (double)P * (double)S, fixed = (45.0 + 3.0 * L) / members;
     if (kmode == COS_MODE_COUNT_I64) return fixed + es / 9.5e5;
     if (kmode == COS_MODE_FP64) return fixed + es / 5.4e5 + ps / 1.5e5;
     return fixed + es / (kmode == kModeMixedAbs ? 8.5e5 : 1.65e6) + ps / 3e5;
 }
 
 // The shape with the least model time; on chip when that is below the general kernels'.
-// Measured on both sides of the line, general / on-chip: medium graph 2.35 / 1.66 ms
-// (FP32), 3.00 / 2.26 ms (with A), 3.2 / 2.2 ms (count), FP64 6.34 / 6.89 ms (both held
-// by the FP64 pipe; general); 117,000 nodes, levels of 11,500 (FP32, two samples per
-// chunk) 7.69 / 7.61 ms, levels of 19,500 5.44 / 5.80 ms (general), but 3,000 samples of
-// the latter 0.48 / 0.42 ms and 300 samples of levels of 30,000 102 / 63 us.
+// Measured on both sides of the line, general / on-chip: medium graph 2.35 / 1.61 ms
+// (FP32), 3.00 / 2.20 ms (with A), 3.1 / 1.86 ms (count), FP64, 16,384 samples, 1.60 / 1.63 ms
+// (both held by the FP64 pipe; general), 10,000 nodes of order 4, FP64, 2,000 samples 226 /
+// 169 us; FP32 with two samples per chunk: 100,000 nodes, levels of 12,200, 4,000 samples 868 /
+// 988 us (general), 500 samples 198 / 131; levels of 19,500 5.44 / 5.80 ms (general), but
+// 3,000 samples of the latter 0.48 / 0.42 ms and 300 samples of levels of 30,000 102 / 63 us.
+// The members of a batch share the fixed times of either side and the last rounds.
 bool chip_plan(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, int32_t D, bool table, int64_t S, int sms,
-               ChipPlan* out) {
+               int members, ChipPlan* out) {
     if (g.max_width <= 0 || S <= 0 || sms <= 0 || kmode == kModeFp64Abs) return false;
     const int nb = node_bytes(kmode);
     bool found = false;
@@ -1146,7 +1150,7 @@ bool chip_plan(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, i
         for (int ctas = 1; ctas <= 4; ctas *= 2) {
             const ChipLayout y = chip_layout(g, kmode, P, K, D, table, rb, smem_limit(ctas));
             if (y.total > smem_limit(ctas) || 512 / ctas / 32 < rb / lane) continue;   // (a group needs rb / lane warps)
-            const double cost = chip_time_us(g, kmode, L, P, K, D, table, S, sms, rb, lane, ctas);
+            const double cost = chip_time_us(g, kmode, L, P, K, D, table, S, sms, rb, lane, ctas, members);
             if (found && cost >= out->cost) continue;
             found = true;
             out->rb_log2 = 31 - __builtin_clz((unsigned)rb);
@@ -1157,7 +1161,7 @@ bool chip_plan(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, i
             out->cost = cost;
         }
     }
-    return found && out->cost < 0.97 * general_time_us(g, kmode, L, P, S);
+    return found && out->cost < 0.97 * general_time_us(g, kmode, L, P, S, members);
 }
 
 void chip_shape(int kmode, const ChipPlan& plan, ChipParams* p) {

@@ -62,9 +62,10 @@ struct ChipPlan {
 };
 
 // Best launch shape for `kmode` on S samples of a graph (max D of the kinds' times,
-// P slots, K kinds); false when the graph does not fit on chip.
+// P slots, K kinds), one of `members` evaluations that run together; false when the graph
+// does not fit on chip or the general kernels are expected to be faster.
 bool chip_plan(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, int32_t D, bool table, int64_t S, int sms,
-               ChipPlan* out);
+               int members, ChipPlan* out);
 // Fill the shape-dependent fields of p (rb_log2 .. coef_off, nchunks).
 void chip_shape(int kmode, const ChipPlan& plan, ChipParams* p);
 // One evaluation, parameters by value.
@@ -76,7 +77,8 @@ int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const Chi
                      unsigned* ticket, unsigned* exits, int sms, cudaStream_t st);
 // Parameters and launch shape of an evaluation of g in kernel mode `kmode` (cos_graph.cu);
 // *on_chip = 0 when it is the general kernels' (no schedule, no fit, or a launch shape set).
-int prepare_chip(cos_graph_t g, int kmode, void* per_sample_out, ChipParams* out, ChipPlan* plan, int* sms, int* on_chip);
+int prepare_chip(cos_graph_t g, int kmode, void* per_sample_out, int members, ChipParams* out, ChipPlan* plan, int* sms,
+                 int* on_chip);
 // The handle's row schedule.
 void chip_view(cos_graph_t g, ChipGraph* out);
 // Phase rows the row schedule of a graph is made for: the widest rows that fit on chip

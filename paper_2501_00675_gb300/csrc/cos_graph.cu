@@ -589,7 +589,7 @@ int cos_graph_info(cos_graph_t g, int64_t* info, int32_t n) {
         for (int km = 0; km <= kModeMixedAbs; ++km) {
             ChipPlan plan;
             if (chip_allowed(g) && chip_plan(g->chip, km, g->L, (int32_t)g->P, g->K, g->D, g->d_ptab != nullptr,
-                                             std::max<int64_t>(g->S, 1), sms, &plan))
+                                             std::max<int64_t>(g->S, 1), sms, 1, &plan))
                 info[10] |= 1LL << km;
         }
     }
@@ -965,7 +965,7 @@ int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean
         ChipPlan plan;
         int sms = 0;
         int on_chip = 0;
-        int rc = prepare_chip(g, km, per_sample_out, &cp, &plan, &sms, &on_chip);
+        int rc = prepare_chip(g, km, per_sample_out, 1, &cp, &plan, &sms, &on_chip);
         if (rc == COS_OK && on_chip) {
             if (mean_out) cp.mean_out = g->h_means;
             rc = launch_chip(km, plan, cp, sms, st);
@@ -1172,11 +1172,13 @@ static int ensure_result_buffer(cos_graph_t g, int64_t nout) {
 
 void chip_view(cos_graph_t g, ChipGraph* out) { *out = g->chip; }
 
-int prepare_chip(cos_graph_t g, int kmode, void* per_sample_out, ChipParams* out, ChipPlan* plan, int* sms, int* on_chip) {
+int prepare_chip(cos_graph_t g, int kmode, void* per_sample_out, int members, ChipParams* out, ChipPlan* plan, int* sms,
+                 int* on_chip) {
     *on_chip = 0;
     if (!g->has_samples || !chip_allowed(g)) return COS_OK;   // (the general path reports missing samples)
     if (cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess) return COS_OK;
-    if (!chip_plan(g->chip, kmode, g->L, (int32_t)g->P, g->K, g->D, g->d_ptab != nullptr, g->S, *sms, plan)) return COS_OK;
+    if (!chip_plan(g->chip, kmode, g->L, (int32_t)g->P, g->K, g->D, g->d_ptab != nullptr, g->S, *sms, members, plan))
+        return COS_OK;
     const bool abs2 = mode_has_abs(kmode);
     if (!per_sample_out) {
         const int rc = ensure_result_buffer(g, std::max<int64_t>(g->S, 1) * (abs2 ? 2 : 1));

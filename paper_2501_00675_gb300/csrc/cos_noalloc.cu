@@ -222,7 +222,7 @@ extern "C" int cos_evaluate_static(cos_graph_t g, int32_t mode, int64_t num_samp
     ChipPlan plan;
     chip_view(g, &cg);
     const bool on_chip = S > 0 && nblk <= kStaticBlocks && !p.skip_barrier_phase &&
-                         chip_plan(cg, mode, gv.L, gv.P, gv.K, gv.D, gv.ptab != nullptr, S, sms, &plan);
+                         chip_plan(cg, mode, gv.L, gv.P, gv.K, gv.D, gv.ptab != nullptr, S, sms, 1, &plan);
     if (on_chip) {
         ChipParams q;
         memset(&q, 0, sizeof(q));
