@@ -296,8 +296,9 @@ int cos_graph_info(cos_graph_t g, int64_t* info, int32_t n);
  *                     the chains are issued in wavefront order, so about L windows
  *                     are in flight.  Results are bitwise the same either way.
  *                     Automatic: 2 in FP64 and FP32 mixed modes with at least 1e9
- *                     edge x samples or when the widest level has at least 65536
- *                     nodes, else 1.
+ *                     edge x samples (3e8 in FP64 with tabulated propagators, unless
+ *                     the stream is being captured) or when the widest level has at
+ *                     least 65536 nodes, else 1.
  *                     Batched launches always use the
  *                     work queue, with windows when window_chunks > 0.
  *   window_chunks     chunks (of 32*samples_per_lane samples, 32 in the grouped
