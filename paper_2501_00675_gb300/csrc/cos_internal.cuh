@@ -23,7 +23,7 @@ struct LevelDesc {
 };
 
 // Per-launch control block in device memory: grid-barrier counter, error word,
-// and the reduced result (mean and its compensated sum; the mean of A(s) when the
+// and the reduced result (mean and its sum; the mean of A(s) when the
 // walk also accumulates sums of |path| values).
 struct Ctrl {
     unsigned long long barrier;
@@ -72,11 +72,11 @@ struct WalkParams {
     const double* exp_tab;     // [128]: 2^{j/64}, then 2^{-j/64}, j = 0..63; followed by the same
                                // 128 values as float-float (hi, lo) pairs (256 floats)
     void* R;                   // [S] sink value per sample (double, or int64 in count mode)
-    double* partials;          // [ceil(S/kReduceBlock)] compensated partial sums
+    double* partials;          // [ceil(S/kReduceBlock)] block sums
     // sums of |path| values in the same walk (kernel modes kModeFp64Abs, kModeMixedAbs)
     void* aslab[2];            // [nchunk][W][CH] float node values of A, as slab[]
     double* Rabs;              // [S] A(s) per sample
-    double* partials_abs;      // [ceil(S/kReduceBlock)] compensated partial sums of A
+    double* partials_abs;      // [ceil(S/kReduceBlock)] block sums of A
     Ctrl* ctrl;
     int64_t tile;              // samples per tile (multiple of CH)
     int32_t rows_per_warp;
@@ -101,7 +101,7 @@ struct WalkParams {
 
 constexpr int kThreads = 256;           // 8 warps per CTA
 constexpr int kWarps = kThreads / 32;
-constexpr int kReduceBlock = 1024;      // samples per compensated partial sum
+constexpr int kReduceBlock = 1024;      // samples per block sum
 
 // Device-resident view of a graph handle (read-only), for entry points that
 // evaluate an existing graph with scratch memory of their own.

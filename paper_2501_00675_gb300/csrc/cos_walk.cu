@@ -5,7 +5,7 @@
 //   3. the levels in order (Sec. II.C "Windowing": a level is complete before any
 //      of its out-edges is used), a grid-wide barrier between levels, every
 //      destination row summing its in-edges in CSR order,
-// and finally reduces the per-sample sink values into a compensated mean.  The
+// and finally reduces the per-sample sink values into their mean.  The
 // work items of each phase are in cos_items.cuh.
 #include <algorithm>
 #include <cstdio>
