@@ -619,8 +619,9 @@ constexpr unsigned kBlockSummed = 0xffffffffu;   // arrival word of a block whos
 // nullptr: of all).
 template <typename T>
 __device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S, int b, int nblk, const unsigned* arrive, CtaSum& c) {
-    // the next block to sum: 32 arrival words at a time (they change no more, so that every
-    // warp finds the same)
+    // the next block to sum: 32 arrival words at a time, read by one warp for all -- the loop
+    // below has block barriers, and a launch that overlaps on the same words changes them
+    __shared__ unsigned s_open;
     int base = -1;
     unsigned open = 0;
     auto skip = [&](int q) {
@@ -628,7 +629,13 @@ __device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S
             if ((q & ~31) != base) {
                 base = q & ~31;
                 const int at = base + (int)(threadIdx.x & 31);
-                open = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != kBlockSummed);
+                __syncthreads();   // everyone has the word before
+                if (threadIdx.x < 32) {
+                    const unsigned left = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != kBlockSummed);
+                    if (threadIdx.x == 0) s_open = left;
+                }
+                __syncthreads();
+                open = s_open;
             }
             const unsigned left = open >> (q - base);
             if (left) return q + __ffs((int)left) - 1;
