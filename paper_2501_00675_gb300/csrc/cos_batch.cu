@@ -40,8 +40,10 @@ struct BatchCtrl {
     int err;
     int err_task;
     unsigned chip_ticket[kChipLaunches];
-    unsigned chip_exits[kChipLaunches];
 };
+// Arrival words of the members on chip (ChipParams::arrive) lie behind it and are cleared
+// with it; word 0 of a launch's first member counts the launch's CTAs.
+static_assert(sizeof(BatchCtrl) % sizeof(unsigned long long) == 0, "the words behind it are aligned");
 
 struct BatchArgs {
     const Task* tasks;
@@ -239,7 +241,8 @@ struct cos_batch {
     unsigned* d_done = nullptr;
     double* d_means = nullptr;
     BatchCtrl* d_ctrl = nullptr;
-    size_t cap_tasks = 0, cap_graphs = 0, cap_joins = 0;
+    size_t cap_tasks = 0, cap_graphs = 0, cap_joins = 0, cap_words = 0;
+    size_t ctrl_bytes = sizeof(BatchCtrl);   // control block and arrival words of the plan
     int32_t ntasks = 0;
     int64_t total = 0;
     int grid = 0;
@@ -308,10 +311,10 @@ void free_buffers(cos_batch* b) {
     b->h_chip = nullptr;
     b->h_means = nullptr;
     b->h_ctrl = nullptr;
-    b->cap_tasks = b->cap_graphs = b->cap_joins = 0;
+    b->cap_tasks = b->cap_graphs = b->cap_joins = b->cap_words = 0;
 }
 
-int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins) {
+int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins, size_t nwords) {
     cudaError_t e = cudaSuccess;
     if (njoins > b->cap_joins || ntasks > b->cap_tasks || ngraphs > b->cap_graphs) {
         const int rc = wait_staged(b);   // pending copies still read the old staging buffers
@@ -329,10 +332,14 @@ int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins) 
             return set_error(COS_ERR_OOM, "batch joins: %s", cudaGetErrorString(e));
         b->cap_joins = cap;
     }
-    if (!b->d_ctrl) {
-        if ((e = cudaMalloc(&b->d_ctrl, sizeof(BatchCtrl))) != cudaSuccess ||
-            (e = cudaMallocHost(&b->h_ctrl, sizeof(BatchCtrl))) != cudaSuccess)
+    if (!b->d_ctrl || nwords > b->cap_words) {
+        cudaFree(b->d_ctrl);
+        b->d_ctrl = nullptr;
+        const size_t cap = std::max<size_t>(nwords, 2 * b->cap_words);
+        if ((e = cudaMalloc(&b->d_ctrl, sizeof(BatchCtrl) + sizeof(unsigned long long) * cap)) != cudaSuccess ||
+            (!b->h_ctrl && (e = cudaMallocHost(&b->h_ctrl, sizeof(BatchCtrl))) != cudaSuccess))
             return set_error(COS_ERR_OOM, "batch control: %s", cudaGetErrorString(e));
+        b->cap_words = cap;
     }
     if (ntasks > b->cap_tasks) {
         cudaFree(b->d_tasks);
@@ -470,8 +477,10 @@ int plan(cos_batch* b) {
     if (b->tuning.blocks_per_sm > 0) bps = std::min(bps, b->tuning.blocks_per_sm);
     b->resolved.blocks_per_sm = bps;
     b->grid = sms * bps;
+    size_t words = 0;
+    for (const OnChip& oc : on_chip) words += 1 + (size_t)((oc.p.S + kReduceBlock - 1) / kReduceBlock);
     int rc = ensure_capacity(b, std::max<size_t>(b->tasks.size(), 1), std::max<int32_t>(b->n, 1),
-                             std::max<size_t>(b->joins.size(), 1));
+                             std::max<size_t>(b->joins.size(), 1), words);
     if (rc != COS_OK) return rc;
     for (int32_t g = 0; g < b->n; ++g) b->params[(size_t)g].mean_out = b->d_means + 2 * g;   // (mean R, mean A)
     // one launch per (lane width, CTA size), its longest evaluations first
@@ -482,12 +491,17 @@ int plan(cos_batch* b) {
     });
     b->chip.clear();
     b->chip_launches.clear();
+    b->ctrl_bytes = sizeof(BatchCtrl) + sizeof(unsigned long long) * words;
+    unsigned long long* arrive = reinterpret_cast<unsigned long long*>(b->d_ctrl + 1);
     for (OnChip& oc : on_chip) {
         if (b->chip_launches.empty() || b->chip_launches.back().lane_bytes != oc.plan.lane_bytes ||
             b->chip_launches.back().threads != oc.plan.threads)
             b->chip_launches.push_back({oc.plan.lane_bytes, oc.plan.threads, 0, (int)b->chip.size(), 0, 0});
         cos_batch::ChipLaunch& cl = b->chip_launches.back();
         oc.p.mean_out = b->d_means + 2 * oc.g;
+        oc.p.arrive = arrive;
+        oc.p.tag = kBatchTag;
+        arrive += 1 + (oc.p.S + kReduceBlock - 1) / kReduceBlock;
         oc.p.first_chunk = cl.chunks;
         cl.chunks += oc.p.nchunks;
         cl.n++;
@@ -506,7 +520,7 @@ int enqueue_run(cos_batch* b, cudaStream_t st) {
     cudaError_t e;
     if ((b->ntasks > 0 &&
          (e = cudaMemsetAsync(b->d_done, 0, sizeof(unsigned) * b->ntasks, st)) != cudaSuccess) ||
-        (e = cudaMemsetAsync(b->d_ctrl, 0, sizeof(BatchCtrl), st)) != cudaSuccess)
+        (e = cudaMemsetAsync(b->d_ctrl, 0, b->ctrl_bytes, st)) != cudaSuccess)
         return set_error(COS_ERR_CUDA, "reset batch counters: %s", cudaGetErrorString(e));
     BatchArgs a;
     a.tasks = b->d_tasks;
@@ -526,7 +540,7 @@ int enqueue_run(cos_batch* b, cudaStream_t st) {
     for (size_t q = 0; q < b->chip_launches.size(); ++q) {
         const cos_batch::ChipLaunch& cl = b->chip_launches[q];
         const int rc = launch_chip_list(b->mode, cl.lane_bytes, cl.threads, cl.smem, b->d_chip + cl.first, cl.n, cl.chunks,
-                                        &b->d_ctrl->chip_ticket[q], &b->d_ctrl->chip_exits[q], b->sms, st);
+                                        &b->d_ctrl->chip_ticket[q], b->chip[(size_t)cl.first].arrive, b->sms, st);
         if (rc != COS_OK) return rc;
     }
     return COS_OK;

@@ -34,6 +34,7 @@
 // 1,000 samples, mixed, one launch: 20.5 -> 14.4 us; order 2, 1,000 nodes, 10,007 samples:
 // 96 -> 84 us.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <type_traits>
 
@@ -145,7 +146,8 @@ struct ChipArgs {
     ChipParams one;
     const ChipParams* list;   // nullptr: `one`, chunks dealt out by CTA number
     unsigned* ticket;
-    unsigned* exits;          // CTAs that have left (zero between launches)
+    unsigned long long* exits;   // CTAs that have left, under `tag`
+    unsigned long long tag;
     int n, total;
     int tmem_cols;            // 0: no level goes through TMEM
     int few;                  // so few blocks of samples that the last CTA sums them all
@@ -613,12 +615,16 @@ __device__ __forceinline__ void cta_sum(double (&v)[kPerThread], const T* x, dou
         if (lane == 0) partials[b] = sum;
     }
 }
-constexpr unsigned kBlockSummed = 0xffffffffu;   // arrival word of a block whose partial sum is written
+// Arrival word of a block whose partial sum is written.  (A launch's own counts end at
+// kReduceBlock, 2^10: those of calls that overlap stay out of the tag and below this one.)
+__device__ __forceinline__ unsigned long long tagged(unsigned long long tag, unsigned n) { return tag << kTagShift | n; }
+constexpr unsigned kBlockSummed = 1u << (kTagShift - 1);
 
-// Partial sums of blocks [b, nblk) whose arrival word is not kBlockSummed (arrive
-// nullptr: of all).
+// Partial sums of blocks [b, nblk) whose arrival word is not `summed` (arrive nullptr: of
+// all).
 template <typename T>
-__device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S, int b, int nblk, const unsigned* arrive, CtaSum& c) {
+__device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S, int b, int nblk, const unsigned long long* arrive,
+                                         unsigned long long summed, CtaSum& c) {
     // the next block to sum: 32 arrival words at a time, read by one warp for all -- the loop
     // below has block barriers, and a launch that overlaps on the same words changes them
     __shared__ unsigned s_open;
@@ -631,7 +637,7 @@ __device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S
                 const int at = base + (int)(threadIdx.x & 31);
                 __syncthreads();   // everyone has the word before
                 if (threadIdx.x < 32) {
-                    const unsigned left = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != kBlockSummed);
+                    const unsigned left = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != summed);
                     if (threadIdx.x == 0) s_open = left;
                 }
                 __syncthreads();
@@ -656,11 +662,13 @@ __device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S
     }
 }
 template <int MODE>
-__device__ __noinline__ void chip_sums(const ChipParams& p, unsigned char* sm, int b, int nblk, const unsigned* arrive) {
+__device__ __noinline__ void chip_sums(const ChipParams& p, unsigned char* sm, int b, int nblk, bool all) {
+    const unsigned long long* arrive = all ? nullptr : p.arrive + 1;
+    const unsigned long long summed = tagged(p.tag, kBlockSummed);
     CtaSum& c = *reinterpret_cast<CtaSum*>(sm);   // (the level buffer, free by now)
-    if constexpr (Traits<MODE>::kCount) cta_sums(static_cast<const long long*>(p.R), p.partials, p.S, b, nblk, arrive, c);
-    else cta_sums(static_cast<const double*>(p.R), p.partials, p.S, b, nblk, arrive, c);
-    if constexpr (Traits<MODE>::kAbs) cta_sums(p.Rabs, p.partials_abs, p.S, b, nblk, arrive, c);
+    if constexpr (Traits<MODE>::kCount) cta_sums(static_cast<const long long*>(p.R), p.partials, p.S, b, nblk, arrive, summed, c);
+    else cta_sums(static_cast<const double*>(p.R), p.partials, p.S, b, nblk, arrive, summed, c);
+    if constexpr (Traits<MODE>::kAbs) cta_sums(p.Rabs, p.partials_abs, p.S, b, nblk, arrive, summed, c);
 }
 
 
@@ -669,7 +677,12 @@ __device__ __noinline__ void chip_sums(const ChipParams& p, unsigned char* sm, i
 __device__ __forceinline__ void chip_arrive(const ChipParams& p, int chunk) {
     const int64_t s0 = (int64_t)chunk << p.s_log2;
     const unsigned mine = (unsigned)min((int64_t)1 << p.s_log2, p.S - s0);
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.arrive + s0 / kReduceBlock), "r"(mine) : "memory");
+    unsigned long long* w = p.arrive + 1 + s0 / kReduceBlock;
+    // (an older launch's count is below every word of this one's tag; a newer one's, met only
+    // where launches run in another order than they were made, stays, and then the last CTA
+    // sums the block)
+    asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(w), "l"(tagged(p.tag, 0u)) : "memory");
+    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"((unsigned long long)mine) : "memory");
 }
 
 __device__ __forceinline__ int chip_blocks(const ChipParams& p) { return (int)((p.S + kReduceBlock - 1) / kReduceBlock); }
@@ -682,26 +695,17 @@ __device__ __forceinline__ void chip_sum_own(const ChipParams& p, unsigned char*
     const int nblk = chip_blocks(p), grid = gridDim.x;
     for (int b = (int)((blockIdx.x + grid - first % grid) % grid); b < nblk; b += grid) {
         if (threadIdx.x == 0)
-            s_full = ld_acquire_gpu_u32(p.arrive + b) == (unsigned)min((int64_t)kReduceBlock, p.S - (int64_t)b * kReduceBlock);
+            s_full = ld_acquire_gpu(p.arrive + 1 + b) ==
+                     tagged(p.tag, (unsigned)min((int64_t)kReduceBlock, p.S - (int64_t)b * kReduceBlock));
         __syncthreads();
         const bool full = s_full != 0;
         __syncthreads();
         if (!full) continue;
-        chip_sums<MODE>(p, sm, b, b + 1, nullptr);
-        if (threadIdx.x == 0) p.arrive[b] = kBlockSummed;   // (read by the last CTA, after this one's release)
+        chip_sums<MODE>(p, sm, b, b + 1, true);
+        if (threadIdx.x == 0) p.arrive[1 + b] = tagged(p.tag, kBlockSummed);   // (read by the last CTA, after this one's release)
     }
 }
 
-// The last CTA of the launch: the blocks nobody has summed, then the means.  The
-// arrival words are left at zero.
-template <int MODE>
-__device__ __forceinline__ void chip_sum_rest(const ChipParams& p, unsigned char* sm, bool all) {
-    const int nblk = chip_blocks(p);
-    chip_sums<MODE>(p, sm, 0, nblk, all ? nullptr : p.arrive);
-    if (all) return;
-    __syncthreads();
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) p.arrive[b] = 0;
-}
 template <int MODE>
 __device__ __noinline__ void chip_mean(const ChipParams& p, int lane) {
     const int64_t nblk = (p.S + kReduceBlock - 1) / kReduceBlock;
@@ -946,6 +950,14 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
     __shared__ int s_last;
     __shared__ ChipParams s_p;
     const int warp = threadIdx.x >> 5;
+    // the exit word, taken over for this launch further below by one compare-and-swap of every
+    // CTA: one that fails has lost to a CTA of this launch, nobody else writes the word
+    const bool claims = threadIdx.x == 32;
+    unsigned long long found = 0;
+    if (claims) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(found) : "l"(a.exits) : "memory");
+    auto claim = [&] {
+        if (claims && found >> kTagShift != a.tag) atomicCAS(a.exits, found, tagged(a.tag, 0u));
+    };
     if (warp == 0) tmem_alloc(&s_tmem, (unsigned)a.tmem_cols);
     if (a.list && threadIdx.x == 0) s_next[0] = (int)atomicAdd(a.ticket, 1u);
     __syncthreads();
@@ -959,6 +971,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
         chip_setup<MODE>(a.one, sm);
         cs.word = lane < a.one.g.nsink ? __ldg(a.one.g.sink + lane) : 0u;
         chip_times<MODE>(a.one, sm, blockIdx.x);   // (the grid has no CTA without a chunk)
+        claim();
         cp_async_wait<0>();
         __syncthreads();
         for (int c = blockIdx.x; c < a.one.nchunks; c += gridDim.x)
@@ -970,6 +983,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
         if (!a.few) chip_sum_own<MODE>(a.one, sm, 0);
     } else {
         int g = -1;
+        claim();
         for (int buf = 0;; buf ^= 1) {
             const int c = s_next[buf];
             if (c >= a.total) break;
@@ -1004,20 +1018,19 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
     __syncthreads();
     if (threadIdx.x == 0) {
         // (one atomic with both orders: between two fences it took 1,000 cycles longer)
-        unsigned before;
-        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(before) : "l"(a.exits) : "memory");
-        s_last = before + 1u == gridDim.x;
+        unsigned long long before;
+        asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(before) : "l"(a.exits) : "memory");
+        s_last = before + 1u == tagged(a.tag, gridDim.x);
     }
     __syncthreads();
     if (s_last) {   // every other CTA has counted its chunks in and left
         const int n = a.list ? a.n : 1;
         for (int h = 0; h < n; ++h) {
             const ChipParams& p = a.list ? a.list[h] : a.one;
-            chip_sum_rest<MODE>(p, sm, a.few != 0);
+            chip_sums<MODE>(p, sm, 0, chip_blocks(p), a.few != 0);   // the blocks nobody has summed
         }
         __syncthreads();
         for (int h = warp; h < n; h += blockDim.x >> 5) chip_mean<MODE>(a.list ? a.list[h] : a.one, threadIdx.x & 31);
-        if (threadIdx.x == 0) *a.exits = 0;
     }
     __syncthreads();
     if (warp == 0 && a.tmem_cols) tmem_dealloc(base, (unsigned)a.tmem_cols);
@@ -1211,11 +1224,23 @@ int launch(int kmode, int lane_bytes, int threads, int smem, bool staged, ChipAr
 
 }  // namespace
 
+unsigned long long next_chip_tag() {
+    static std::atomic<unsigned long long> tag{kBatchTag};
+    return ++tag;
+}
+
 int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, cudaStream_t st) {
     ChipArgs a{};
     a.one = p;
     const int64_t blocks = (p.S + kReduceBlock - 1) / kReduceBlock;
-    a.exits = p.arrive + blocks;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();   // (the launch reports it)
+    if (cap != cudaStreamCaptureStatusNone) {   // replays carry one tag
+        const cudaError_t e = cudaMemsetAsync(p.arrive, 0, sizeof(*p.arrive) * (size_t)(blocks + 1), st);
+        if (e != cudaSuccess) return set_error(COS_ERR_CUDA, "clear arrival counters: %s", cudaGetErrorString(e));
+    }
+    a.exits = p.arrive;
+    a.tag = p.tag;
     a.few = blocks <= few_blocks(plan.threads);
     // with room for any two levels none goes through TMEM, whose allocation takes 700 cycles
     const bool staged = p.lev_bytes < 2 * round128(((int64_t)p.g.max_width + 1) << p.rb_log2);
@@ -1223,9 +1248,10 @@ int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, c
 }
 
 int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const ChipParams* list, int n, int total,
-                     unsigned* ticket, unsigned* exits, int sms, cudaStream_t st) {
+                     unsigned* ticket, unsigned long long* exits, int sms, cudaStream_t st) {
     ChipArgs a{};
     a.exits = exits;
+    a.tag = kBatchTag;
     a.list = list;
     a.n = n;
     a.total = total;

@@ -24,6 +24,16 @@ struct ChipGraph {
     int64_t edges = 0, rows = 0;
 };
 
+// Arrivals are counted under the launch's tag (the upper 44 bits of a word, the count in the
+// lower 20), a number that no other launch of the process has: whatever an earlier launch
+// left in a word -- calls that share the words and overlapped, which spoils their own
+// results, among them -- a later launch counts from zero.  Clearing the words on the stream
+// before each launch instead would cost a node of some 2 us in front of a tiny graph's 14;
+// only a captured launch, whose replays carry one tag, is preceded by one.
+constexpr int kTagShift = 20;
+constexpr unsigned long long kBatchTag = 1;   // of a batch's launches, whose words are cleared with its counters
+unsigned long long next_chip_tag();
+
 constexpr int kChipMaxTimes = 48;   // D: the sign masks of all (i, j) pairs are kept in shared memory
 
 // Everything the kernel needs about one evaluation.
@@ -40,7 +50,10 @@ struct ChipParams {
     double* partials_abs;
     Ctrl* ctrl;
     double* mean_out;          // optional second destination of the mean(s)
-    unsigned* arrive;          // [blocks of kReduceBlock samples + 1], zero between launches
+    // [1 + blocks of kReduceBlock samples] words of launch tag and count: word 0 the CTAs that
+    // have left, word 1 + b the samples of block b that are written (see kTagShift)
+    unsigned long long* arrive;
+    unsigned long long tag;    // this launch's number
     double beta, ptab_inv_h;
     int64_t S, t_ld;
     int32_t L, P, K, D, ptab_T, abs_weights;
@@ -72,9 +85,9 @@ void chip_shape(int kmode, const ChipPlan& plan, ChipParams* p);
 int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, cudaStream_t st);
 // Evaluations of n graphs that share (lane_bytes, threads): parameters in device
 // memory, chunks [0, total) drawn from *ticket, leaving CTAs counted in *exits (both zero
-// at launch).
+// at launch, the words of every member's arrivals too; tag kBatchTag).
 int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const ChipParams* list, int n, int total,
-                     unsigned* ticket, unsigned* exits, int sms, cudaStream_t st);
+                     unsigned* ticket, unsigned long long* exits, int sms, cudaStream_t st);
 // Parameters and launch shape of an evaluation of g in kernel mode `kmode` (cos_graph.cu);
 // *on_chip = 0 when it is the general kernels' (no schedule, no fit, or a launch shape set).
 int prepare_chip(cos_graph_t g, int kmode, void* per_sample_out, int members, ChipParams* out, ChipPlan* plan, int* sms,

@@ -137,7 +137,7 @@ struct cos_graph {
     size_t arena_bytes = 0;
     double* d_partials = nullptr;
     int64_t partial_cap = 0;
-    unsigned* d_arrive = nullptr;   // on-chip walk: arrival counters [partial_cap + 1] behind the partials, zero between launches
+    unsigned long long* d_arrive = nullptr;   // on-chip walk: arrival words [1 + partial_cap] behind the partials (ChipParams::arrive)
     ChipGraph chip;                 // on-chip walk: row schedule (max_width 0: none)
     void* d_R = nullptr;            // internal per-sample output when the caller passes none
     int64_t R_cap = 0;
@@ -817,9 +817,9 @@ static int attach_samples(cos_graph_t g, int64_t num_samples, const double* t, i
         // two arrays: partial sums of R, then of A (when the walk also sums |path| values),
         // and the arrival counters of the on-chip walk
         g->partial_cap = 0;
-        COS_CUDA(cudaMalloc(&g->d_partials, 2 * sizeof(double) * cap + sizeof(unsigned) * (cap + 1)), "cudaMalloc partials");
-        g->d_arrive = reinterpret_cast<unsigned*>(g->d_partials + 2 * cap);
-        COS_CUDA(cudaMemsetAsync(g->d_arrive, 0, sizeof(unsigned) * (cap + 1), st), "clear arrival counters");
+        COS_CUDA(cudaMalloc(&g->d_partials, 2 * sizeof(double) * cap + sizeof(*g->d_arrive) * (cap + 1)), "cudaMalloc partials");
+        g->d_arrive = reinterpret_cast<unsigned long long*>(g->d_partials + 2 * cap);
+        COS_CUDA(cudaMemsetAsync(g->d_arrive, 0, sizeof(*g->d_arrive) * (cap + 1), st), "clear arrival counters");
         g->partial_cap = cap;
     }
     // Workspace arena: enough for the FP64 mode over all samples, up to the budget.
@@ -967,6 +967,7 @@ int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean
         int on_chip = 0;
         int rc = prepare_chip(g, km, per_sample_out, 1, &cp, &plan, &sms, &on_chip);
         if (rc == COS_OK && on_chip) {
+            cp.tag = next_chip_tag();
             if (mean_out) cp.mean_out = g->h_means;
             rc = launch_chip(km, plan, cp, sms, st);
         }

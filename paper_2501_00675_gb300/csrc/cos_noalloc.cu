@@ -34,10 +34,10 @@ namespace {
 
 static __device__ __align__(256) unsigned char g_static_scratch[COS_STATIC_SCRATCH_BYTES];
 
-// Arrival counters of the on-chip walk, zero between launches (its other working memory
-// is on chip; the partial sums and the control block are in the scratch array).
+// Arrival words of the on-chip walk (its other working memory is on chip; the partial sums
+// and the control block are in the scratch array).
 constexpr int kStaticBlocks = 4096;
-static __device__ unsigned g_static_arrive[kStaticBlocks + 1];
+static __device__ unsigned long long g_static_arrive[kStaticBlocks + 1];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_addr_mutex;
@@ -235,7 +235,8 @@ extern "C" int cos_evaluate_static(cos_graph_t g, int32_t mode, int64_t num_samp
         q.R = per_sample_out;
         q.partials = reinterpret_cast<double*>(b + part_at);
         q.ctrl = p.ctrl;
-        q.arrive = static_cast<unsigned*>(arrive);
+        q.arrive = static_cast<unsigned long long*>(arrive);
+        q.tag = next_chip_tag();
         q.beta = beta;
         q.ptab_inv_h = p.ptab_inv_h;
         q.S = S;
