@@ -124,7 +124,8 @@ int cos_graph_share(cos_graph_t src, cos_graph_t* out);
  * schedule or of an internal result buffer; cos_evaluate_static never allocates.)
  * The copy is asynchronous: a host t must stay valid until the stream reaches
  * this point.
- * Errors: COS_ERR_INVALID, COS_ERR_OOM, COS_ERR_CUDA.
+ * Errors: COS_ERR_INVALID (the samples attached before stay), COS_ERR_OOM,
+ * COS_ERR_CUDA (the handle is left without samples).
  */
 int cos_set_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t t_flags,
                     const double* eps, double beta, void* stream);

@@ -782,6 +782,34 @@ static int stage_energies(cos_graph_t g, const double* eps, cudaStream_t st, Ene
     return COS_OK;
 }
 
+// Energies and inverse temperature of a sample set.
+static int check_energies(cos_graph_t g, const double* eps, double beta) {
+    if (!eps) return fail(COS_ERR_INVALID, "eps is NULL");
+    if (!(beta > 0.0) || !std::isfinite(beta)) return fail(COS_ERR_INVALID, "beta must be positive and finite");
+    for (int32_t k = 0; k < g->K; ++k)
+        if (!std::isfinite(eps[k]) || std::fabs(eps[k]) * beta > 600.0)
+            return fail(COS_ERR_INVALID, "eps[%d] * beta must be finite with magnitude <= 600", k);
+    return COS_OK;
+}
+
+// A new sample set takes over the handle's buffers: until it is attached the handle has
+// none, so that a failure half way (an allocation above all) leaves no evaluation, walker or
+// batch plan that would use freed or overwritten buffers.
+static void drop_samples(cos_graph_t g) {
+    g->has_samples = false;
+    g->generation++;
+}
+
+// Room for `values` times in the handle's own buffer.
+static int ensure_times(cos_graph_t g, int64_t values) {
+    if (values <= g->t_cap) return COS_OK;
+    g->t_cap = 0;
+    dfree(g->d_t);
+    COS_CUDA(cudaMalloc(&g->d_t, sizeof(double) * values), "cudaMalloc t");
+    g->t_cap = values;
+    return COS_OK;
+}
+
 // cos_set_samples; with `rest` the caller's launch writes the energies (left in *rest) and
 // the times.
 static int attach_samples(cos_graph_t g, int64_t num_samples, const double* t, int32_t t_flags, const double* eps,
@@ -789,14 +817,11 @@ static int attach_samples(cos_graph_t g, int64_t num_samples, const double* t, i
     if (!g) return fail(COS_ERR_INVALID, "graph is NULL");
     if (num_samples < 0) return fail(COS_ERR_INVALID, "num_samples must be >= 0");
     if (num_samples > 0 && !t) return fail(COS_ERR_INVALID, "t is NULL");
-    if (!eps) return fail(COS_ERR_INVALID, "eps is NULL");
     if (t_flags & ~(COS_T_HOST | COS_T_SAMPLE_MAJOR | COS_T_BORROW)) return fail(COS_ERR_INVALID, "unknown t_flags bits");
     if ((t_flags & COS_T_BORROW) && (t_flags & (COS_T_HOST | COS_T_SAMPLE_MAJOR)))
         return fail(COS_ERR_INVALID, "COS_T_BORROW needs a device [D][t_ld] buffer");
-    if (!(beta > 0.0) || !std::isfinite(beta)) return fail(COS_ERR_INVALID, "beta must be positive and finite");
-    for (int32_t k = 0; k < g->K; ++k)
-        if (!std::isfinite(eps[k]) || std::fabs(eps[k]) * beta > 600.0)
-            return fail(COS_ERR_INVALID, "eps[%d] * beta must be finite with magnitude <= 600", k);
+    int rc = check_energies(g, eps, beta);
+    if (rc != COS_OK) return rc;
     DeviceGuard dg(g->device);
     if (!dg.ok) return fail(COS_ERR_CUDA, "cannot select device %d", g->device);
     cudaStream_t st = (cudaStream_t)stream;
@@ -804,19 +829,17 @@ static int attach_samples(cos_graph_t g, int64_t num_samples, const double* t, i
     const int64_t t_ld = std::max<int64_t>(round_up(S, 128), 128);
     const int32_t D = g->D;
     const bool borrow = (t_flags & COS_T_BORROW) != 0;
-    if (!borrow && t_ld * D > g->t_cap) {
-        dfree(g->d_t);
-        COS_CUDA(cudaMalloc(&g->d_t, sizeof(double) * t_ld * D), "cudaMalloc t");
-        g->t_cap = t_ld * D;
-    }
+    drop_samples(g);
+    if (!borrow && (rc = ensure_times(g, t_ld * D)) != COS_OK) return rc;
     if (!g->d_eps) COS_CUDA(cudaMalloc(&g->d_eps, sizeof(double) * g->K), "cudaMalloc eps");
     const int64_t nblk = std::max<int64_t>((S + kReduceBlock - 1) / kReduceBlock, 1);
     if (nblk > g->partial_cap) {
-        dfree(g->d_partials);
         const int64_t cap = std::max<int64_t>(nblk, 4096);   // room for 4M samples without regrowth
         // two arrays: partial sums of R, then of A (when the walk also sums |path| values),
         // and the arrival counters of the on-chip walk
         g->partial_cap = 0;
+        g->d_arrive = nullptr;
+        dfree(g->d_partials);
         COS_CUDA(cudaMalloc(&g->d_partials, 2 * sizeof(double) * cap + sizeof(*g->d_arrive) * (cap + 1)), "cudaMalloc partials");
         g->d_arrive = reinterpret_cast<unsigned long long*>(g->d_partials + 2 * cap);
         COS_CUDA(cudaMemsetAsync(g->d_arrive, 0, sizeof(*g->d_arrive) * (cap + 1), st), "clear arrival counters");
@@ -841,7 +864,7 @@ static int attach_samples(cos_graph_t g, int64_t num_samples, const double* t, i
         }
     }
     Energies energies;
-    int rc = stage_energies(g, eps, st, &energies);
+    rc = stage_energies(g, eps, st, &energies);
     if (rc != COS_OK) return rc;
     g->t_borrowed = borrow ? t : nullptr;
     PlaceFrom from = borrow ? PLACE_NOTHING : PLACE_PADDING;
@@ -856,6 +879,7 @@ static int attach_samples(cos_graph_t g, int64_t num_samples, const double* t, i
             from = PLACE_SAMPLE_MAJOR;
             if (host) {
                 if (S * D > g->stage_cap) {
+                    g->stage_cap = 0;
                     dfree(g->d_stage);
                     COS_CUDA(cudaMalloc(&g->d_stage, sizeof(double) * S * D), "cudaMalloc staging");
                     g->stage_cap = S * D;
@@ -888,24 +912,26 @@ int cos_set_samples_uniform(cos_graph_t g, int64_t num_samples, uint64_t seed, i
                             const double* eps, double beta, void* stream) {
     if (!g) return fail(COS_ERR_INVALID, "graph is NULL");
     if (num_samples < 0 || first_sample < 0) return fail(COS_ERR_INVALID, "num_samples and first_sample must be >= 0");
-    // attach as a borrowed empty sample set first (validates eps/beta, sizes the workspace) ...
+    int rc = check_energies(g, eps, beta);
+    if (rc != COS_OK) return rc;
+    // attach as a borrowed sample set first (sizes the workspace) ...
     DeviceGuard dg(g->device);
     if (!dg.ok) return fail(COS_ERR_CUDA, "cannot select device %d", g->device);
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t t_ld = std::max<int64_t>(round_up(num_samples, 128), 128);
-    if (t_ld * g->D > g->t_cap) {
-        dfree(g->d_t);
-        COS_CUDA(cudaMalloc(&g->d_t, sizeof(double) * t_ld * g->D), "cudaMalloc t");
-        g->t_cap = t_ld * g->D;
-    }
+    drop_samples(g);
+    if ((rc = ensure_times(g, t_ld * g->D)) != COS_OK) return rc;
     Energies energies;
-    int rc = attach_samples(g, num_samples, g->d_t, COS_T_BORROW, eps, beta, stream, &energies);
+    rc = attach_samples(g, num_samples, g->d_t, COS_T_BORROW, eps, beta, stream, &energies);
     if (rc != COS_OK) return rc;
     // ... then fill the graph's own time buffer with the counter-based draws
     g->t_borrowed = nullptr;
     g->generation++;
     rc = launch_uniform_times(seed, first_sample, num_samples, g->D, beta, g->d_t, t_ld, energies, st);
-    if (rc != COS_OK) return fail(rc, "sampler launch failed");
+    if (rc != COS_OK) {
+        drop_samples(g);
+        return fail(rc, "sampler launch failed");
+    }
     return COS_OK;
 }
 
