@@ -314,6 +314,18 @@ void free_buffers(cos_batch* b) {
     b->cap_tasks = b->cap_graphs = b->cap_joins = b->cap_words = 0;
 }
 
+// (hook of a test: every allocation fails while the variable is set)
+template <class T>
+cudaError_t device_buffer(T** p, size_t n) {
+    return getenv("COS_TEST_FAIL_ALLOC") ? cudaErrorMemoryAllocation : cudaMalloc(p, sizeof(T) * n);
+}
+int no_room(const char* what, cudaError_t e) {
+    cudaGetLastError();   // (or a later launch would report it)
+    return set_error(COS_ERR_OOM, "%s: %s", what, cudaGetErrorString(e));
+}
+
+// Buffers for a plan of this size.  A capacity is taken back before its buffers are freed, so
+// that after a failure the next plan, however small, allocates them anew.
 int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins, size_t nwords) {
     cudaError_t e = cudaSuccess;
     if (njoins > b->cap_joins || ntasks > b->cap_tasks || ngraphs > b->cap_graphs) {
@@ -322,40 +334,46 @@ int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins, 
         b->staged_valid = false;
     }
     if (njoins > b->cap_joins) {
+        const size_t cap = std::max<size_t>(njoins, 2 * b->cap_joins);
+        b->cap_joins = 0;
         cudaFree(b->d_joins);
         cudaFreeHost(b->h_joins);
         b->d_joins = nullptr;
         b->h_joins = nullptr;
-        const size_t cap = std::max<size_t>(njoins, 2 * b->cap_joins);
-        if ((e = cudaMalloc(&b->d_joins, sizeof(int32_t) * cap)) != cudaSuccess ||
+        if ((e = device_buffer(&b->d_joins, cap)) != cudaSuccess ||
             (e = cudaMallocHost(&b->h_joins, sizeof(int32_t) * cap)) != cudaSuccess)
-            return set_error(COS_ERR_OOM, "batch joins: %s", cudaGetErrorString(e));
+            return no_room("batch joins", e);
         b->cap_joins = cap;
     }
+    if (!b->h_ctrl && (e = cudaMallocHost(&b->h_ctrl, sizeof(BatchCtrl))) != cudaSuccess) return no_room("batch control", e);
     if (!b->d_ctrl || nwords > b->cap_words) {
+        const size_t cap = std::max<size_t>(nwords, 2 * b->cap_words);
+        b->cap_words = 0;
         cudaFree(b->d_ctrl);
         b->d_ctrl = nullptr;
-        const size_t cap = std::max<size_t>(nwords, 2 * b->cap_words);
-        if ((e = cudaMalloc(&b->d_ctrl, sizeof(BatchCtrl) + sizeof(unsigned long long) * cap)) != cudaSuccess ||
-            (!b->h_ctrl && (e = cudaMallocHost(&b->h_ctrl, sizeof(BatchCtrl))) != cudaSuccess))
-            return set_error(COS_ERR_OOM, "batch control: %s", cudaGetErrorString(e));
+        char* block = nullptr;
+        if ((e = device_buffer(&block, sizeof(BatchCtrl) + sizeof(unsigned long long) * cap)) != cudaSuccess)
+            return no_room("batch control", e);
+        b->d_ctrl = reinterpret_cast<BatchCtrl*>(block);
         b->cap_words = cap;
     }
     if (ntasks > b->cap_tasks) {
+        const size_t cap = std::max<size_t>(ntasks, 2 * b->cap_tasks);
+        b->cap_tasks = 0;
         cudaFree(b->d_tasks);
         cudaFree(b->d_done);
         cudaFreeHost(b->h_tasks);
         b->d_tasks = nullptr;
         b->d_done = nullptr;
         b->h_tasks = nullptr;
-        const size_t cap = std::max<size_t>(ntasks, 2 * b->cap_tasks);
-        if ((e = cudaMalloc(&b->d_tasks, sizeof(Task) * cap)) != cudaSuccess ||
-            (e = cudaMalloc(&b->d_done, sizeof(unsigned) * cap)) != cudaSuccess ||
+        if ((e = device_buffer(&b->d_tasks, cap)) != cudaSuccess || (e = device_buffer(&b->d_done, cap)) != cudaSuccess ||
             (e = cudaMallocHost(&b->h_tasks, sizeof(Task) * cap)) != cudaSuccess)
-            return set_error(COS_ERR_OOM, "batch task list: %s", cudaGetErrorString(e));
+            return no_room("batch task list", e);
         b->cap_tasks = cap;
     }
     if (ngraphs > b->cap_graphs) {
+        const size_t cap = std::max<size_t>(ngraphs, 2 * b->cap_graphs);
+        b->cap_graphs = 0;
         cudaFree(b->d_params);
         cudaFree(b->d_chip);
         cudaFree(b->d_means);
@@ -368,14 +386,12 @@ int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins, 
         b->d_means = nullptr;
         b->h_params = nullptr;
         b->h_means = nullptr;
-        const size_t cap = std::max<size_t>(ngraphs, 2 * b->cap_graphs);
-        if ((e = cudaMalloc(&b->d_params, sizeof(WalkParams) * cap)) != cudaSuccess ||
-            (e = cudaMalloc(&b->d_means, 2 * sizeof(double) * cap)) != cudaSuccess ||
+        if ((e = device_buffer(&b->d_params, cap)) != cudaSuccess || (e = device_buffer(&b->d_means, 2 * cap)) != cudaSuccess ||
+            (e = device_buffer(&b->d_chip, cap)) != cudaSuccess ||
             (e = cudaMallocHost(&b->h_params, sizeof(WalkParams) * cap)) != cudaSuccess ||
-            (e = cudaMalloc(&b->d_chip, sizeof(ChipParams) * cap)) != cudaSuccess ||
             (e = cudaMallocHost(&b->h_chip, sizeof(ChipParams) * cap)) != cudaSuccess ||
             (e = cudaMallocHost(&b->h_means, 2 * sizeof(double) * cap)) != cudaSuccess)
-            return set_error(COS_ERR_OOM, "batch parameters: %s", cudaGetErrorString(e));
+            return no_room("batch parameters", e);
         b->cap_graphs = cap;
     }
     return COS_OK;
