@@ -151,7 +151,7 @@ struct cos_graph {
     double* d_ptab = nullptr;       // user-tabulated propagators [K][2][ptab_T+1], or none
     int32_t ptab_T = 0;
     double ptab_tau_max = 0.0;
-    bool capturing = false;         // during cos_evaluate: its stream is being captured
+    bool no_plan = false;           // during cos_evaluate: the work queue's plan is not to be had (capture, no memory)
     int last_wave = 0;              // the last evaluate ran the windowed schedule
     // page-locked (mean R, mean A), written by the on-chip walk of a call that waits for its
     // mean: reading the control block takes a copy after the kernel (nullptr: no such memory)
@@ -633,8 +633,9 @@ static int resolve_tuning(cos_graph_t g, int kmode, cos_tuning* out, int64_t* ti
     // their integer arithmetic (see item_props), is ahead from fewer samples on: medium
     // graph, level-synchronous / work queue, 4,096 samples (1.9e8) 630 / 660 us, 8,192 1,106 /
     // 1,007, 16,384 2,063 / 1,865; 100,000 nodes, 1,024 (2.6e8) 853 / 870, 2,048 1,454 / 1,302.
-    // Not on a capturing stream, which the work queue's uploads do not suit.
-    const bool tables = g->d_ptab && kmode == COS_MODE_FP64 && work >= 3e8 && !g->capturing;
+    // Not on a capturing stream, which the work queue's uploads do not suit, nor where its plan
+    // finds no memory: the level-synchronous kernel takes these sizes without any.
+    const bool tables = g->d_ptab && kmode == COS_MODE_FP64 && work >= 3e8 && !g->no_plan;
     if (t.schedule <= 0)
         t.schedule = ((big && (mode == COS_MODE_FP64 || mode == COS_MODE_FP32_MIXED)) || tables || g->Wmax >= 65536) ? 2 : 1;
     // level-synchronous: 8 rows per warp measured best for the FP32 walk (medium: 2.46 ms
@@ -977,6 +978,43 @@ static int collect(cos_graph_t g, double* mean_out, cudaStream_t st) {
     return COS_OK;
 }
 
+// cos_evaluate by the general kernels; no_plan: not by a work queue that the tables alone ask
+// for (resolve_tuning).
+static int evaluate_general(cos_graph_t g, int km, void* per_sample_out, double* mean_out, cudaStream_t st, bool no_plan) {
+    WalkParams p;
+    cos_tuning tn;
+    g->no_plan = no_plan;
+    int rc = cosgpu::prepare_walk(g, km, nullptr, per_sample_out, &p, &tn);
+    g->no_plan = false;
+    if (rc != COS_OK) return rc;
+    if (const char* env = getenv("COS_TEST_SKIP_BARRIER_PHASE")) p.skip_barrier_phase = atoi(env);
+    if (g->d_trace) {
+        p.trace = g->d_trace;
+        p.trace_cap = g->trace_cap;
+        COS_CUDA(cudaMemsetAsync(g->d_trace, 0, sizeof(unsigned long long) * 2 * g->trace_cap, st), "reset trace");
+    }
+    COS_CUDA(cudaMemsetAsync(g->d_ctrl, 0, sizeof(Ctrl), st), "reset control block");
+    if (tn.schedule == 2) {
+        rc = launch_windowed(g, &g->wave, km, per_sample_out, tn, st);
+        // (a plan that finds no memory has enqueued nothing)
+        if (rc == COS_ERR_OOM && g->d_ptab && !no_plan) return evaluate_general(g, km, per_sample_out, mean_out, st, true);
+        if (rc != COS_OK) return rc;
+        g->last_wave = 1;
+    } else {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
+        const int grid = sms * tn.blocks_per_sm;
+        char msg[256] = {0};
+        rc = launch_walk(km, tn.samples_per_lane, tn.layout, p, grid, st, msg, sizeof(msg));
+        if (rc != COS_OK) return fail(rc, "walker launch failed: %s", msg);
+        g->last_wave = 0;
+    }
+    g->last_mode = km;
+    g->last_status_pending = 1;
+    if (mean_out) return collect(g, mean_out, st);
+    return COS_OK;
+}
+
 int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean_out, void* stream) {
     if (!g) return fail(COS_ERR_INVALID, "graph is NULL");
     DeviceGuard dg(g->device);
@@ -1014,37 +1052,9 @@ int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean
             return mean_out ? collect(g, mean_out, st) : COS_OK;
         }
     }
-    WalkParams p;
-    cos_tuning tn;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    g->capturing = g->d_ptab && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
-    int rc = cosgpu::prepare_walk(g, km, nullptr, per_sample_out, &p, &tn);
-    g->capturing = false;
-    if (rc != COS_OK) return rc;
-    if (const char* env = getenv("COS_TEST_SKIP_BARRIER_PHASE")) p.skip_barrier_phase = atoi(env);
-    if (g->d_trace) {
-        p.trace = g->d_trace;
-        p.trace_cap = g->trace_cap;
-        COS_CUDA(cudaMemsetAsync(g->d_trace, 0, sizeof(unsigned long long) * 2 * g->trace_cap, st), "reset trace");
-    }
-    COS_CUDA(cudaMemsetAsync(g->d_ctrl, 0, sizeof(Ctrl), st), "reset control block");
-    if (tn.schedule == 2) {
-        rc = launch_windowed(g, &g->wave, km, per_sample_out, tn, st);
-        if (rc != COS_OK) return rc;
-        g->last_wave = 1;
-    } else {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device);
-        const int grid = sms * tn.blocks_per_sm;
-        char msg[256] = {0};
-        rc = launch_walk(km, tn.samples_per_lane, tn.layout, p, grid, st, msg, sizeof(msg));
-        if (rc != COS_OK) return fail(rc, "walker launch failed: %s", msg);
-        g->last_wave = 0;
-    }
-    g->last_mode = km;
-    g->last_status_pending = 1;
-    if (mean_out) return collect(g, mean_out, st);
-    return COS_OK;
+    const bool captured = g->d_ptab && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone;
+    return evaluate_general(g, km, per_sample_out, mean_out, st, captured);
 }
 
 int cos_set_trace(cos_graph_t g, int32_t capacity) {

@@ -5,6 +5,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
+from workloads import medium  # noqa: E402
 from workloads.generate import BETA, FaninSpec, make_graph  # noqa: E402
 
 pytestmark = pytest.mark.gpu
@@ -74,3 +75,26 @@ def test_work_queue_after_a_failed_growth(cg, monkeypatch):
     assert [g.evaluate(0) for g in (h, big)] == refs
     h.close()
     big.close()
+
+
+def test_tabulated_evaluation_without_memory_for_a_plan(cg, monkeypatch):
+    # FP64 with tables takes the work queue for its speed alone: without memory for its plan
+    # the level-synchronous kernel, which needs none, evaluates as it does from the same samples
+    wl = medium(num_samples=8192)
+    s = wl.samples
+    table = 0.5 * np.tanh(np.random.default_rng(7).normal(size=(wl.graph.num_kinds, 2, 18)))
+    gr = cg.Graph.from_workload_graph(wl.graph)
+    gr.set_propagator_table(table, s.beta)
+    gr.set_samples(torch.from_numpy(s.t).cuda(), s.eps, s.beta, cg.COS_T_SAMPLE_MAJOR)
+    assert not gr.info()["on_chip"] & 1 and gr.get_tuning(0)["schedule"] == 2
+    out, ref = (torch.empty(8192, dtype=torch.float64, device="cuda") for _ in range(2))
+    gr.set_tuning(schedule=1)
+    mean = gr.evaluate(0, out=ref)
+    gr.set_tuning()
+    monkeypatch.setenv("COS_TEST_FAIL_ALLOC", "1")
+    assert gr.evaluate(0, out=out) == mean
+    assert torch.equal(out, ref)
+    monkeypatch.delenv("COS_TEST_FAIL_ALLOC")
+    assert gr.evaluate(0, out=out) == mean
+    assert torch.equal(out, ref)
+    gr.close()
