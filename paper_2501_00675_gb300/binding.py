@@ -38,7 +38,7 @@ COS_T_BORROW = 4
 EXPORTED = ["cos_create_graph", "cos_set_samples", "cos_evaluate", "cos_get_result", "cos_graph_info",
             "cos_set_tuning", "cos_get_tuning", "cos_set_trace", "cos_get_trace", "cos_evaluate_static",
             "cos_graph_share", "cos_batch_create", "cos_batch_reset", "cos_batch_set_tuning", "cos_batch_get_tuning", "cos_batch_autotune",
-            "cos_batch_launch", "cos_batch_results", "cos_batch_destroy", "cos_evaluate_batch",
+            "cos_batch_launch", "cos_batch_results", "cos_batch_info", "cos_batch_destroy", "cos_evaluate_batch",
             "cos_selftest_exp", "cos_probe_fma_rate", "cos_set_samples_uniform", "cos_copy_times", "cos_server_create",
             "cos_server_submit", "cos_server_poll", "cos_server_wait", "cos_server_stats", "cos_server_destroy",
             "cos_destroy", "cos_last_error"]
@@ -113,6 +113,7 @@ def load_library(build_if_missing: bool = False):
         lib.cos_batch_autotune.argtypes = [vp, vp, ctypes.POINTER(CosTuning)]
         lib.cos_batch_launch.argtypes = [vp, vp]
         lib.cos_batch_results.argtypes = [vp, vp, vp]
+        lib.cos_batch_info.argtypes = [vp, vp, i32]
         lib.cos_batch_destroy.argtypes = [vp]
         lib.cos_evaluate_batch.argtypes = [i32, vp, vp, vp, vp, vp]
         lib.cos_selftest_exp.argtypes = [vp, i64, vp, vp, vp, vp]
@@ -386,6 +387,11 @@ class Batch:
 
     def launch(self, stream=None):
         _check(load_library().cos_batch_launch(self._h, _stream_handle(stream)))
+
+    def info(self) -> dict:
+        arr = np.zeros(2, dtype=np.int64)
+        _check(load_library().cos_batch_info(self._h, _ptr(arr), 2))
+        return {"members": int(arr[0]), "on_chip": int(arr[1])}
 
     def results(self, stream=None, allow_overflow: bool = False) -> np.ndarray:
         """Each graph's mean ([n]); [n][2] (mean R, mean A) for a COS_EVAL_ABS batch."""

@@ -844,6 +844,14 @@ int cos_batch_autotune(cos_batch_t b, void* stream, cos_tuning* best_out) {
     return rc;
 }
 
+int cos_batch_info(cos_batch_t b, int64_t* info, int32_t n) {
+    if (!b || !info || n < 0) return set_error(COS_ERR_INVALID, "bad arguments");
+    if (!b->planned) return set_error(COS_ERR_STATE, "batch has not been launched");
+    const int64_t v[2] = {b->n, (int64_t)b->chip.size()};
+    for (int32_t q = 0; q < n && q < 2; ++q) info[q] = v[q];
+    return COS_OK;
+}
+
 int cos_batch_destroy(cos_batch_t b) {
     if (!b) return COS_OK;
     {
