@@ -18,9 +18,7 @@ struct ChipGraph {
     int32_t nsink = 0;
     int32_t max_width = 0;          // 0: the graph has no schedule
     int32_t tail_width = 0;         // width of the level before the sink
-    int32_t phase_rows = 0;
     int32_t tables = 0;             // 16-byte units of lev
-    int32_t pad = 0;
     int64_t edges = 0, rows = 0;
 };
 

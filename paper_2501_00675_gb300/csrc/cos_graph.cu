@@ -7,8 +7,10 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <future>
 #include <memory>
 #include <string>
+#include <system_error>
 #include <vector>
 
 #include "cos_chip.cuh"
@@ -221,56 +223,95 @@ void alloc_means(cos_graph* g) {
         cudaGetLastError();   // the control block serves without it
 }
 
-// Row schedule of the on-chip walk for a graph whose levels fit shared memory (none
-// otherwise: the graph is evaluated by the general kernels alone).
-cudaError_t upload_chip(cos_graph* g, const std::vector<int32_t>& row_ptr, const std::vector<int2>& csr,
-                        const std::vector<int32_t>& slot_kij, SharedArrays& a) {
+// Row schedule of the on-chip walk for a graph whose levels fit shared memory (bytes empty
+// otherwise: the graph is evaluated by the general kernels alone), as it goes to the device:
+// levels and group descriptors, edge words, slots, sink.
+struct ChipImage {
+    std::vector<char> bytes;
+    size_t words_at = 0, slots_at = 0, sink_at = 0;
+    int32_t units = 0, nsink = 0, max_width = 0;
+};
+
+ChipImage make_chip(int32_t L, int32_t K, int32_t D, const std::vector<int64_t>& off, const std::vector<int32_t>& row_ptr,
+                    const std::vector<int2>& csr, const std::vector<int32_t>& slot_kij) {
+    ChipImage im;
+    const int64_t P = (int64_t)slot_kij.size() / 3;
     int64_t wmax = 1;
-    for (int32_t l = 0; l + 1 < g->L; ++l) wmax = std::max(wmax, g->widths[(size_t)l]);
-    if ((int64_t)g->K * g->D > 65535 || g->K > 32767 || g->D > kChipMaxTimes) return cudaSuccess;   // 16-bit slot factors
-    const int phase = chip_phase_rows(wmax, g->P, g->K, g->D);
-    if (phase == 0) return cudaSuccess;
+    for (int32_t l = 0; l + 1 < L; ++l) wmax = std::max(wmax, off[(size_t)l + 1] - off[(size_t)l]);
+    if ((int64_t)K * D > 65535 || K > 32767 || D > kChipMaxTimes) return im;   // 16-bit slot factors
+    const int phase = chip_phase_rows(wmax, P, K, D);
+    if (phase == 0) return im;
     ChipSchedule cs;
-    if (!build_chip(g->L, g->off.data(), row_ptr.data(), g->P, phase, [&](int32_t q) { return csr[(size_t)q].x; },
+    if (!build_chip(L, off.data(), row_ptr.data(), P, phase, [&](int32_t q) { return csr[(size_t)q].x; },
                     [&](int32_t q) { return csr[(size_t)q].y; }, cs))
-        return cudaSuccess;
-    // one allocation: levels and group descriptors, edge words, slots, sink
+        return im;
     static_assert(sizeof(ChipLevel) == sizeof(int4), "read as int4");
     const size_t units = cs.lev.size() + (cs.grp.size() + 3) / 4;
-    const size_t words_at = units * sizeof(int4), slots_at = words_at + (cs.words.size() * 4 + 15) / 16 * 16,
-                 sink_at = slots_at + (size_t)g->P * sizeof(uint2), bytes = sink_at + cs.sink.size() * 4;
-    std::vector<char> h(bytes + 16);
-    memcpy(h.data(), cs.lev.data(), cs.lev.size() * sizeof(int4));
-    if (!cs.grp.empty()) memcpy(h.data() + cs.lev.size() * sizeof(int4), cs.grp.data(), cs.grp.size() * 4);
-    if (!cs.words.empty()) memcpy(h.data() + words_at, cs.words.data(), cs.words.size() * 4);
-    if (!cs.sink.empty()) memcpy(h.data() + sink_at, cs.sink.data(), cs.sink.size() * 4);
-    uint2* slots = reinterpret_cast<uint2*>(h.data() + slots_at);
-    for (int64_t q = 0; q < g->P; ++q) {
+    im.words_at = units * sizeof(int4);
+    im.slots_at = im.words_at + (cs.words.size() * 4 + 15) / 16 * 16;
+    im.sink_at = im.slots_at + (size_t)P * sizeof(uint2);
+    im.units = (int32_t)units;
+    im.nsink = (int32_t)cs.sink.size();
+    im.max_width = cs.max_width;
+    im.bytes.resize(im.sink_at + cs.sink.size() * 4 + 16);
+    char* h = im.bytes.data();
+    memcpy(h, cs.lev.data(), cs.lev.size() * sizeof(int4));
+    if (!cs.grp.empty()) memcpy(h + cs.lev.size() * sizeof(int4), cs.grp.data(), cs.grp.size() * 4);
+    if (!cs.words.empty()) memcpy(h + im.words_at, cs.words.data(), cs.words.size() * 4);
+    if (!cs.sink.empty()) memcpy(h + im.sink_at, cs.sink.data(), cs.sink.size() * 4);
+    uint2* slots = reinterpret_cast<uint2*>(h + im.slots_at);
+    for (int64_t q = 0; q < P; ++q) {
         const uint32_t k = (uint32_t)slot_kij[(size_t)(3 * q)], i = (uint32_t)slot_kij[(size_t)(3 * q + 1)],
-                       jw = (uint32_t)slot_kij[(size_t)(3 * q + 2)], j = jw & (uint32_t)kKindMask, D = (uint32_t)g->D;
-        slots[q] = make_uint2((k * D + i) | (k * D + j) << 16, (i * D + j) | k << 16 | ((jw & (uint32_t)kSignBit) << 1));
+                       jw = (uint32_t)slot_kij[(size_t)(3 * q + 2)], j = jw & (uint32_t)kKindMask, d = (uint32_t)D;
+        slots[q] = make_uint2((k * d + i) | (k * d + j) << 16, (i * d + j) | k << 16 | ((jw & (uint32_t)kSignBit) << 1));
     }
-    cudaError_t e = cudaMalloc(&a.chip, h.size());
+    return im;
+}
+
+cudaError_t upload_chip(cos_graph* g, const ChipImage& im, SharedArrays& a) {
+    if (im.bytes.empty()) return cudaSuccess;
+    cudaError_t e = cudaMalloc(&a.chip, im.bytes.size());
     if (e == cudaErrorMemoryAllocation) {   // the general kernels need none of this
         cudaGetLastError();
         a.chip = nullptr;
         return cudaSuccess;
     }
-    if (e == cudaSuccess) e = cudaMemcpy(a.chip, h.data(), h.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(a.chip, im.bytes.data(), im.bytes.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
     ChipGraph& c = g->chip;
     c.lev = reinterpret_cast<const int4*>(a.chip);
-    c.words = reinterpret_cast<const uint32_t*>(a.chip + words_at);
-    c.slots = reinterpret_cast<const uint2*>(a.chip + slots_at);
-    c.sink = reinterpret_cast<const uint32_t*>(a.chip + sink_at);
-    c.nsink = (int32_t)cs.sink.size();
-    c.max_width = cs.max_width;
+    c.words = reinterpret_cast<const uint32_t*>(a.chip + im.words_at);
+    c.slots = reinterpret_cast<const uint2*>(a.chip + im.slots_at);
+    c.sink = reinterpret_cast<const uint32_t*>(a.chip + im.sink_at);
+    c.nsink = im.nsink;
+    c.max_width = im.max_width;
     c.tail_width = (int32_t)g->widths[(size_t)g->L - 2];
-    c.tables = (int32_t)units;
-    c.phase_rows = cs.phase_rows;
+    c.tables = im.units;
     c.edges = g->E;
     c.rows = g->N;
     return cudaSuccess;
+}
+
+// 2^{j/64} and 2^{-j/64}, j = 0..63, for the table-driven exponentials, followed by the same
+// values as float-float pairs (hi, lo) for the FP32 path.  (Made once: 128 long double powers
+// take 59 us on a Grace core.)
+const std::vector<double>& exp_table() {
+    static const std::vector<double> table = [] {
+        std::vector<double> tab(128 + 128);
+        float* tff = reinterpret_cast<float*>(tab.data() + 128);
+        for (int j = 0; j < 64; ++j) {
+            const long double vp = std::exp2l((long double)j / 64.0L), vm = std::exp2l(-(long double)j / 64.0L);
+            tab[(size_t)j] = (double)vp;
+            tab[(size_t)j + 64] = (double)vm;
+            const float hp = (float)vp, hm = (float)vm;
+            tff[2 * j] = hp;
+            tff[2 * j + 1] = (float)(vp - (long double)hp);
+            tff[2 * (64 + j)] = hm;
+            tff[2 * (64 + j) + 1] = (float)(vm - (long double)hm);
+        }
+        return tab;
+    }();
+    return table;
 }
 
 // The on-chip walk serves evaluations whose launch shape is left to the library; a
@@ -412,6 +453,16 @@ int cos_create_graph(int32_t num_levels, const int64_t* level_width, const int64
     row_ptr[(size_t)N] = (int32_t)E;   // (root row: row_ptr[0] = row_ptr[1] = 0)
     row_ptr[0] = 0;
 
+    // The row schedule of the on-chip walk, on another thread beside the path count and the
+    // uploads where it is long (medium graph: 0.8 ms, of which 0.45 are hidden: creation 1.28).
+    auto schedule = [&] { return make_chip(L, num_kinds, num_times, off, row_ptr, csr, slot_kij); };
+    std::future<ChipImage> chip;
+    try {
+        chip = std::async(N < 4096 ? std::launch::deferred : std::launch::async, schedule);
+    } catch (const std::system_error&) {   // no thread to be had
+        chip = std::async(std::launch::deferred, schedule);
+    }
+
     // Exact path count (unit weights), 128-bit with saturation, for the overflow flag.
     std::vector<unsigned __int128> cexact((size_t)N, 0);
     std::vector<uint64_t> cwrap((size_t)N, 0);
@@ -463,20 +514,7 @@ int cos_create_graph(int32_t num_levels, const int64_t* level_width, const int64
         std::vector<int32_t> ks((size_t)num_kinds + 1, 0);
         for (int64_t q = 0; q < P; ++q) ks[(size_t)slot_kij[3 * q] + 1]++;
         for (int32_t k = 0; k < num_kinds; ++k) ks[(size_t)k + 1] += ks[(size_t)k];
-        // 2^{j/64} and 2^{-j/64}, j = 0..63, for the table-driven exponentials
-        // followed by the same values as float-float pairs (hi, lo) for the FP32 path
-        std::vector<double> tab(128 + 128);
-        float* tff = reinterpret_cast<float*>(tab.data() + 128);
-        for (int j = 0; j < 64; ++j) {
-            const long double vp = std::exp2l((long double)j / 64.0L), vm = std::exp2l(-(long double)j / 64.0L);
-            tab[(size_t)j] = (double)vp;
-            tab[(size_t)j + 64] = (double)vm;
-            const float hp = (float)vp, hm = (float)vm;
-            tff[2 * j] = hp;
-            tff[2 * j + 1] = (float)(vp - (long double)hp);
-            tff[2 * (64 + j)] = hm;
-            tff[2 * (64 + j) + 1] = (float)(vm - (long double)hm);
-        }
+        const std::vector<double>& tab = exp_table();
         if ((e = cudaMalloc(&g->d_kind_slot, sizeof(int32_t) * (num_kinds + 1))) != cudaSuccess) return cleanup_fail(e, "cudaMalloc kind slots");
         if ((e = cudaMalloc(&g->d_exp_tab, sizeof(double) * tab.size())) != cudaSuccess) return cleanup_fail(e, "cudaMalloc exp table");
         if ((e = cudaMemcpy(g->d_kind_slot, ks.data(), sizeof(int32_t) * (num_kinds + 1), cudaMemcpyHostToDevice)) != cudaSuccess) return cleanup_fail(e, "copy kind slots");
@@ -489,7 +527,7 @@ int cos_create_graph(int32_t num_levels, const int64_t* level_width, const int64
     if ((e = cudaMemset(g->d_ctrl, 0, sizeof(Ctrl))) != cudaSuccess) return cleanup_fail(e, "memset ctrl");
     auto arr = std::make_shared<SharedArrays>();
     arr->device = g->device;
-    if ((e = upload_chip(g, row_ptr, csr, slot_kij, *arr)) != cudaSuccess) return cleanup_fail(e, "on-chip row schedule");
+    if ((e = upload_chip(g, chip.get(), *arr)) != cudaSuccess) return cleanup_fail(e, "on-chip row schedule");
     arr->levels = g->d_levels;
     arr->row_ptr = g->d_row_ptr;
     arr->edges = g->d_edges;
