@@ -254,6 +254,40 @@ def profiled_traffic(kernel_tag: str, samples: int, schedule: int, layout: int):
     return v["bytes_per_launch"] * samples / v["samples"]
 
 
+SMEM_BYTES_PER_CLK_SM = 128.0    # shared-memory bandwidth of an SM (nominal)
+
+
+def smem_peak(sms: int):
+    """Shared-memory bandwidth of the device in GB/s at its maximum SM clock."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            mhz = float(json.load(f)["sm_max_mhz"])
+    except (OSError, KeyError, ValueError):
+        mhz = 2070.0
+    return (SMEM_BYTES_PER_CLK_SM * sms * mhz * 1e6 / 1e9,
+            f"nominal: {sms} SMs x {SMEM_BYTES_PER_CLK_SM:g} bytes/clk x {mhz:g} MHz")
+
+
+def memory_roofline(mode: int, with_abs: bool, E: int, N: int, S: int, D: int, seconds: float, on_chip: bool,
+                    traffic, sms: int):
+    """The memory bound of one walk.  In the workspace every node value is written and read
+    once in HBM; on chip none leaves the SM, and what is moved is the parent and the
+    propagator of every edge and sample, out of shared memory."""
+    if on_chip:
+        operands = {0: 16, 1: 12 if with_abs else 8, 2: 8}[mode]
+        moved, (peak, source) = float(E) * S * operands, smem_peak(sms)
+        return {"bound": "smem", "achieved": moved / seconds / 1e9, "peak": peak, "unit": "GB/s",
+                "frac": moved / seconds / 1e9 / peak, "peak_source": source, "traffic": None,
+                "operand_bytes_per_launch": moved}
+    moved = S * (2.0 * N * (4 if mode == 1 else 8) + D * 8 + 8)
+    if with_abs:                                                        # A's float node values and result
+        moved += S * (2.0 * N * 4 + 8)
+    peak, kind = hbm_peak()
+    return {"bound": "hbm", "achieved": moved / seconds / 1e9, "peak": peak, "unit": "GB/s",
+            "frac": moved / seconds / 1e9 / peak, "peak_source": f"{kind} (MEASURED_PEAKS.json hbm_gbs)"
+            if kind == "measured" else "fallback 6.8 TB/s", "traffic": traffic, "algorithmic_bytes_per_launch": moved}
+
+
 # ------------------------------------------------------------------ CPU oracle timing
 
 def oracle_rate(graph, samples, seconds: float, nthreads: int = 0):
@@ -320,7 +354,6 @@ def run_ours(args, rank, world, local):
     gr.get_result(stream)
     torch.cuda.synchronize()
     tuning = gr.get_tuning(emode)
-    # (the profiled DRAM traffic is the workspace kernels'; the on-chip walk has next to none)
     on_chip = bool(gr.info()["on_chip"] >> (4 if mode == 1 and args.abs else mode) & 1) and not (mode == 0 and args.abs)
 
     uuid = None
@@ -353,28 +386,20 @@ def run_ours(args, rank, world, local):
     value = units / total_s
 
     # roofline of the walker kernel (one launch per evaluate)
-    w_bytes = 4 if mode == 1 else 8
-    alg_bytes = S * (2.0 * N * w_bytes + D * 8 + 8)
-    if args.abs:                                                        # A's float node values and result
-        alg_bytes += S * (2.0 * N * 4 + 8)
     walk_s = statistics.mean(walk_ms) / 1e3
-    peak, peak_kind = hbm_peak()
-    hbm = {"bound": "hbm", "achieved": alg_bytes / walk_s / 1e9, "peak": peak, "unit": "GB/s",
-           "frac": alg_bytes / walk_s / 1e9 / peak, "peak_source": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)"
-           if peak_kind == "measured" else "fallback 6.8 TB/s",
-           "traffic": None if on_chip else
-           profiled_traffic(f"walk_{mode_name}{'_abs' if args.abs else ''}_{args.workload}",
-                            S, tuning["schedule"], tuning["layout"]),
-           "algorithmic_bytes_per_launch": alg_bytes}
+    memory = memory_roofline(mode, bool(args.abs), E, N, S, D, walk_s, on_chip,
+                             profiled_traffic(f"walk_{mode_name}{'_abs' if args.abs else ''}_{args.workload}",
+                                              S, tuning["schedule"], tuning["layout"]),
+                             torch.cuda.get_device_properties(dev).multi_processor_count)
     if mode == 0:
         tflops = 2.0 * E * S / walk_s / 1e12
         fp64_peak, fp64_src = fp64_fma_peak(cg, local)
         alu = {"bound": "alu", "achieved": tflops, "peak": fp64_peak, "unit": "TFLOP/s",
                "frac": tflops / fp64_peak, "peak_source": fp64_src,
-               "traffic": hbm["traffic"], "algorithmic_flops_per_launch": 2.0 * E * S}
-        roofline, other = (alu, hbm) if alu["frac"] >= hbm["frac"] else (hbm, alu)
+               "traffic": memory["traffic"], "algorithmic_flops_per_launch": 2.0 * E * S}
+        roofline, other = (alu, memory) if alu["frac"] >= memory["frac"] else (memory, alu)
     else:
-        roofline, other = hbm, None
+        roofline, other = memory, None
 
     # end to end through the public API with host buffers
     e2e = None
@@ -520,6 +545,7 @@ def run_batched(args, rank, world, local):
     barrier(world)
     step_ms = max_over_ranks(e0.elapsed_time(e1) / 1e3, world, local) * 1e3 / max(args.steps, 1)
     b.results(stream)
+    plan = b.info()
     # the timed launch's first samples of every graph, kept for the oracle check below
     n_chk = BATCH_CHECK_SAMPLES
     got = [o[:min(n_chk, w.samples.num_samples)].cpu().numpy() for o, w in zip(outs, wls)]
@@ -545,7 +571,7 @@ def run_batched(args, rank, world, local):
     t_b = step_ms / 1e3
     w_bytes = 4 if mode == 1 else 8
     alg_bytes = float(sum(w.samples.num_samples * (2.0 * w.graph.num_nodes * w_bytes + 8 * w.graph.num_times + 8)
-                          for w in wls))
+                          for w in wls)) - 2.0 * w_bytes * plan["on_chip_values"]   # (those never leave an SM)
     peak, peak_kind = hbm_peak()
     roofline = {"bound": "hbm", "achieved": alg_bytes / t_b / 1e9, "peak": peak, "unit": "GB/s",
                 "frac": alg_bytes / t_b / 1e9 / peak, "traffic": None,
@@ -555,7 +581,8 @@ def run_batched(args, rank, world, local):
         "metric": "edge·sample updates/s", "value": units * world / t_b, "unit": "edge·sample updates/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": step_ms, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": DTYPE[args.mode or "mixed"], "data": "synthetic",
-        "config": {"workload": batched_desc(len(wls)), "autotuned": best, "generation_s": gen_s,
+        "config": {"workload": batched_desc(len(wls)), "autotuned": best,
+                   "members_on_chip": plan["on_chip"], "generation_s": gen_s,
                    "edge_samples": units, "l2": "no flush: every step's working set is GBs of node values"},
         "roofline": roofline, "gpu_launches": args.steps,
         "sequential_ms": min(seq), "batched_speedup_vs_sequential": min(seq) / step_ms,

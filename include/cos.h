@@ -401,7 +401,8 @@ int cos_batch_get_tuning(cos_batch_t b, cos_tuning* tuning);
 int cos_batch_autotune(cos_batch_t b, void* stream, cos_tuning* best);
 int cos_batch_launch(cos_batch_t b, void* stream);
 int cos_batch_results(cos_batch_t b, double* means, void* stream);
-/* The last launch's plan, written to info[0..n) (n <= 2): members, members that run on chip. */
+/* The last launch's plan, written to info[0..n) (n <= 3): members, members that run on chip,
+ * node values (nodes x samples) of the latter. */
 int cos_batch_info(cos_batch_t b, int64_t* info, int32_t n);
 int cos_batch_destroy(cos_batch_t b);
 int cos_evaluate_batch(int32_t n, const cos_graph_t* graphs, const int32_t* modes, void* const* per_sample_outs,

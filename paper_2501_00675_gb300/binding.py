@@ -389,9 +389,10 @@ class Batch:
         _check(load_library().cos_batch_launch(self._h, _stream_handle(stream)))
 
     def info(self) -> dict:
-        arr = np.zeros(2, dtype=np.int64)
-        _check(load_library().cos_batch_info(self._h, _ptr(arr), 2))
-        return {"members": int(arr[0]), "on_chip": int(arr[1])}
+        """The last launch's plan: members, how many run on chip, and their nodes x samples."""
+        arr = np.zeros(3, dtype=np.int64)
+        _check(load_library().cos_batch_info(self._h, _ptr(arr), 3))
+        return {"members": int(arr[0]), "on_chip": int(arr[1]), "on_chip_values": int(arr[2])}
 
     def results(self, stream=None, allow_overflow: bool = False) -> np.ndarray:
         """Each graph's mean ([n]); [n][2] (mean R, mean A) for a COS_EVAL_ABS batch."""

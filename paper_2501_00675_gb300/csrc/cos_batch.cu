@@ -847,8 +847,10 @@ int cos_batch_autotune(cos_batch_t b, void* stream, cos_tuning* best_out) {
 int cos_batch_info(cos_batch_t b, int64_t* info, int32_t n) {
     if (!b || !info || n < 0) return set_error(COS_ERR_INVALID, "bad arguments");
     if (!b->planned) return set_error(COS_ERR_STATE, "batch has not been launched");
-    const int64_t v[2] = {b->n, (int64_t)b->chip.size()};
-    for (int32_t q = 0; q < n && q < 2; ++q) info[q] = v[q];
+    int64_t values = 0;
+    for (const ChipParams& p : b->chip) values += p.g.rows * p.S;
+    const int64_t v[3] = {b->n, (int64_t)b->chip.size(), values};
+    for (int32_t q = 0; q < n && q < 3; ++q) info[q] = v[q];
     return COS_OK;
 }
 

@@ -61,7 +61,8 @@ def test_batch_members_that_run_on_chip(cg, mode):  # noqa: F811
             o.fill_(-1)
         b.launch()
         means = b.results()
-        assert b.info() == {"members": 4, "on_chip": 3}
+        assert b.info() == {"members": 4, "on_chip": 3,
+                            "on_chip_values": 6 * 5000 + 122 * 3000 + 762 * 400}
         for o, m, ref in zip(outs, means, refs):
             np.testing.assert_array_equal(o.cpu().numpy(), ref[0])
             assert tuple(np.atleast_1d(m)) == tuple(np.atleast_1d(ref[1]))
