@@ -336,8 +336,10 @@ int cos_get_tuning(cos_graph_t g, int32_t mode, cos_tuning* tuning);
  * rows per warp, two vector widths; fields already set > 0 stay fixed), keep the
  * fastest as g's tuning and, if best is non-NULL, store its resolved form there.
  * An evaluation that the automatic shape runs on chip is timed too, and the shape stays
- * automatic when that is the fastest.  Runs 39 evaluations at most on `stream` (writing per_sample_out, which may be
- * NULL) and synchronizes; results are bitwise the same for every candidate.
+ * automatic when that is the fastest (*best is then the shape that it would have off chip,
+ * as in cos_get_tuning; setting it would take the evaluation off the chip).  Runs 39
+ * evaluations at most on `stream` (writing per_sample_out, which may be NULL) and
+ * synchronizes; results are bitwise the same for every candidate.
  * The paper has no counterpart; cos_batch_autotune does the same for batches.
  */
 int cos_autotune(cos_graph_t g, int32_t mode, void* per_sample_out, void* stream, cos_tuning* best);
@@ -374,7 +376,9 @@ int cos_autotune(cos_graph_t g, int32_t mode, void* per_sample_out, void* stream
  *                     prefetch; other fields come from each graph.
  *   cos_batch_autotune  times every (samples_per_lane, rows_per_warp, layout)
  *                     candidate on the batch itself (and the automatic shape, where it
- *                     runs members on chip), keeps the fastest and returns it in *best.
+ *                     runs members on chip), keeps the fastest and returns it in *best --
+ *                     or, when the automatic shape stays, the one the members off
+ *                     chip have then (cos_batch_info tells whether any are on chip).
  *   cos_batch_launch  enqueue one evaluation of all graphs on `stream`.  The first
  *                     launch of a plan uploads it (stream-ordered) and runs the
  *                     kernel directly; the second captures counter reset + kernel
