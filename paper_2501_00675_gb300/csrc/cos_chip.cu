@@ -1167,6 +1167,8 @@ bool chip_plan(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, i
     bool found = false;
     for (int rb = std::max(nb, 4); rb <= 128; rb *= 2) {
         const int lane = std::min(kmode == kModeMixedAbs ? rb / 2 : rb, 16);   // (a piece is wholly R or wholly A)
+        // the chunks of a launch, those of a batch's members together, are counted in 32 bits
+        if ((S + rb / nb - 1) / (rb / nb) > (INT32_MAX - (1 << 20)) / std::max(members, 1)) continue;
         for (int ctas = 1; ctas <= 4; ctas *= 2) {
             const ChipLayout y = chip_layout(g, kmode, P, K, D, table, rb, smem_limit(ctas));
             if (y.total > smem_limit(ctas) || 512 / ctas / 32 < rb / lane) continue;   // (a group needs rb / lane warps)

@@ -124,3 +124,15 @@ def test_captured_sample_sets_read_the_energies_at_replay(cg):  # noqa: F811
         torch.cuda.synchronize()
         np.testing.assert_array_equal(out.cpu().numpy(), want)
     gr.close()
+
+
+@pytest.mark.parametrize("S,on_chip", [(4 << 30, True), (8 << 30, False)])
+def test_chunks_beyond_32_bits_stay_off_chip(cg, S, on_chip):  # noqa: F811
+    # levels of 8,000 rows: four FP32 samples per chunk (nothing is evaluated: the times, borrowed,
+    # are not there)
+    g = make_graph([1, 100, 8000, 8000, 8000, 100, 1], FaninSpec("uniform", 4), 6, 1, np.random.default_rng(2))
+    gr = cg.Graph.from_workload_graph(g)
+    t = torch.zeros(128, dtype=torch.float64, device="cuda")
+    gr.set_samples(t, np.zeros(6), BETA, cg.COS_T_BORROW, num_samples=S)
+    assert _on_chip(cg, gr, 1) == on_chip
+    gr.close()
