@@ -442,13 +442,13 @@ int cos_get_trace(cos_graph_t g, int64_t* out, int32_t capacity, int32_t* count)
  * partial sums of the sample reduction, the grid-barrier counter, the error word
  * and the result -- lives in one file-scope __device__ array of
  * COS_STATIC_SCRATCH_BYTES (64 MiB) inside the library; every GPU that loads the
- * library holds it until the process exits.  A second one of 32 KiB holds the
+ * library holds it until the process exits.  A second one of 16 KiB holds the
  * arrival counters of the on-chip kernel (cos_evaluate), which leaves only its
  * partial sums and result in the first.  The function calls no cudaMalloc,
  * cudaFree or other allocating routine.  The barrier counter and result are
- * cleared on every call that does not run on chip; the arrival counters carry the
- * number of their launch (captured launches clear them); the rest keeps the last
- * call's contents and is overwritten before use.  Every call on a device shares the
+ * cleared on every call that does not run on chip; the arrival counters are left at
+ * zero, or else found out by the next call; the rest keeps the last call's contents
+ * and is overwritten before use.  Every call on a device shares the
  * arrays, so calls whose execution overlaps on the GPU (different streams, or host
  * threads) race and give wrong results: serialise them.  Later calls that do not
  * overlap are not affected.  Set-up: the first call on a device,

@@ -40,10 +40,9 @@ struct BatchCtrl {
     int err;
     int err_task;
     unsigned chip_ticket[kChipLaunches];
+    unsigned long long chip_exits[kChipLaunches];
 };
-// Arrival words of the members on chip (ChipParams::arrive) lie behind it and are cleared
-// with it; word 0 of a launch's first member counts the launch's CTAs.
-static_assert(sizeof(BatchCtrl) % sizeof(unsigned long long) == 0, "the words behind it are aligned");
+// (behind it, cleared with it: arrival words of the members on chip, ChipParams::arrive)
 
 struct BatchArgs {
     const Task* tasks;
@@ -352,7 +351,7 @@ int ensure_capacity(cos_batch* b, size_t ntasks, size_t ngraphs, size_t njoins, 
         cudaFree(b->d_ctrl);
         b->d_ctrl = nullptr;
         char* block = nullptr;
-        if ((e = device_buffer(&block, sizeof(BatchCtrl) + sizeof(unsigned long long) * cap)) != cudaSuccess)
+        if ((e = device_buffer(&block, sizeof(BatchCtrl) + sizeof(unsigned) * cap)) != cudaSuccess)
             return no_room("batch control", e);
         b->d_ctrl = reinterpret_cast<BatchCtrl*>(block);
         b->cap_words = cap;
@@ -494,7 +493,7 @@ int plan(cos_batch* b) {
     b->resolved.blocks_per_sm = bps;
     b->grid = sms * bps;
     size_t words = 0;
-    for (const OnChip& oc : on_chip) words += 1 + (size_t)((oc.p.S + kReduceBlock - 1) / kReduceBlock);
+    for (const OnChip& oc : on_chip) words += (size_t)((oc.p.S + kReduceBlock - 1) / kReduceBlock);
     int rc = ensure_capacity(b, std::max<size_t>(b->tasks.size(), 1), std::max<int32_t>(b->n, 1),
                              std::max<size_t>(b->joins.size(), 1), words);
     if (rc != COS_OK) return rc;
@@ -507,8 +506,8 @@ int plan(cos_batch* b) {
     });
     b->chip.clear();
     b->chip_launches.clear();
-    b->ctrl_bytes = sizeof(BatchCtrl) + sizeof(unsigned long long) * words;
-    unsigned long long* arrive = reinterpret_cast<unsigned long long*>(b->d_ctrl + 1);
+    b->ctrl_bytes = sizeof(BatchCtrl) + sizeof(unsigned) * words;
+    unsigned* arrive = reinterpret_cast<unsigned*>(b->d_ctrl + 1);
     for (OnChip& oc : on_chip) {
         if (b->chip_launches.empty() || b->chip_launches.back().lane_bytes != oc.plan.lane_bytes ||
             b->chip_launches.back().threads != oc.plan.threads)
@@ -516,8 +515,10 @@ int plan(cos_batch* b) {
         cos_batch::ChipLaunch& cl = b->chip_launches.back();
         oc.p.mean_out = b->d_means + 2 * oc.g;
         oc.p.arrive = arrive;
-        oc.p.tag = kBatchTag;
-        arrive += 1 + (oc.p.S + kReduceBlock - 1) / kReduceBlock;
+        oc.p.exits = nullptr;
+        oc.p.tag = kClearedTag;
+        oc.p.arrive_cap = (int32_t)((oc.p.S + kReduceBlock - 1) / kReduceBlock);
+        arrive += oc.p.arrive_cap;
         oc.p.first_chunk = cl.chunks;
         cl.chunks += oc.p.nchunks;
         cl.n++;
@@ -556,7 +557,7 @@ int enqueue_run(cos_batch* b, cudaStream_t st) {
     for (size_t q = 0; q < b->chip_launches.size(); ++q) {
         const cos_batch::ChipLaunch& cl = b->chip_launches[q];
         const int rc = launch_chip_list(b->mode, cl.lane_bytes, cl.threads, cl.smem, b->d_chip + cl.first, cl.n, cl.chunks,
-                                        &b->d_ctrl->chip_ticket[q], b->chip[(size_t)cl.first].arrive, b->sms, st);
+                                        &b->d_ctrl->chip_ticket[q], &b->d_ctrl->chip_exits[q], b->sms, st);
         if (rc != COS_OK) return rc;
     }
     return COS_OK;

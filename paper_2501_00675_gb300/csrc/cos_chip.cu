@@ -146,7 +146,7 @@ struct ChipArgs {
     ChipParams one;
     const ChipParams* list;   // nullptr: `one`, chunks dealt out by CTA number
     unsigned* ticket;
-    unsigned long long* exits;   // CTAs that have left, under `tag`
+    unsigned long long* exits;   // CTAs that have left
     unsigned long long tag;
     int n, total;
     int tmem_cols;            // 0: no level goes through TMEM
@@ -615,16 +615,12 @@ __device__ __forceinline__ void cta_sum(double (&v)[kPerThread], const T* x, dou
         if (lane == 0) partials[b] = sum;
     }
 }
-// Arrival word of a block whose partial sum is written.  (A launch's own counts end at
-// kReduceBlock, 2^10: those of calls that overlap stay out of the tag and below this one.)
-__device__ __forceinline__ unsigned long long tagged(unsigned long long tag, unsigned n) { return tag << kTagShift | n; }
-constexpr unsigned kBlockSummed = 1u << (kTagShift - 1);
+constexpr unsigned kBlockSummed = 0xffffffffu;   // arrival word of a block whose partial sum is written
 
-// Partial sums of blocks [b, nblk) whose arrival word is not `summed` (arrive nullptr: of
-// all).
+// Partial sums of blocks [b, nblk) whose arrival word is not kBlockSummed (arrive
+// nullptr: of all).
 template <typename T>
-__device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S, int b, int nblk, const unsigned long long* arrive,
-                                         unsigned long long summed, CtaSum& c) {
+__device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S, int b, int nblk, const unsigned* arrive, CtaSum& c) {
     // the next block to sum: 32 arrival words at a time, read by one warp for all -- the loop
     // below has block barriers, and a launch that overlaps on the same words changes them
     __shared__ unsigned s_open;
@@ -637,7 +633,7 @@ __device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S
                 const int at = base + (int)(threadIdx.x & 31);
                 __syncthreads();   // everyone has the word before
                 if (threadIdx.x < 32) {
-                    const unsigned left = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != summed);
+                    const unsigned left = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != kBlockSummed);
                     if (threadIdx.x == 0) s_open = left;
                 }
                 __syncthreads();
@@ -662,27 +658,27 @@ __device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S
     }
 }
 template <int MODE>
-__device__ __noinline__ void chip_sums(const ChipParams& p, unsigned char* sm, int b, int nblk, bool all) {
-    const unsigned long long* arrive = all ? nullptr : p.arrive + 1;
-    const unsigned long long summed = tagged(p.tag, kBlockSummed);
+__device__ __noinline__ void chip_sums(const ChipParams& p, unsigned char* sm, int b, int nblk, const unsigned* arrive) {
     CtaSum& c = *reinterpret_cast<CtaSum*>(sm);   // (the level buffer, free by now)
-    if constexpr (Traits<MODE>::kCount) cta_sums(static_cast<const long long*>(p.R), p.partials, p.S, b, nblk, arrive, summed, c);
-    else cta_sums(static_cast<const double*>(p.R), p.partials, p.S, b, nblk, arrive, summed, c);
-    if constexpr (Traits<MODE>::kAbs) cta_sums(p.Rabs, p.partials_abs, p.S, b, nblk, arrive, summed, c);
+    if constexpr (Traits<MODE>::kCount) cta_sums(static_cast<const long long*>(p.R), p.partials, p.S, b, nblk, arrive, c);
+    else cta_sums(static_cast<const double*>(p.R), p.partials, p.S, b, nblk, arrive, c);
+    if constexpr (Traits<MODE>::kAbs) cta_sums(p.Rabs, p.partials_abs, p.S, b, nblk, arrive, c);
 }
 
 
-// Count a chunk's results in (one thread; they were written by its warp).  Called a
-// phase after the writes, when the release has nothing left to wait for.
+__device__ __forceinline__ unsigned long long ld_relaxed_gpu(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long tagged(unsigned long long tag, unsigned n) { return tag << kTagShift | n; }
+
+// Count a chunk's results in (one thread, after the writes and, unless it is one of theirs, a
+// block barrier).
 __device__ __forceinline__ void chip_arrive(const ChipParams& p, int chunk) {
     const int64_t s0 = (int64_t)chunk << p.s_log2;
     const unsigned mine = (unsigned)min((int64_t)1 << p.s_log2, p.S - s0);
-    unsigned long long* w = p.arrive + 1 + s0 / kReduceBlock;
-    // (an older launch's count is below every word of this one's tag; a newer one's, met only
-    // where launches run in another order than they were made, stays, and then the last CTA
-    // sums the block)
-    asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(w), "l"(tagged(p.tag, 0u)) : "memory");
-    asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(w), "l"((unsigned long long)mine) : "memory");
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.arrive + s0 / kReduceBlock), "r"(mine) : "memory");
 }
 
 __device__ __forceinline__ int chip_blocks(const ChipParams& p) { return (int)((p.S + kReduceBlock - 1) / kReduceBlock); }
@@ -690,22 +686,32 @@ __device__ __forceinline__ int chip_blocks(const ChipParams& p) { return (int)((
 // A CTA that has no chunk left sums its share of the evaluation's blocks, as far as
 // they are complete; `first`: number of this evaluation's block 0 in the launch.
 template <int MODE>
-__device__ __forceinline__ void chip_sum_own(const ChipParams& p, unsigned char* sm, int first) {
+__device__ __forceinline__ void chip_sum_own(const ChipParams& p, unsigned char* sm, int first, const unsigned long long* exits,
+                                             unsigned long long tag) {
     __shared__ int s_full;
     const int nblk = chip_blocks(p), grid = gridDim.x;
     for (int b = (int)((blockIdx.x + grid - first % grid) % grid); b < nblk; b += grid) {
-        if (threadIdx.x == 0)
-            s_full = ld_acquire_gpu(p.arrive + 1 + b) ==
-                     tagged(p.tag, (unsigned)min((int64_t)kReduceBlock, p.S - (int64_t)b * kReduceBlock));
+        if (threadIdx.x == 0) {   // (two loads in flight together)
+            const unsigned long long e = tag ? ld_relaxed_gpu(exits) : 0;
+            const unsigned n = ld_acquire_gpu_u32(p.arrive + b);
+            s_full = e >> kTagShift == tag && !(e & kExitsUntrusted) &&
+                     n == (unsigned)min((int64_t)kReduceBlock, p.S - (int64_t)b * kReduceBlock);
+        }
         __syncthreads();
         const bool full = s_full != 0;
         __syncthreads();
         if (!full) continue;
-        chip_sums<MODE>(p, sm, b, b + 1, true);
-        if (threadIdx.x == 0) p.arrive[1 + b] = tagged(p.tag, kBlockSummed);   // (read by the last CTA, after this one's release)
+        chip_sums<MODE>(p, sm, b, b + 1, nullptr);
+        if (threadIdx.x == 0) p.arrive[b] = kBlockSummed;   // (read by the last CTA, after this one's release)
     }
 }
 
+// The last CTA of the launch: the blocks nobody has summed (`all`: every block), then the
+// means.
+template <int MODE>
+__device__ __forceinline__ void chip_sum_rest(const ChipParams& p, unsigned char* sm, bool all) {
+    chip_sums<MODE>(p, sm, 0, chip_blocks(p), all ? nullptr : p.arrive);
+}
 template <int MODE>
 __device__ __noinline__ void chip_mean(const ChipParams& p, int lane) {
     const int64_t nblk = (p.S + kReduceBlock - 1) / kReduceBlock;
@@ -779,7 +785,7 @@ __device__ __forceinline__ void chip_sink(const ChipParams& p, unsigned char* sm
 // State of a CTA between chunks.
 struct ChipState {
     int pending;        // chunk whose sink has not been summed (-1: none); its tail level is in place
-    int written;        // chunk whose results are written but not counted in (warp 0)
+    int written;        // chunk whose results are written but not counted in
     unsigned word;      // this lane's sink word
     bool counts;        // results are counted in block by block
 };
@@ -800,8 +806,8 @@ __device__ __forceinline__ void chip_chunk(const ChipParams& p, int chunk, unsig
     // the previous chunk's sink beside the exponentials
     if (warp == 0 && cs.pending >= 0) {
         chip_sink<MODE>(p, sm, p.tail_off, cs.pending, cs.word);
-        cs.written = cs.pending;
     }
+    if (cs.pending >= 0) cs.written = cs.pending;
     int cur = p.L == 2 ? p.tail_off : 0;   // where the current level is
     if (tid * 4 < RB) reinterpret_cast<unsigned*>(sm + cur)[tid] = 0u;                        // the zero row
     if (tid * (int)sizeof(Val) < RB) reinterpret_cast<Val*>(sm + cur + RB)[tid] = (Val)1;     // the root holds 1
@@ -853,7 +859,11 @@ __device__ __forceinline__ void chip_chunk(const ChipParams& p, int chunk, unsig
         load_words(m, words + (d >> 11 << 6), d & 0x7ffu, r32);
     };
     if (p.L > 2) open(1);
-    if (cs.counts && tid == 0 && cs.written >= 0) chip_arrive(p, cs.written);
+    // In count mode, where no propagators lie between, the release waits for the sink's writes,
+    // and not in warp 0, which has had the sink to sum: by it medium count took 1.8 % longer.
+    // Elsewhere the last warp, which has formed the most exponentials, would be the wrong one
+    // (14 levels of 8 rows, FP32, 1.5 % longer).
+    if (cs.counts && tid == (Tr::kCount ? T - 32 : 0) && cs.written >= 0) chip_arrive(p, cs.written);
     cs.written = -1;
     for (int l = 1; l + 1 < p.L; ++l) {
         const int W = lv.x, groups = lv.y, dst = lv.w & 0x7fffffff;
@@ -921,8 +931,8 @@ __device__ __forceinline__ void chip_chunk(const ChipParams& p, int chunk, unsig
     } else {
         if (warp == 0) {
             chip_sink<MODE>(p, sm, cur, chunk, cs.word);
-            cs.written = chunk;
         }
+        cs.written = chunk;
         __syncthreads();
     }
 }
@@ -942,6 +952,27 @@ __device__ __forceinline__ void chip_finish(const ChipParams& p, unsigned char* 
     __syncthreads();
 }
 
+// The exit word does not belong to this launch when one of its CTAs leaves: those that claim it
+// have not started yet.  Takes it over, or counts on what another CTA made of it.  (Out of
+// line: the last CTA fetches the code behind it cold.)
+__device__ __noinline__ unsigned long long chip_exit_early(unsigned long long* exits, unsigned long long tag) {
+    unsigned long long before = 0;
+    __threadfence();
+    for (int q = 0; q < (1 << 20); ++q) {   // (a try fails when another CTA's succeeds)
+        const unsigned long long now = ld_relaxed_gpu(exits);
+        if (now >> kTagShift == tag) {
+            before = atomicAdd(exits, 1ull);
+            break;
+        }
+        if (atomicCAS(exits, now, tagged(tag, kExitsUntrusted | 1u)) == now) {
+            before = tagged(tag, kExitsUntrusted);
+            break;
+        }
+    }
+    __threadfence();
+    return before;
+}
+
 template <int MODE, int LB>
 __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ ChipArgs a) {
     extern __shared__ __align__(128) unsigned char sm[];
@@ -950,14 +981,11 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
     __shared__ int s_last;
     __shared__ ChipParams s_p;
     const int warp = threadIdx.x >> 5;
-    // the exit word, taken over for this launch further below by one compare-and-swap of every
-    // CTA: one that fails has lost to a CTA of this launch, nobody else writes the word
-    const bool claims = threadIdx.x == 32;
+    // the first CTAs take the exit word over for this launch, by a compare-and-swap that nobody
+    // waits for (by every CTA it cost 1.2 us, hundreds at one address)
+    const bool claims = a.tag && blockIdx.x < 4 && threadIdx.x == 32;
     unsigned long long found = 0;
-    if (claims) asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(found) : "l"(a.exits) : "memory");
-    auto claim = [&] {
-        if (claims && found >> kTagShift != a.tag) atomicCAS(a.exits, found, tagged(a.tag, 0u));
-    };
+    if (claims) found = ld_relaxed_gpu(a.exits);
     if (warp == 0) tmem_alloc(&s_tmem, (unsigned)a.tmem_cols);
     if (a.list && threadIdx.x == 0) s_next[0] = (int)atomicAdd(a.ticket, 1u);
     __syncthreads();
@@ -971,19 +999,21 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
         chip_setup<MODE>(a.one, sm);
         cs.word = lane < a.one.g.nsink ? __ldg(a.one.g.sink + lane) : 0u;
         chip_times<MODE>(a.one, sm, blockIdx.x);   // (the grid has no CTA without a chunk)
-        claim();
         cp_async_wait<0>();
         __syncthreads();
+        if (claims && found >> kTagShift != a.tag) {
+            const bool clean = found == 0 || ((unsigned)found & ((1u << kTagShift) - 1u)) == kExitsDone;
+            atomicCAS(a.exits, found, tagged(a.tag, clean ? 0u : kExitsUntrusted));
+        }
         for (int c = blockIdx.x; c < a.one.nchunks; c += gridDim.x)
             chip_chunk<MODE, LB>(a.one, c, sm, tmem, cs, [&] {
                 const int n = c + (int)gridDim.x;
                 return n < a.one.nchunks ? n : -1;
             });
         chip_finish<MODE>(a.one, sm, cs);
-        if (!a.few) chip_sum_own<MODE>(a.one, sm, 0);
+        if (!a.few) chip_sum_own<MODE>(a.one, sm, 0, a.exits, a.tag);
     } else {
         int g = -1;
-        claim();
         for (int buf = 0;; buf ^= 1) {
             const int c = s_next[buf];
             if (c >= a.total) break;
@@ -1011,7 +1041,7 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
         if (g >= 0) chip_finish<MODE>(s_p, sm, cs);
         int first = 0;
         for (int h = 0; h < a.n && !a.few; ++h) {
-            chip_sum_own<MODE>(a.list[h], sm, first);
+            chip_sum_own<MODE>(a.list[h], sm, first, a.exits, kClearedTag);
             first += (int)((a.list[h].S + kReduceBlock - 1) / kReduceBlock);
         }
     }
@@ -1020,17 +1050,25 @@ __global__ void __launch_bounds__(512, 1) chip_kernel(const __grid_constant__ Ch
         // (one atomic with both orders: between two fences it took 1,000 cycles longer)
         unsigned long long before;
         asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], 1;" : "=l"(before) : "l"(a.exits) : "memory");
-        s_last = before + 1u == tagged(a.tag, gridDim.x);
+        if (before >> kTagShift != a.tag) before = chip_exit_early(a.exits, a.tag);
+        const unsigned n = (unsigned)(before - tagged(a.tag, 0u)) + 1u;   // CTAs that have left, or more than all
+        s_last = n == gridDim.x ? 1 : n == (gridDim.x | kExitsUntrusted) ? 2 : 0;
     }
     __syncthreads();
     if (s_last) {   // every other CTA has counted its chunks in and left
         const int n = a.list ? a.n : 1;
         for (int h = 0; h < n; ++h) {
             const ChipParams& p = a.list ? a.list[h] : a.one;
-            chip_sums<MODE>(p, sm, 0, chip_blocks(p), a.few != 0);   // the blocks nobody has summed
+            chip_sum_rest<MODE>(p, sm, a.few || s_last == 2);
         }
         __syncthreads();
         for (int h = warp; h < n; h += blockDim.x >> 5) chip_mean<MODE>(a.list ? a.list[h] : a.one, threadIdx.x & 31);
+        if (!a.list && warp > 0) {   // beside the mean (a batch's words are cleared before each launch)
+            const int words = s_last == 2 ? a.one.arrive_cap : a.few ? 0 : chip_blocks(a.one);
+            for (int b = threadIdx.x - 32; b < words; b += blockDim.x - 32) a.one.arrive[b] = 0;
+            if (threadIdx.x == 32)
+                atomicCAS(a.exits, tagged(a.tag, (s_last == 2 ? kExitsUntrusted : 0u) | gridDim.x), tagged(a.tag, kExitsDone));
+        }
     }
     __syncthreads();
     if (warp == 0 && a.tmem_cols) tmem_dealloc(base, (unsigned)a.tmem_cols);
@@ -1227,22 +1265,24 @@ int launch(int kmode, int lane_bytes, int threads, int smem, bool staged, ChipAr
 }  // namespace
 
 unsigned long long next_chip_tag() {
-    static std::atomic<unsigned long long> tag{kBatchTag};
+    static std::atomic<unsigned long long> tag{kClearedTag};
     return ++tag;
 }
 
-int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, cudaStream_t st) {
+int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, bool waits, cudaStream_t st) {
     ChipArgs a{};
     a.one = p;
     const int64_t blocks = (p.S + kReduceBlock - 1) / kReduceBlock;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();   // (the launch reports it)
+    if (!waits && cudaStreamIsCapturing(st, &cap) != cudaSuccess) cudaGetLastError();   // (the launch reports it)
     if (cap != cudaStreamCaptureStatusNone) {   // replays carry one tag
-        const cudaError_t e = cudaMemsetAsync(p.arrive, 0, sizeof(*p.arrive) * (size_t)(blocks + 1), st);
+        a.one.tag = kClearedTag;
+        cudaError_t e = cudaMemsetAsync(p.arrive, 0, sizeof(*p.arrive) * (size_t)p.arrive_cap, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(p.exits, 0, sizeof(*p.exits), st);
         if (e != cudaSuccess) return set_error(COS_ERR_CUDA, "clear arrival counters: %s", cudaGetErrorString(e));
     }
-    a.exits = p.arrive;
-    a.tag = p.tag;
+    a.exits = p.exits;
+    a.tag = a.one.tag;
     a.few = blocks <= few_blocks(plan.threads);
     // with room for any two levels none goes through TMEM, whose allocation takes 700 cycles
     const bool staged = p.lev_bytes < 2 * round128(((int64_t)p.g.max_width + 1) << p.rb_log2);
@@ -1253,7 +1293,7 @@ int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const Chi
                      unsigned* ticket, unsigned long long* exits, int sms, cudaStream_t st) {
     ChipArgs a{};
     a.exits = exits;
-    a.tag = kBatchTag;
+    a.tag = kClearedTag;
     a.list = list;
     a.n = n;
     a.total = total;

@@ -22,14 +22,19 @@ struct ChipGraph {
     int64_t edges = 0, rows = 0;
 };
 
-// Arrivals are counted under the launch's tag (the upper 44 bits of a word, the count in the
-// lower 20), a number that no other launch of the process has: whatever an earlier launch
-// left in a word -- calls that share the words and overlapped, which spoils their own
-// results, among them -- a later launch counts from zero.  Clearing the words on the stream
-// before each launch instead would cost a node of some 2 us in front of a tiny graph's 14;
-// only a captured launch, whose replays carry one tag, is preceded by one.
+// A launch leaves the block words at zero.  Launches that share them and overlap (which
+// spoils their own results) do not, so that the exit word also tells whether they can be
+// trusted: its upper 44 bits are the number of the launch that counts its CTAs there, a
+// number that no other launch of the process has, and the last CTA of a launch that
+// nothing came between marks it kExitsDone.  A launch that finds neither this nor zero
+// counts under kExitsUntrusted: its last CTA sums every block itself and clears all block words.
+// A CTA of an overlapping launch that wrote a block word after that leaves later still, and
+// its count spoils the mark again.  Clearing the words on the stream before each launch instead
+// would cost a node of some 2 us in front of a tiny graph's 14; that is what a captured
+// launch has, whose replays carry one number, and a batch's.
 constexpr int kTagShift = 20;
-constexpr unsigned long long kBatchTag = 1;   // of a batch's launches, whose words are cleared with its counters
+constexpr unsigned long long kClearedTag = 0;   // of launches whose words are cleared before
+constexpr unsigned kExitsDone = 1u << 19, kExitsUntrusted = 1u << 18;
 unsigned long long next_chip_tag();
 
 constexpr int kChipMaxTimes = 48;   // D: the sign masks of all (i, j) pairs are kept in shared memory
@@ -48,14 +53,14 @@ struct ChipParams {
     double* partials_abs;
     Ctrl* ctrl;
     double* mean_out;          // optional second destination of the mean(s)
-    // [1 + blocks of kReduceBlock samples] words of launch tag and count: word 0 the CTAs that
-    // have left, word 1 + b the samples of block b that are written (see kTagShift)
-    unsigned long long* arrive;
+    unsigned* arrive;          // [blocks of kReduceBlock samples]: samples that are written
+    unsigned long long* exits; // CTAs of the launch that have left (see kTagShift)
     unsigned long long tag;    // this launch's number
     double beta, ptab_inv_h;
     int64_t S, t_ld;
     int32_t L, P, K, D, ptab_T, abs_weights;
     int32_t clear_err;         // 1: a completed evaluation clears ctrl->err
+    int32_t arrive_cap;        // words at `arrive`
     int32_t nchunks, first_chunk;
     int32_t rb_log2, s_log2;   // bytes of a node's row; samples per chunk
     uint32_t d_magic;          // ceil(2^32 / D): r / D = mulhi(r, d_magic) for r < 65536 (D > 1)
@@ -79,11 +84,12 @@ bool chip_plan(const ChipGraph& g, int kmode, int32_t L, int32_t P, int32_t K, i
                int members, ChipPlan* out);
 // Fill the shape-dependent fields of p (rb_log2 .. coef_off, nchunks).
 void chip_shape(int kmode, const ChipPlan& plan, ChipParams* p);
-// One evaluation, parameters by value.
-int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, cudaStream_t st);
+// One evaluation, parameters by value; waits: the caller waits for it (which no capture
+// survives).
+int launch_chip(int kmode, const ChipPlan& plan, const ChipParams& p, int sms, bool waits, cudaStream_t st);
 // Evaluations of n graphs that share (lane_bytes, threads): parameters in device
 // memory, chunks [0, total) drawn from *ticket, leaving CTAs counted in *exits (both zero
-// at launch, the words of every member's arrivals too; tag kBatchTag).
+// at launch, the block words of every member too).
 int launch_chip_list(int kmode, int lane_bytes, int threads, int smem, const ChipParams* list, int n, int total,
                      unsigned* ticket, unsigned long long* exits, int sms, cudaStream_t st);
 // Parameters and launch shape of an evaluation of g in kernel mode `kmode` (cos_graph.cu);

@@ -139,7 +139,9 @@ struct cos_graph {
     size_t arena_bytes = 0;
     double* d_partials = nullptr;
     int64_t partial_cap = 0;
-    unsigned long long* d_arrive = nullptr;   // on-chip walk: arrival words [1 + partial_cap] behind the partials (ChipParams::arrive)
+    // on-chip walk, behind the partials: exit word, then arrival words [partial_cap] (ChipParams)
+    unsigned long long* d_exits = nullptr;
+    unsigned* d_arrive = nullptr;
     ChipGraph chip;                 // on-chip walk: row schedule (max_width 0: none)
     void* d_R = nullptr;            // internal per-sample output when the caller passes none
     int64_t R_cap = 0;
@@ -877,11 +879,14 @@ static int attach_samples(cos_graph_t g, int64_t num_samples, const double* t, i
         // two arrays: partial sums of R, then of A (when the walk also sums |path| values),
         // and the arrival counters of the on-chip walk
         g->partial_cap = 0;
+        g->d_exits = nullptr;
         g->d_arrive = nullptr;
         dfree(g->d_partials);
-        COS_CUDA(cudaMalloc(&g->d_partials, 2 * sizeof(double) * cap + sizeof(*g->d_arrive) * (cap + 1)), "cudaMalloc partials");
-        g->d_arrive = reinterpret_cast<unsigned long long*>(g->d_partials + 2 * cap);
-        COS_CUDA(cudaMemsetAsync(g->d_arrive, 0, sizeof(*g->d_arrive) * (cap + 1), st), "clear arrival counters");
+        const size_t words = sizeof(*g->d_exits) + sizeof(*g->d_arrive) * (size_t)cap;
+        COS_CUDA(cudaMalloc(&g->d_partials, 2 * sizeof(double) * cap + words), "cudaMalloc partials");
+        g->d_exits = reinterpret_cast<unsigned long long*>(g->d_partials + 2 * cap);
+        g->d_arrive = reinterpret_cast<unsigned*>(g->d_exits + 1);
+        COS_CUDA(cudaMemsetAsync(g->d_exits, 0, words, st), "clear arrival counters");
         g->partial_cap = cap;
     }
     // Workspace arena: enough for the FP64 mode over all samples, up to the budget.
@@ -1071,7 +1076,7 @@ int cos_evaluate(cos_graph_t g, int32_t mode, void* per_sample_out, double* mean
         if (rc == COS_OK && on_chip) {
             cp.tag = next_chip_tag();
             if (mean_out) cp.mean_out = g->h_means;
-            rc = launch_chip(km, plan, cp, sms, st);
+            rc = launch_chip(km, plan, cp, sms, mean_out != nullptr, st);
         }
         if (rc != COS_OK) return rc;
         if (on_chip) {
@@ -1273,6 +1278,8 @@ int prepare_chip(cos_graph_t g, int kmode, void* per_sample_out, int members, Ch
     p.partials_abs = abs2 ? g->d_partials + g->partial_cap : nullptr;
     p.ctrl = g->d_ctrl;
     p.arrive = g->d_arrive;
+    p.arrive_cap = (int32_t)std::min<int64_t>(g->partial_cap, INT32_MAX);
+    p.exits = g->d_exits;
     p.beta = g->beta;
     p.ptab_inv_h = g->d_ptab ? (double)g->ptab_T / g->ptab_tau_max : 0.0;
     p.S = g->S;

@@ -37,14 +37,18 @@ static __device__ __align__(256) unsigned char g_static_scratch[COS_STATIC_SCRAT
 // Arrival words of the on-chip walk (its other working memory is on chip; the partial sums
 // and the control block are in the scratch array).
 constexpr int kStaticBlocks = 4096;
-static __device__ unsigned long long g_static_arrive[kStaticBlocks + 1];
+struct StaticWords {
+    unsigned long long exits;
+    unsigned arrive[kStaticBlocks];
+};
+static __device__ StaticWords g_static_words;
 
 constexpr int kMaxDevices = 64;
 std::mutex g_addr_mutex;
 struct ScratchAddr {
     void* ctx;    // the context the address belongs to
     void* ptr;    // device address of g_static_scratch in that context
-    void* arrive; // ... and of g_static_arrive
+    void* words;  // ... and of g_static_words
 };
 ScratchAddr g_scratch_addr[kMaxDevices] = {};
 
@@ -71,7 +75,7 @@ void* current_context() {
 // is kept together with the context it was taken in and looked up again when the
 // device's context differs (after cudaDeviceReset, a new primary context may load
 // the module elsewhere).
-int scratch_address(int device, void** out, void** arrive) {
+int scratch_address(int device, void** out, void** words) {
     if (device < 0 || device >= kMaxDevices) return set_error(COS_ERR_INVALID, "device ordinal %d not supported", device);
     void* ctx = current_context();
     std::lock_guard<std::mutex> lock(g_addr_mutex);
@@ -79,7 +83,7 @@ int scratch_address(int device, void** out, void** arrive) {
     if (!a.ptr || !ctx || a.ctx != ctx) {
         void* ptr = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&ptr, g_static_scratch);
-        if (e == cudaSuccess) e = cudaGetSymbolAddress(&a.arrive, g_static_arrive);
+        if (e == cudaSuccess) e = cudaGetSymbolAddress(&a.words, g_static_words);
         if (e != cudaSuccess || !ptr) {
             a.ptr = nullptr;
             return set_error(COS_ERR_CUDA, "cudaGetSymbolAddress(static scratch) failed: %s", cudaGetErrorString(e));
@@ -88,7 +92,7 @@ int scratch_address(int device, void** out, void** arrive) {
         a.ctx = ctx;
     }
     *out = a.ptr;
-    *arrive = a.arrive;
+    *words = a.words;
     return COS_OK;
 }
 
@@ -143,8 +147,8 @@ extern "C" int cos_evaluate_static(cos_graph_t g, int32_t mode, int64_t num_samp
     int cur = -1;
     if (cudaGetDevice(&cur) != cudaSuccess || cur != gv.device)
         return set_error(COS_ERR_INVALID, "the graph's device (%d) must be current", gv.device);
-    void *base = nullptr, *arrive = nullptr;
-    rc = scratch_address(gv.device, &base, &arrive);
+    void *base = nullptr, *words = nullptr;
+    rc = scratch_address(gv.device, &base, &words);
     if (rc != COS_OK) return rc;
 
     // Carve the static array: control block, partial sums, coefficients, then one tile's working set.
@@ -235,7 +239,9 @@ extern "C" int cos_evaluate_static(cos_graph_t g, int32_t mode, int64_t num_samp
         q.R = per_sample_out;
         q.partials = reinterpret_cast<double*>(b + part_at);
         q.ctrl = p.ctrl;
-        q.arrive = static_cast<unsigned long long*>(arrive);
+        q.arrive = static_cast<StaticWords*>(words)->arrive;   // (device addresses)
+        q.arrive_cap = kStaticBlocks;
+        q.exits = &static_cast<StaticWords*>(words)->exits;
         q.tag = next_chip_tag();
         q.beta = beta;
         q.ptab_inv_h = p.ptab_inv_h;
@@ -247,7 +253,7 @@ extern "C" int cos_evaluate_static(cos_graph_t g, int32_t mode, int64_t num_samp
         q.D = gv.D;
         q.ptab_T = gv.ptab_T;
         chip_shape(mode, plan, &q);
-        rc = launch_chip(mode, plan, q, sms, st);
+        rc = launch_chip(mode, plan, q, sms, mean_out != nullptr, st);
         if (rc != COS_OK) return rc;
         return mean_out ? static_result(gv, mode, p.ctrl, mean_out, st) : COS_OK;
     }
