@@ -19,20 +19,20 @@
 // results are bitwise theirs.
 //
 // What bounds it (ncu, medium graph, FP32, 16,384 samples): the shared-memory pipe, two
-// 16-byte reads per edge and lane, 68 % of all cycles busy, a third of that bank conflicts
-// that the row order of cos_chip.h leaves; issue slots 38 %, DRAM 0.  A chunk of 8 samples
+// 16-byte reads per edge and lane, 68 % of all cycles busy, a quarter of the load wavefronts
+// bank conflicts that the row order of cos_chip.h leaves; issue slots 41 %, DRAM 0.  A chunk of 8 samples
 // takes 64,600 cycles, 43,000 of them in its four levels of 4,096 rows, 9,000 in the
 // propagators; a small level costs some 900 cycles whatever it holds.  Medium graph, 65,536
-// samples, before (general kernels) and after: FP32 2.35 -> 1.61 ms, with A 3.00 -> 2.20,
-// count 3.2 -> 1.87.  The FP64 walk is bound by the FP64 pipe on both paths (6.3 / 6.9 ms).
+// samples, before (general kernels) and after: FP32 2.35 -> 1.62 ms, with A 3.89 -> 2.86,
+// count 3.2 -> 1.85.  The FP64 walk is bound by the FP64 pipe on both paths (6.3 / 6.9 ms).
 //
 // CTAs never wait for one another: a CTA that has no chunk left sums its share of the
 // blocks of kReduceBlock samples that are complete, the last CTA the others, and it forms
 // the mean.  A block is summed by the whole CTA in 128-bit integers (cos_fixed.h): 2,800
 // cycles from the first load to the partial sum, most of them latency, against 15,800 for
 // one warp's compensated additions, which the end of every launch waits for.  Tiny graph,
-// 1,000 samples, mixed, one launch: 20.5 -> 14.4 us; order 2, 1,000 nodes, 10,007 samples:
-// 96 -> 84 us.
+// 1,000 samples, mixed, one launch: 20.5 -> 14.3 us; order 2, 1,000 nodes, 10,007 samples:
+// 96 -> 84 us (66 with the exponentials below and two CTAs per SM).
 #include <algorithm>
 #include <atomic>
 #include <cstdio>
@@ -220,7 +220,8 @@ __device__ __forceinline__ void chip_times(const ChipParams& p, unsigned char* s
 // them FP64; 38 % of the issue slots used) and fetching them: the loops have one copy of
 // their code, and a graph whose kinds need no double arithmetic never enters its loop.  Order
 // 2, 32 kinds, 32 samples a chunk: exponentials 18,000 -> 14,000 cycles, slots 15,700 ->
-// 10,900, of 50,000 -> 45,000 (84 -> 72 us for 10,007 samples).
+// 10,900, of 50,000 -> 45,000 (84 -> 72 us for 10,007 samples in this shape; 66 in two CTAs
+// per SM).
 //
 // Exponentials of the kinds [k0, k0 + kn), times and samples of the chunk, with the
 // arithmetic of item_props of the general kernels.  Returns whether a time lies so far
@@ -1191,8 +1192,8 @@ double general_time_us(const ChipGraph& g, int kmode, int32_t L, int32_t P, int6
 }
 
 // The shape with the least model time; on chip when that is below the general kernels'.
-// Measured on both sides of the line, general / on-chip: medium graph 2.35 / 1.61 ms
-// (FP32), 3.00 / 2.20 ms (with A), 3.1 / 1.86 ms (count), FP64, 16,384 samples, 1.60 / 1.63 ms
+// Measured on both sides of the line, general / on-chip: medium graph, 65,536 samples, 2.35 /
+// 1.62 ms (FP32), 3.89 / 2.86 ms (with A), 3.1 / 1.85 ms (count), FP64, 16,384 samples, 1.60 / 1.63 ms
 // (both held by the FP64 pipe; general), 10,000 nodes of order 4, FP64, 2,000 samples 226 /
 // 169 us; FP32 with two samples per chunk: 100,000 nodes, levels of 12,200, 4,000 samples 868 /
 // 988 us (general), 500 samples 198 / 131; levels of 19,500 5.44 / 5.80 ms (general), but
@@ -1242,7 +1243,8 @@ void chip_shape(int kmode, const ChipPlan& plan, ChipParams* p) {
 
 namespace {
 
-// Blocks of samples up to which the last CTA sums them all, two rounds of its teams.
+// Blocks of samples up to which the last CTA sums them all, one after another: 2 for a CTA of
+// 128 threads, 8 for one of 512.
 int few_blocks(int threads) { return 2 * (threads / 128); }
 
 int launch(int kmode, int lane_bytes, int threads, int smem, bool staged, ChipArgs& a, int chunks, int sms, cudaStream_t st) {

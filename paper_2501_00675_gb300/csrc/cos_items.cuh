@@ -406,7 +406,8 @@ __device__ __forceinline__ FmaConst fma_const(int x) {
 // Leading 24 significant bits of a double as a float, by truncation with 32-bit
 // integer operations on the double's two halves only (no FP64 conversion; 64-bit
 // integer operations occupy GB300's FP64 pipe); |x| below 2^-126 gives a signed zero.
-// The callers keep |x| below 2^127.
+// |x| of 2^128 or more gives no meaningful value; the callers' results are defined for far
+// smaller arguments only (|x| <= 708).
 __device__ __forceinline__ float trunc_to_float(double x) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     const unsigned e = (hi >> 20) & 0x7ffu;
