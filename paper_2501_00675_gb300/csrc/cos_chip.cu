@@ -618,39 +618,46 @@ __device__ __forceinline__ void cta_sum(double (&v)[kPerThread], const T* x, dou
 }
 constexpr unsigned kBlockSummed = 0xffffffffu;   // arrival word of a block whose partial sum is written
 
+// The first block from q on whose arrival word is not kBlockSummed; 32 words at a time, read by
+// one warp for all -- the callers' loop has block barriers, and a launch that overlaps on the
+// same words changes them.  (Out of line: short launches sum every block, and fetch the code
+// behind it cold.)
+__device__ __noinline__ int next_open(const unsigned* arrive, int q, int nblk, bool first) {
+    __shared__ unsigned s_open;
+    __shared__ int s_base;
+    int base = first ? -1 : s_base;
+    unsigned open = first ? 0u : s_open;
+    while (q < nblk) {
+        if ((q & ~31) != base) {
+            base = q & ~31;
+            const int at = base + (int)(threadIdx.x & 31);
+            __syncthreads();   // everyone has the words before
+            if (threadIdx.x < 32) {
+                const unsigned left = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != kBlockSummed);
+                if (threadIdx.x == 0) {
+                    s_open = left;
+                    s_base = base;
+                }
+            }
+            __syncthreads();
+            open = s_open;
+        }
+        const unsigned left = open >> (q - base);
+        if (left) return q + __ffs((int)left) - 1;
+        q = base + 32;
+    }
+    return nblk;
+}
+
 // Partial sums of blocks [b, nblk) whose arrival word is not kBlockSummed (arrive
 // nullptr: of all).
 template <typename T>
 __device__ __forceinline__ void cta_sums(const T* x, double* partials, int64_t S, int b, int nblk, const unsigned* arrive, CtaSum& c) {
-    // the next block to sum: 32 arrival words at a time, read by one warp for all -- the loop
-    // below has block barriers, and a launch that overlaps on the same words changes them
-    __shared__ unsigned s_open;
-    int base = -1;
-    unsigned open = 0;
-    auto skip = [&](int q) {
-        while (arrive && q < nblk) {
-            if ((q & ~31) != base) {
-                base = q & ~31;
-                const int at = base + (int)(threadIdx.x & 31);
-                __syncthreads();   // everyone has the word before
-                if (threadIdx.x < 32) {
-                    const unsigned left = __ballot_sync(0xffffffffu, at < nblk && __ldcg(arrive + at) != kBlockSummed);
-                    if (threadIdx.x == 0) s_open = left;
-                }
-                __syncthreads();
-                open = s_open;
-            }
-            const unsigned left = open >> (q - base);
-            if (left) return q + __ffs((int)left) - 1;
-            q = base + 32;
-        }
-        return min(q, nblk);
-    };
+    if (arrive) b = next_open(arrive, b, nblk, true);
     double v[kPerThread], next[kPerThread];
-    b = skip(b);
     if (b < nblk) cta_load(v, x, S, b);
     while (b < nblk) {
-        const int n = skip(b + 1);
+        const int n = arrive ? next_open(arrive, b + 1, nblk, false) : b + 1;
         if (n < nblk) cta_load(next, x, S, n);   // a block ahead
         cta_sum(v, x, partials, S, b, c);
 #pragma unroll
